@@ -3,7 +3,7 @@
 //
 // One group of T threads owns one leaf for its whole pursuit.  The leaf's M
 // correlations c_j = <r, phi_j> live in registers as double-float pairs, E of
-// them per thread (element j = lane + T s).  Each step:
+// them per thread (struct Atoms says which).  Each step:
 //   (a3) argmax |c_j|, lowest j among equals;
 //   (a4) alpha = c_j*; c <- c - alpha G[:, j*].  The dictionary is the union
 //        of two orthonormal separable bases (DCT-II and Haar), so its Gram
@@ -21,13 +21,13 @@
 // next level's queue.  Leaves are handed out through a device
 // counter, so a group that finishes a short pursuit takes the next leaf.
 //
-// Argmax cost.  Each thread keeps, per atom family, the top two |hi| keys of
-// its elements (with the top's index, sign and low word).  A step changes one
-// family (and zeroes one element of the other), so only that family's top-2
-// is recomputed.  The group reduction carries (top key, index | sign, second
-// key, low word): alpha arrives with the reduction, and whether any other
-// atom lies within the decision window of the best is read off the second
-// key, with no extra pass over the elements.
+// Argmax cost.  Each thread keeps the largest magnitude of its elements
+// (struct Summary).  A step changes one family (and zeroes one element of the
+// other), so only that family's summaries are formed anew.  The group reduces
+// the magnitudes alone; the warp that holds the largest then looks its words
+// up and hands (hi, lo, atom, largest other magnitude) to the others.  Where
+// the last word reaches the decision window of the leader, the step is decided
+// from the full words of every element.
 //
 // Equality in finite precision: correlations within 2^-32 ||y|| of the
 // largest count as tied and the lowest index among them wins; an energy
@@ -138,34 +138,33 @@ __global__ void __launch_bounds__(T > 32 ? T : 256, MINB)
 mp_kernel(MPArgs a) {
     constexpr int n = B * B;
     constexpr int M = NF * n;
-    constexpr int E = (M + T - 1) / T;
-    static_assert(T % B == 0, "thread count must be a multiple of the side");
+    constexpr int E = M / T;
     constexpr int NW = T / 32;               // warps per group (T > 32)
-    static_assert(!RESC || (DF && T > 32 && NW >= 8 && E <= 32 && (M % T) == 0), "rescore layout");
-    // SPLIT: the first E/2 elements of every thread are DCT atoms and the
-    // rest Haar atoms, each family cached separately; otherwise one group.
-    constexpr bool SPLIT = NF == 2 && (n % T) == 0 && (E % 2) == 0;
-    constexpr int NG = SPLIT ? 2 : 1;
+    static_assert(!RESC || (DF && T > 32 && NW >= 8 && E <= 32), "rescore layout");
+    // SPLIT: with several warps per leaf, half of them keep the DCT family and
+    // half the Haar family.  A step chosen from one family updates the other,
+    // so the warps of the chosen family are free meanwhile: they keep their
+    // summaries, one of them carries the energy, the stop test and the step
+    // record, and the owner's work on its zeroed element is off the critical
+    // path.  A sub-partition holds as many warps of each family, so the update
+    // itself keeps all FP32 pipes busy either way.  With the packed update and
+    // the magnitude-only summaries: 12 uneven RGB piecewise images 20.7 -> 17.3
+    // ms, 64 gradient ones 17.3 -> 15.9 ms, the 512x512 sweep 1.85 -> 1.72 ms
+    // (whole encodes; same bits).
+    constexpr bool SPLIT = NF == 2 && T > 32;
+    constexpr int FT = SPLIT ? T / 2 : T;    // threads of one family
+    constexpr int NG = NF == 2 && !SPLIT ? 2 : 1;   // families per thread, a summary for each
     constexpr int G = E / NG;
-    constexpr bool FULL = (M % T) == 0;      // every (lane, s) is an atom
-    // STALE: when the chosen atom was the top of its owner's summary, its
-    // removal leaves that summary's second key as the exact new largest
-    // magnitude; the owner keeps it with an unknown index (low word 0)
-    // instead of rescanning its registers every step, and rescans only if
-    // such a summary ever holds the group's largest key.  Equal keys put an
-    // atom within the decision window, which is decided from the registers.
-    // Measured on the 512x512 sweep: 9% faster at b = 32, 20% at b = 16; at
-    // b = 64 the bookkeeping costs more than the rescan it saves (the
-    // owner's rescan overlaps seven other warps' updates), so it is off there.
-    constexpr bool STALE = SPLIT && DF && B < 64;
-
+    using At = Atoms<B, FT, G>;
     extern __shared__ __align__(16) unsigned char smem[];
-    float2 *sW = reinterpret_cast<float2 *>(smem);             // W[p][p'] (hi, lo)
-    float2 *sWT = sW + B * B;                                    // W^T
-    unsigned char *after_tables = smem + (NF == 2 ? 2 * B * B * sizeof(float2) : 0);
-    uint4 *sPart = reinterpret_cast<uint4 *>(after_tables);      // [3][NW] top-2 partials
-    uint32_t *sMisc = reinterpret_cast<uint32_t *>(sPart + 3 * NW);               // [12]
-    unsigned long long *sRk = reinterpret_cast<unsigned long long *>(sMisc + 12); // [NW]
+    // the high and low words of W[p][p'] then W^T, as planes: 2 b^2 floats each
+    float *sWh = reinterpret_cast<float *>(smem);
+    float *sWl = sWh + 2 * B * B;
+    unsigned char *after_tables = smem + (NF == 2 ? 4 * B * B * sizeof(float) : 0);
+    uint4 *sWin = reinterpret_cast<uint4 *>(after_tables);       // [8] leaders: by buffer, or by warp (T == 32)
+    uint2 *sPart = reinterpret_cast<uint2 *>(sWin + 8);          // [3][NW, even] the warps' two largest magnitudes
+    uint32_t *sMisc = reinterpret_cast<uint32_t *>(sPart + 3 * (NW + NW % 2) + NW % 2);   // [16]
+    unsigned long long *sRk = reinterpret_cast<unsigned long long *>(sMisc + 16); // [NW]
     uint32_t *sRj = reinterpret_cast<uint32_t *>(sRk + NW);      // [NW]
     StepRec *sSteps = reinterpret_cast<StepRec *>(sRj + NW);
     // RESC: the leaf's pixels (transposed), its bounds (FP16, rounded up),
@@ -187,9 +186,10 @@ mp_kernel(MPArgs a) {
     if (T == 32 && threadIdx.x < 3) sCnt[threadIdx.x] = 0ull;
     if (threadIdx.x == 0) sMaxT = 0u;
     if (NF == 2) {
-        for (int i = threadIdx.x; i < B * B; i += blockDim.x) {
-            sW[i] = a.W[i];
-            sWT[i] = a.WT[i];
+        for (int i = threadIdx.x; i < 2 * B * B; i += blockDim.x) {
+            const float2 w = i < B * B ? a.W[i] : a.WT[i - B * B];
+            sWh[i] = w.x;
+            sWl[i] = w.y;
         }
     }
     __syncthreads();
@@ -198,6 +198,11 @@ mp_kernel(MPArgs a) {
     const int group = (T == 32) ? (threadIdx.x >> 5) : 0;
     StepRec *steps = sSteps + (size_t)group * lv.k;
     const int p_own = lane % B;
+    const int warp = lane >> 5;
+    const int fam_own = SPLIT ? warp / (NW / 2) : 0;          // uniform in a warp
+    const uint32_t abase = At::base(SPLIT ? lane % FT : lane, fam_own);
+    // the thread that holds atom j
+    auto owner_of = [](uint32_t j) { return At::owner(j) + (SPLIT ? (uint32_t)FT * (j / (uint32_t)n) : 0u); };
     const unsigned count = *lv.count;
     const int k = lv.k;
     unsigned *work = a.work ? a.work : &a.ctr->work_next[lv.level];
@@ -232,28 +237,16 @@ mp_kernel(MPArgs a) {
         // rule may depend on the low words: a few ulps plus the tie band
         const float pre = ldexpf(S_f, -32) * 1.05f + ldexpf(S_f, -37) * 1.05f;
 
-        float ch[E], cl[E];
-        Top2 top[NG];
-        bool stale[NG];             // see STALE below
+        Corr<E> c;
+        Summary<E, G> sm;
         const float2 *cp = a.c0 + (size_t)leaf * M;
 #pragma unroll
-        for (int g = 0; g < NG; ++g) {
-            top[g] = top2_empty();
-            stale[g] = false;
+        for (int s = 0; s < E; s += 2) {
+            const float2 v0 = cp[At::atom(abase, s)], v1 = cp[At::atom(abase, s + 1)];
+            c.h[s / 2] = f2_make(v0.x, v1.x);
+            c.l[s / 2] = DF ? f2_make(v0.y, v1.y) : 0ull;
         }
-#pragma unroll
-        for (int s = 0; s < E; ++s) {
-            const int j = lane + T * s;
-            if (FULL || j < M) {
-                const float2 v = cp[j];
-                ch[s] = v.x;
-                cl[s] = DF ? v.y : 0.0f;
-                top2_fold(top[s / G], v.x, cl[s], (uint32_t)j);
-            } else {
-                ch[s] = 0.0f;
-                cl[s] = 0.0f;
-            }
-        }
+        sm.template form<0, E>(c);
 
         float my_emax = 0.0f;               // RESC: largest bound of this thread's non-exact atoms
         uint32_t exm = 0u;                  // RESC: this thread's exact slots (the bitmask's own bits)
@@ -263,7 +256,7 @@ mp_kernel(MPArgs a) {
         if constexpr (RESC) {
 #pragma unroll
             for (int s2 = 0; s2 < E; ++s2) {
-                const uint32_t j = (uint32_t)(lane + T * s2);
+                const uint32_t j = At::atom(abase, s2);
                 const __half e = __float2half_ru(a.ebound[(size_t)leaf * M + j]);
                 my_emax = fmaxf(my_emax, __half2float(e));       // the value the scans compare with
                 sE[j] = e;
@@ -287,67 +280,121 @@ mp_kernel(MPArgs a) {
 
         int t = 0, windows = 0;
         bool conv = false, tie = false;
-        // With several warps per leaf, warp 0 alone keeps the residual energy
-        // and takes the accuracy test; its verdict travels with the step's
-        // argmax exchange (the test still decides before the step is used).
-        const bool energy_warp = T == 32 || lane < 32;
-        for (;;) {
-            // (a6) accuracy test before every step, strict
-            bool below = false;
-            if (energy_warp) {
-                below = DF ? df_lt(En, thrE) : (En.hi < eps2_f);
-                if (DF && fabsf(En.hi - thrE.hi) <= bandE_f * 1.01f + 0x1p-20f * fabsf(thrE.hi)) {
-                    if (fabs(df_to_double(En) - df_to_double(thrE)) < ldexp((double)e0, -37)) tie = true;
-                }
+        // (a6) accuracy test on the energy, strict; taken before every step
+        auto accuracy = [&](const df &e) {
+            if (DF && __builtin_expect(fabsf(e.hi - thrE.hi) <= bandE_f * 1.01f + 0x1p-20f * fabsf(thrE.hi), 0)) {
+                if (energy_in_band(e, thrE, e0)) tie = true;
             }
+            return DF ? df_lt(e, thrE) : (e.hi < eps2_f);
+        };
+        // (a5) the energy after a step
+        auto spend = [&](const df &e, const df &alpha) {
+            return DF ? df_sub(e, df_mul(alpha, alpha)) : df{__fmaf_rn(-alpha.hi, alpha.hi, e.hi), 0.0f};
+        };
+        // With several warps per leaf the energy lives in shared memory; the
+        // verdict for step t is left in word 8 + (t & 1) and read with the
+        // step's argmax exchange.
+        if (T > 32 && lane == 0) {
+            sMisc[12] = __float_as_uint(En.hi);
+            sMisc[13] = __float_as_uint(En.lo);
+            sMisc[8] = accuracy(En) ? 1u : 0u;
+        }
+        uint32_t wtop = 0u, wsec = 0u;      // T > 32: this warp's two largest magnitudes ...
+        bool dirty = true;                  // ... to be found anew (uniform in a warp)
+        bool stop = false;
+        // (a3) argmax |c| on the cached summaries; T > 32: through buffer `buf`.
+        // Every warp learns the group's largest magnitude and which warp has
+        // it; that warp alone looks the words up.
+        auto group_lead = [&](int buf) {
+            uint32_t M, M2;
+            bool holds;
             if (T == 32) {
-                if (below) { conv = true; break; }
-                if (t == k) break;
-            } else if (t == k) {
-                if (lane == 0) sMisc[10] = below ? 1u : 0u;
+                const uint32_t m = __float_as_uint(sm.top());
+                warp_two(m, 0u, M, M2, holds);
+                write_lead<At, E, G>(sm, c, abase, M, holds, M2, &sWin[threadIdx.x >> 5]);
+                __syncwarp();
+                const Lead r = unpack_lead(sWin[threadIdx.x >> 5]);
+                __syncwarp();
+                return r;
+            }
+            const uint32_t m = __float_as_uint(sm.top());
+            if (dirty) warp_two(m, 0u, wtop, wsec, holds);
+            dirty = false;
+            if ((lane & 31) == 0) sPart[buf * NW + warp] = make_uint2(wtop, wsec);
+            __syncthreads();
+            if (buf < 2) stop = sMisc[8 + buf] != 0u;
+            const uint2 v = (lane & 31) < NW ? sPart[buf * NW + (lane & 31)] : make_uint2(0u, 0u);
+            warp_two(v.x, v.y, M, M2, holds);
+            if (wtop == M)                  // (several warps: then M2 is M, whoever writes last)
+                write_lead<At, E, G>(sm, c, abase, M, m == M, M2, &sWin[buf]);
+            __syncthreads();
+            return unpack_lead(sWin[buf]);
+        };
+        // whether another magnitude reaches the leader's decision window (the
+        // FP32 form: the leader)
+        auto window_of = [&](float amax) { return DF ? amax * 0x1p-20f + pre : 0.0f; };
+        auto contested = [&](const Lead &l) {
+            return __uint_as_float(l.k2) >= fabsf(l.hi) - window_of(fabsf(l.hi));
+        };
+        // the value of atom j, from its owner to the whole group
+        auto words_of = [&](uint32_t j) {
+            const df w = pick_slot<E, E, 0>(c, (NG == 2 ? (uint32_t)G * (j / (uint32_t)n) : 0u) + At::slot(j));
+            if (T == 32)
+                return df{__shfl_sync(0xffffffffu, w.hi, (int)At::owner(j)),
+                          __shfl_sync(0xffffffffu, w.lo, (int)At::owner(j))};
+            if ((uint32_t)lane == owner_of(j)) {
+                sMisc[4] = __float_as_uint(w.hi);
+                sMisc[5] = __float_as_uint(w.lo);
+            }
+            __syncthreads();
+            const df r{__uint_as_float(sMisc[4]), __uint_as_float(sMisc[5])};
+            __syncthreads();
+            return r;
+        };
+        // the lowest of the group's candidates
+        auto lowest_of = [&](uint32_t j) {
+            if (T == 32) return warp_min(j);
+            if (lane == 0) sMisc[6] = kNone;
+            __syncthreads();
+            if (j != kNone) atomicMin(&sMisc[6], j);
+            __syncthreads();
+            return sMisc[6];
+        };
+        // the leader from the full words: the lowest index among equal
+        // magnitudes, and the exact second magnitude
+        auto group_exact = [&]() {
+            const Pair2 m = magnitudes_of<E>(c);
+            uint32_t A, A2;
+            bool holds;
+            warp_two(__float_as_uint(m.m1), __float_as_uint(m.m2), A, A2, holds);
+            if (T > 32) {
+                if ((lane & 31) == 0) sRk[warp] = ((unsigned long long)A << 32) | A2;
                 __syncthreads();
-                conv = sMisc[10] != 0u;
-                break;
+                const unsigned long long v = (lane & 31) < NW ? sRk[lane & 31] : 0ull;
+                warp_two((uint32_t)(v >> 32), (uint32_t)v, A, A2, holds);
+                __syncthreads();
             }
-
-            // (a3) argmax |c| on the cached top-2 summaries
-            bool stop = false;
-            auto group_best = [&](int buf) {
-                Top2 b = top[0];
+            uint32_t j = kNone;
 #pragma unroll
-                for (int g = 1; g < NG; ++g) b = top2_merge(b, top[g]);
-                b = warp_top2(b);
-                if (T > 32) {
-                    if ((lane & 31) == 0)
-                        sPart[buf * NW + (lane >> 5)] =
-                            make_uint4((uint32_t)b.P, (uint32_t)(b.P >> 32), b.k2, __float_as_uint(b.lo1));
-                    if (buf < 2 && lane == 0) sMisc[8 + buf] = below ? 1u : 0u;
-                    __syncthreads();
-                    if (buf < 2) stop = sMisc[8 + buf] != 0u;
-                    const int l = lane & 31;
-                    if (l < NW) {
-                        const uint4 v = sPart[buf * NW + l];
-                        b = Top2{((unsigned long long)v.y << 32) | v.x, v.z, __uint_as_float(v.w)};
-                    } else {
-                        b = top2_empty();
-                    }
-                    b = warp_top2(b);
-                }
-                return b;
-            };
-            Top2 best = group_best(t & 1);
-            if (T > 32 && stop) { conv = true; break; }
-            if (STALE && (best.P >> 32) != 0ull && (uint32_t)best.P == 0u) {
-                // a summary left stale by the last step holds the largest
-                // magnitude: its owners rescan and the group reduces again
-                if (stale[0]) { top[0] = zero_and_rescan<T, E, G, 0>(ch, cl, lane, kNone); stale[0] = false; }
-                if (stale[NG - 1]) {
-                    top[NG - 1] = zero_and_rescan<T, E, G, G>(ch, cl, lane, kNone);
-                    stale[NG - 1] = false;
-                }
-                best = group_best(2);
+            for (int s = E - 1; s >= 0; --s)
+                if ((__float_as_uint(c.hi(s)) & 0x7fffffffu) == A) j = At::atom(abase, s);
+            j = lowest_of(j);
+            const df w = words_of(j);
+            return Lead{w.hi, w.lo, j, A2};
+        };
+        for (;;) {
+            if (T == 32) {
+                if (accuracy(En)) { conv = true; break; }
+                if (t == k) break;
             }
-            if ((best.P >> 32) == 0ull) break;   // every correlation is exactly zero
+            Lead best = group_lead(t & 1);
+            if (T > 32) {
+                if (stop) { conv = true; break; }
+                if (t == k) break;
+            }
+            bool exact = contested(best);       // the leader comes from the full words
+            if (__builtin_expect(exact, 0)) best = group_exact();
+            if (best.hi == 0.0f) break;         // every correlation is exactly zero
             if constexpr (RESC) {
                 // certify the leader against the bounds: every atom whose
                 // upper bound |c| + e reaches the leader's lower bound less the
@@ -357,30 +404,28 @@ mp_kernel(MPArgs a) {
                 // only for the few slots it leaves
                 uint32_t newly = 0u;
                 for (;;) {
-                    const uint32_t jb = top2_index(best);
-                    const float amb = top2_amax(best);
+                    const uint32_t jb = best.j;
+                    const float amb = fabsf(best.hi);
                     const bool exb = (sEx[jb >> 5] >> (jb & 31)) & 1u;
                     const float eb = exb ? 0.0f : __half2float(sE[jb]);
                     const float L = __fsub_rd(__fsub_rd(amb, eb), __fadd_ru(__fmul_ru(amb, 0x1p-20f), pre));
                     // no atom can reach the leader: nothing to exchange
                     if (exb && __fadd_ru(__uint_as_float(best.k2), emax_all) < L) break;
-                    float mine = top2_amax(top[0]);
-#pragma unroll
-                    for (int g = 1; g < NG; ++g) mine = fmaxf(mine, top2_amax(top[g]));
+                    const float mine = sm.top();
                     bool found = false;
                     if (__fadd_ru(mine, my_emax) >= L) {
                         const float thr = __fsub_rd(L, my_emax);
                         uint32_t cm = 0u;
 #pragma unroll
-                        for (int s2 = 0; s2 < E; ++s2) cm |= (fabsf(ch[s2]) >= thr ? 1u : 0u) << s2;
+                        for (int s2 = 0; s2 < E; ++s2) cm |= (fabsf(c.hi(s2)) >= thr ? 1u : 0u) << s2;
                         cm &= ~exm;
                         while (cm) {
                             const int s2 = __ffs(cm) - 1;
                             cm &= cm - 1u;
                             float m = 0.0f;
 #pragma unroll
-                            for (int s3 = 0; s3 < E; ++s3) m = s3 == s2 ? fabsf(ch[s3]) : m;
-                            const uint32_t j = (uint32_t)(lane + T * s2);
+                            for (int s3 = 0; s3 < E; ++s3) m = s3 == s2 ? fabsf(c.hi(s3)) : m;
+                            const uint32_t j = At::atom(abase, s2);
                             if (__fadd_ru(m, __half2float(sE[j])) >= L) {
                                 const uint32_t idx = atomicAdd(&sRW[0], 1u);
                                 if (idx < 8u) sRW[2 + idx] = j;
@@ -399,12 +444,12 @@ mp_kernel(MPArgs a) {
                     if (mine >= lam * amb) {
                         const float thq = lam * amb;
 #pragma unroll
-                        for (int s2 = 0; s2 < E; ++s2) qmask |= (fabsf(ch[s2]) >= thq ? 1u : 0u) << s2;
+                        for (int s2 = 0; s2 < E; ++s2) qmask |= (fabsf(c.hi(s2)) >= thq ? 1u : 0u) << s2;
                         qmask &= ~exm;
                         // drop the ones listed above (their owner is this thread)
                         for (uint32_t w = 0; w < cnt; ++w) {
                             const uint32_t j = sRW[2 + w];
-                            if (j % (uint32_t)T == (uint32_t)lane) qmask &= ~(1u << (j / (uint32_t)T));
+                            if (owner_of(j) == (uint32_t)lane) qmask &= ~(1u << At::slot(j));
                         }
                     }
                     {
@@ -423,7 +468,7 @@ mp_kernel(MPArgs a) {
                         while (qmask && pos < 8u) {
                             const int s2 = __ffs(qmask) - 1;
                             qmask &= qmask - 1u;
-                            sRW[2 + pos] = (uint32_t)(lane + T * s2);
+                            sRW[2 + pos] = At::atom(abase, s2);
                             ++pos;
                         }
                     }
@@ -441,36 +486,35 @@ mp_kernel(MPArgs a) {
                         ++n_rounds;
                     }
                     // into the owners' registers: one predicated pass per atom
-                    uint32_t touched = 0u;               // bit g: family g's summary to redo
+                    bool touched = false;                // the summary to redo
                     bool redo_e = false;                 // the thread's largest bound left with it
                     for (uint32_t w = 0; w < tot; ++w) {
                         const uint32_t j = sRW[2 + w];
-                        if (j % (uint32_t)T != (uint32_t)lane) continue;
-                        const uint32_t sj = j / (uint32_t)T;
+                        if (owner_of(j) != (uint32_t)lane) continue;
+                        const uint32_t sj = At::slot(j);
                         float vh = 0.0f, vl = 0.0f;
 #pragma unroll
                         for (int s2 = 0; s2 < E; ++s2) {
-                            vh = (uint32_t)s2 == sj ? ch[s2] : vh;
-                            vl = (uint32_t)s2 == sj ? cl[s2] : vl;
+                            vh = (uint32_t)s2 == sj ? c.hi(s2) : vh;
+                            vl = (uint32_t)s2 == sj ? c.lo(s2) : vl;
                         }
                         const float2 d = sRv[w];
-                        const df c = df_add(df{vh, vl}, df{d.x, d.y});
+                        const df v = df_add(df{vh, vl}, df{d.x, d.y});
 #pragma unroll
                         for (int s2 = 0; s2 < E; ++s2) {
-                            ch[s2] = (uint32_t)s2 == sj ? c.hi : ch[s2];
-                            cl[s2] = (uint32_t)s2 == sj ? c.lo : cl[s2];
+                            if ((uint32_t)s2 == sj) c.set(s2, v.hi, v.lo);
                         }
                         exm |= 1u << sj;
                         atomicOr(&sEx[j >> 5], 1u << (j & 31));
-                        touched |= 1u << (sj / (uint32_t)G);
+                        touched = true;
                         redo_e |= __half2float(sE[j]) >= my_emax;
                     }
-                    if (touched & 1u) top[0] = zero_and_rescan<T, E, G, 0>(ch, cl, lane, kNone);
-                    if (NG > 1 && (touched & 2u)) top[NG - 1] = zero_and_rescan<T, E, G, G>(ch, cl, lane, kNone);
+                    if (touched) sm.template form<0, E>(c);
+                    dirty = __any_sync(0xffffffffu, touched);
                     if (redo_e) {
                         my_emax = 0.0f;
                         for (int s2 = 0; s2 < E; ++s2)
-                            if (!((exm >> s2) & 1u)) my_emax = fmaxf(my_emax, __half2float(sE[lane + T * s2]));
+                            if (!((exm >> s2) & 1u)) my_emax = fmaxf(my_emax, __half2float(sE[At::atom(abase, s2)]));
                     }
                     {
                         float v = my_emax;
@@ -482,33 +526,31 @@ mp_kernel(MPArgs a) {
                     emax_all = sEm[0];
 #pragma unroll
                     for (int w = 1; w < NW; ++w) emax_all = fmaxf(emax_all, sEm[w]);
-                    best = group_best(2);
+                    best = group_lead(2);
+                    exact = contested(best);
+                    if (exact) best = group_exact();
                 }
-                if (fallback || (best.P >> 32) == 0ull) break;
+                if (fallback || best.hi == 0.0f) break;
             }
-            uint32_t j1 = top2_index(best);
-            const float amax = top2_amax(best);
-            df alpha = df{top2_negative(best) ? -amax : amax, best.lo1};
-            const float window = amax * 0x1p-20f + pre;
-            bool rare = false;
-            if (DF && __uint_as_float(best.k2) >= amax - window) {
-                rare = true;
-                ++windows;
+            uint32_t j1 = best.j;
+            df alpha = df{best.hi, best.lo};
+            if (DF && __builtin_expect(exact && contested(best), 0)) {
                 // Another atom is within the window: decide in full precision
                 // among the candidates -- the true largest magnitude, then the
                 // lowest index within 2^-32 ||y|| of it; any candidate within
                 // 2^-37 ||y|| of that edge is not certified.
+                const float amax = fabsf(best.hi), window = window_of(amax);
+                ++windows;
                 const double tieC = ldexp((double)S_f, -32);
                 const double bandC = ldexp((double)S_f, -37);
                 unsigned long long mk = 0ull;
                 uint32_t mj = kNone;
 #pragma unroll
                 for (int s = 0; s < E; ++s) {
-                    const int j = lane + T * s;
-                    if ((FULL || j < M) && fabsf(ch[s]) >= amax - window) {
-                        const double m = fabs((double)ch[s] + (double)cl[s]);
+                    if (fabsf(c.hi(s)) >= amax - window) {
+                        const double m = fabs((double)c.hi(s) + (double)c.lo(s));
                         const unsigned long long key = (unsigned long long)__double_as_longlong(m);
-                        if (key > mk) { mk = key; mj = (uint32_t)j; }
+                        if (key > mk) { mk = key; mj = At::atom(abase, s); }
                     }
                 }
                 warp_argmax64(mk, mj);
@@ -527,127 +569,67 @@ mp_kernel(MPArgs a) {
                 uint32_t lower = kNone;
 #pragma unroll
                 for (int s = 0; s < E; ++s) {
-                    const int j = lane + T * s;
-                    if ((FULL || j < M) && fabsf(ch[s]) >= amax - window) {
-                        const double m = fabs((double)ch[s] + (double)cl[s]);
+                    if (fabsf(c.hi(s)) >= amax - window) {
+                        const double m = fabs((double)c.hi(s) + (double)c.lo(s));
+                        const uint32_t j = At::atom(abase, s);
                         if (fabs(m - edge) < bandC) tie = true;
-                        if (m >= edge && (uint32_t)j < lower) lower = (uint32_t)j;
+                        if (m >= edge && j < lower) lower = j;
                     }
                 }
-                float wh = 0.0f, wl = 0.0f;
-                if (T > 32) {
-                    if (lane == 0) sMisc[6] = kNone;
-                    __syncthreads();
-                    if (lower != kNone) atomicMin(&sMisc[6], lower);
-                    __syncthreads();
-                    lower = sMisc[6];
-#pragma unroll
-                    for (int s = 0; s < E; ++s)
-                        if ((uint32_t)(lane + T * s) == lower) { wh = ch[s]; wl = cl[s]; }
-                    if ((uint32_t)lane == lower % (uint32_t)T) {
-                        sMisc[4] = __float_as_uint(wh);
-                        sMisc[5] = __float_as_uint(wl);
-                    }
-                    __syncthreads();
-                    wh = __uint_as_float(sMisc[4]);
-                    wl = __uint_as_float(sMisc[5]);
-                    __syncthreads();
-                } else {
-                    lower = warp_min(lower);
-#pragma unroll
-                    for (int s = 0; s < E; ++s)
-                        if ((uint32_t)(lane + T * s) == lower) { wh = ch[s]; wl = cl[s]; }
-                    wh = __shfl_sync(0xffffffffu, wh, (int)(lower & 31u));
-                    wl = __shfl_sync(0xffffffffu, wl, (int)(lower & 31u));
-                }
-                j1 = lower;
-                alpha = df{wh, wl};
+                j1 = lowest_of(lower);
+                alpha = words_of(j1);
             }
-            if (lane == 0) steps[t] = StepRec{j1, alpha.hi, alpha.lo};
-
-            // (a5) energy
-            if (energy_warp) {
-                if (DF) En = df_sub(En, df_mul(alpha, alpha));
-                else En = df{__fmaf_rn(-alpha.hi, alpha.hi, En.hi), 0.0f};
-            }
-
-            // (a4) correlation update through the Gram matrix
-            const int fam1 = (int)(j1 >= (uint32_t)n);
-            const bool owner = (uint32_t)lane == j1 % (uint32_t)T;
-            if (NF == 2) {
-                const int f1 = (int)j1 - fam1 * n;
-                const int p1 = f1 % B, q1 = f1 / B;
-                const float2 *V = fam1 ? sWT : sW;
-                const float2 vp = V[p1 * B + p_own];
-                const df u = DF ? df_mul(alpha, df{vp.x, vp.y}) : df{__fmul_rn(alpha.hi, vp.x), 0.0f};
-                const float2 *Vq = V + q1 * B;
-                if (SPLIT) {
-                    // the other family: rank-1 update and its new top-2; the
-                    // chosen atom's own family: only its owner changes
-                    if (fam1) {
-                        top[0] = update_family<B, T, E, G, 0, 0, DF>(ch, cl, lane, u, Vq);
-                        stale[0] = false;
-                        if (owner) {
-                            if (STALE && !rare) {
-                                zero_slot<E, G, G>(ch, cl, (int)(j1 / (uint32_t)T) - G);
-                                top[NG - 1] = stale_top2(top[NG - 1]);
-                                stale[NG - 1] = (top[NG - 1].P >> 32) != 0ull;
-                            } else {
-                                top[NG - 1] = zero_and_rescan<T, E, G, G>(ch, cl, lane, j1);
-                                stale[NG - 1] = false;
-                            }
-                        }
-                    } else {
-                        top[NG - 1] = update_family<B, T, E, G, G, n, DF>(ch, cl, lane, u, Vq);
-                        stale[NG - 1] = false;
-                        if (owner) {
-                            if (STALE && !rare) {
-                                zero_slot<E, G, 0>(ch, cl, (int)(j1 / (uint32_t)T));
-                                top[0] = stale_top2(top[0]);
-                                stale[0] = (top[0].P >> 32) != 0ull;
-                            } else {
-                                top[0] = zero_and_rescan<T, E, G, 0>(ch, cl, lane, j1);
-                                stale[0] = false;
-                            }
-                        }
-                    }
+            // (a4) correlation update through the Gram matrix: the other
+            // family is updated and summarised anew, the chosen element is
+            // zeroed on its owner
+            const int fam1 = NF == 2 ? (int)(j1 >= (uint32_t)n) : 0;
+            const uint32_t own1 = owner_of(j1);
+            const bool owner = (uint32_t)lane == own1;
+            const int slot1 = (int)At::slot(j1);
+            const int f1 = (int)j1 - fam1 * n;
+            const int p1 = f1 % B, q1 = f1 / B;
+            const float *Vh = sWh + fam1 * n, *Vl = sWl + fam1 * n;
+            const int col = q1 * B + G * (int)((unsigned)(SPLIT ? lane % FT : lane) / (unsigned)B);
+            auto factor = [&] {                          // alpha W[p1][p'] of this thread's row
+                const df vp{Vh[p1 * B + p_own], DF ? Vl[p1 * B + p_own] : 0.0f};
+                return DF ? df_mul(alpha, vp) : df{__fmul_rn(alpha.hi, vp.hi), 0.0f};
+            };
+            if (T == 32) {
+                if (lane == 0) steps[t] = StepRec{j1, alpha.hi, alpha.lo};
+                En = spend(En, alpha);
+                if (NF == 2) {
+                    const df u = factor();
+                    if (fam1) update_family<E, G, 0, DF>(c, sm, u, Vh + col, Vl + col);
+                    else update_family<E, G, (NG - 1) * G, DF>(c, sm, u, Vh + col, Vl + col);
+                }
+                if (NG == 2 && fam1) {
+                    zero_slot<E, G, (NG - 1) * G>(c, owner ? slot1 : -1);
+                    sm.template form<(NG - 1) * G, G>(c);
                 } else {
-                    Top2 nt = top2_empty();
-#pragma unroll
-                    for (int s = 0; s < E; ++s) {
-                        const int j = lane + T * s;
-                        if (FULL || j < M) {
-                            const int fam = (int)(j >= n);
-                            if (fam != fam1) {
-                                const int q = (j - fam * n) / B;
-                                const float2 w = Vq[q];
-                                if (DF) {
-                                    const df r = df_sub_mul(df{ch[s], cl[s]}, u, df{w.x, w.y});
-                                    ch[s] = r.hi;
-                                    cl[s] = r.lo;
-                                } else {
-                                    ch[s] = __fmaf_rn(-u.hi, w.x, ch[s]);
-                                }
-                            } else if ((uint32_t)j == j1) {
-                                ch[s] = 0.0f;
-                                cl[s] = 0.0f;
-                            }
-                            top2_fold(nt, ch[s], cl[s], (uint32_t)j);
-                        }
-                    }
-                    top[0] = nt;
+                    zero_slot<E, G, 0>(c, owner ? slot1 : -1);
+                    sm.template form<0, G>(c);
                 }
-            } else if (owner) {
-                Top2 nt = top2_empty();
-#pragma unroll
-                for (int s = 0; s < E; ++s) {
-                    const int j = lane + T * s;
-                    if (FULL || j < M) {
-                        if ((uint32_t)j == j1) { ch[s] = 0.0f; cl[s] = 0.0f; }
-                        top2_fold(nt, ch[s], cl[s], (uint32_t)j);
+            } else if (SPLIT && fam_own != fam1) {
+                update_family<E, G, 0, DF>(c, sm, factor(), Vh + col, Vl + col);
+                dirty = true;
+            } else {
+                if (warp == fam1 * (NW / 2)) {
+                    // this family's first warp: the step record, the energy
+                    // and the verdict for the next step
+                    const df e = spend(df{__uint_as_float(sMisc[12]), __uint_as_float(sMisc[13])}, alpha);
+                    const bool below = accuracy(e);
+                    if ((lane & 31) == 0) {
+                        steps[t] = StepRec{j1, alpha.hi, alpha.lo};
+                        sMisc[12] = __float_as_uint(e.hi);
+                        sMisc[13] = __float_as_uint(e.lo);
+                        sMisc[8 + ((t + 1) & 1)] = below ? 1u : 0u;
                     }
                 }
-                top[0] = nt;
+                if ((uint32_t)warp == own1 >> 5) {
+                    zero_slot<E, G, 0>(c, owner ? slot1 : -1);
+                    sm.template form<0, E>(c);
+                    dirty = true;
+                }
             }
             ++t;
         }
@@ -775,7 +757,7 @@ template <int B, int T, int NF>
 static size_t mp_smem_bytes(int k, int groups) {
     constexpr int NW = T / 32;
     size_t bytes = (NF == 2 ? 2 * B * B * sizeof(float2) : 0);
-    bytes += 3 * NW * sizeof(uint4) + 12 * sizeof(uint32_t);           // partials, misc
+    bytes += 8 * sizeof(uint4) + (3 * (NW + NW % 2) + NW % 2) * sizeof(uint2) + 16 * sizeof(uint32_t);
     bytes += NW * sizeof(unsigned long long) + NW * sizeof(uint32_t);  // full-precision partials
     bytes += (size_t)groups * k * sizeof(StepRec);
     return bytes;
@@ -821,12 +803,6 @@ __device__ __forceinline__ void update_other(float (&ch)[M], float (&cl)[M], con
             ch[O + f] = __fmaf_rn(-u[f % B].hi, w.x, ch[O + f]);
         }
     }
-}
-
-// Whether the energy lies within 2^-37 ||y||^2 of the threshold in FP64; out
-// of line, so that its FP64 work runs only when the FP32 pre-test asks.
-__device__ __noinline__ bool energy_in_band(df En, df thrE, uint32_t e0) {
-    return fabs(df_to_double(En) - df_to_double(thrE)) < ldexp((double)e0, -37);
 }
 
 // Side 4, one thread per leaf: a side-4 leaf has only 2 b^2 = 32 correlations,
@@ -1112,11 +1088,10 @@ static cudaError_t launch_mp_thread_t(const MPArgs &a, int num_sms, cudaStream_t
 template <bool DF>
 static cudaError_t launch_mp_prec(const MPArgs &a, int nf, int variant, int num_sms, cudaStream_t st) {
     const int b = a.lv.b;
-    if (b == 4 && a.lv.is_last)            // every side-4 leaf is emitted: one thread per leaf
+    if (b == 4)                            // the smallest side there is: one thread per leaf
         return nf == 2 ? launch_mp_thread_t<2, DF>(a, num_sms, st) : launch_mp_thread_t<1, DF>(a, num_sms, st);
     if (nf == 2) {
         switch (b) {
-            case 4: return launch_mp_t<4, 32, 2, DF>(a, num_sms, st);
             case 8: return launch_mp_t<8, 32, 2, DF>(a, num_sms, st);
             case 16:
                 return variant ? launch_mp_t<16, AQMP_MP_T16_ALT, 2, DF>(a, num_sms, st)
@@ -1134,7 +1109,6 @@ static cudaError_t launch_mp_prec(const MPArgs &a, int nf, int variant, int num_
         }
     } else {
         switch (b) {
-            case 4: return launch_mp_t<4, 32, 1, DF>(a, num_sms, st);
             case 8: return launch_mp_t<8, 32, 1, DF>(a, num_sms, st);
             case 16: return launch_mp_t<16, 32, 1, DF>(a, num_sms, st);
             case 32: return launch_mp_t<32, AQMP_MP_T32, 1, DF>(a, num_sms, st);

@@ -5,15 +5,16 @@
 // pairs: more than one SM holds next to its working registers.  A cluster of
 // C CTAs owns the leaf (C = 4 for the DCT + Haar union, 2 for one family):
 // with the virtual lane v = rank T + lane, thread `lane` of CTA `rank` keeps
-// the 32 elements j = v + C T s in registers -- the single-CTA kernel's
-// layout over C T threads, so every CTA holds a quarter (a half) of each
-// family and each step's update is spread evenly over the cluster.
+// 32 elements in registers -- the single-CTA kernel's layout (struct Atoms)
+// over the cluster's threads, so every CTA holds a quarter (a half) of each
+// family, on half of its warps, and each step's update is spread evenly over
+// the cluster while the other half of the warps carry the step's bookkeeping.
 //
 // A step chosen from one family updates the other through the rank-1 Gram
 // column W[p*, p'] W[q*, q'] (W = C H^T, or its transpose).  An element's row
-// p' is lane mod b, its column q' = 2 rank + lane div b + 8 s'; so a CTA reads
-// only 32 of the b columns of each table -- kept as a local slice -- and one
-// row entry W[p*, p'] per thread.  The full tables (2 x 128 KB) do not fit
+// p' is lane mod b, its column q' = 32 rank + s'; so a CTA
+// reads only 32 consecutive columns of the b of each table -- kept as a local
+// slice -- and one row entry W[p*, p'] per thread.  The full tables (2 x 128 KB) do not fit
 // one CTA; their rows are sharded over the cluster (rows 32 r .. 32 r + 31 on
 // rank r), and each thread loads its row entry from the owning peer through
 // distributed shared memory.
@@ -91,46 +92,11 @@ __device__ __forceinline__ bool try_wait_cluster(uint32_t bar, uint32_t parity) 
     return ok != 0;
 }
 
-__device__ __forceinline__ uint4 pack_top2(const Top2 &t) {
-    return make_uint4((uint32_t)t.P, (uint32_t)(t.P >> 32), t.k2, __float_as_uint(t.lo1));
-}
-
-__device__ __forceinline__ Top2 unpack_top2(const uint4 &v) {
-    return Top2{((unsigned long long)v.y << 32) | v.x, v.z, __uint_as_float(v.w)};
-}
-
 __device__ __forceinline__ float2 ld_peer_f2(uint32_t addr) {
     float2 v;
     asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
     return v;
 }
-
-// Rank-1 update of the G elements in slots [S0, S0 + G) of one family and
-// their new top-2: element (v, S0 + s2) takes u W[q*, q'] with q' the slot's
-// column, read from the CTA's column slice at wcol[2 s2].
-template <int VT, int E, int G, int S0, int TB, bool DF>
-__device__ __forceinline__ Top2 update_cols(float (&ch)[E], float (&cl)[E], int v, const df &u,
-                                            const float2 *wcol) {
-    Run2 acc = run2_empty();
-#pragma unroll
-    for (int s2 = 0; s2 < G; ++s2) {
-        const int s = S0 + s2;
-        const float2 w = wcol[TB * s2];
-        if (DF) {
-            const df r = df_sub_mul(df{ch[s], cl[s]}, u, df{w.x, w.y});
-            ch[s] = r.hi;
-            cl[s] = r.lo;
-        } else {
-            ch[s] = __fmaf_rn(-u.hi, w.x, ch[s]);
-        }
-        run2_fold(acc, ch[s], cl[s], (uint32_t)s);
-    }
-    return run2_top2<VT>(acc, v);
-}
-
-// A low word that no summary carries (a NaN pattern): marks the stop
-// verdict in warp 0's step summary.
-constexpr uint32_t kStopWord = 0x7fffffffu;
 
 // Bounded wait for phase `parity` of a local mbarrier fed by peers; false on
 // timeout or when another CTA has recorded an error (checked while waiting).
@@ -182,35 +148,40 @@ __device__ __forceinline__ bool cluster_exchange(uint4 *xs, unsigned long long *
 template <int B, int C, int NF, bool DF>
 __global__ void __launch_bounds__(kCT, 1) mp_cluster_kernel(MPArgs a) {
     constexpr int T = kCT, n = B * B, M = NF * n, VT = C * T;
-    constexpr int TB = T / B, VB = VT / B;     // a thread's columns: TB rank + lane / B + VB s
-    constexpr int E = M / VT;                  // 32 elements per thread
-    constexpr int NG = NF, G = E / NG;         // one top-2 per family
+    constexpr int FT = T / NF, FVT = VT / NF;  // threads of one family: in a CTA, in the cluster
+    constexpr int E = n / FVT;                 // 32 elements per thread, of one family
+    using At = Atoms<B, FVT, E>;
     constexpr int NW = T / 32;
     constexpr int RS = B / C;                  // table rows held per CTA (NF == 2)
     constexpr int CS = B * T / VT;             // columns of a CTA's slice (NF == 2: 32)
-    static_assert(M % VT == 0 && T % B == 0 && G * VT == n, "layout");
-    static_assert(NF == 1 || (CS % TB == 0 && RS * C == B), "slices");
+    static_assert(M % VT == 0 && T % B == 0 && FT % 32 == 0, "layout");
+    static_assert(NF == 1 || (CS == E * (FT / B) && RS * C == B), "slices");
     static_assert(C * NW <= 32, "one warp merges every warp's summary");
 
     extern __shared__ __align__(16) unsigned char smem[];
-    // NF == 2: column slices colV[fam table][q1][32] and row shards rowV[fam table][32][b]
-    float2 *sCol = reinterpret_cast<float2 *>(smem);                    // [2][B][CS]: W, W^T
-    float2 *sRow = sCol + (NF == 2 ? 2 * B * CS : 0);                   // [2][RS][B]: W, W^T
+    // NF == 2: column slices [fam table][q1][32], a plane of high and one of
+    // low words, and row shards [fam table][32][b]
+    float *sColH = reinterpret_cast<float *>(smem);                     // [2][B][CS]: W, W^T
+    float *sColL = sColH + (NF == 2 ? 2 * B * CS : 0);
+    float2 *sRow = reinterpret_cast<float2 *>(sColL + (NF == 2 ? 2 * B * CS : 0));   // [2][RS][B]: W, W^T
     unsigned char *p = reinterpret_cast<unsigned char *>(sRow + (NF == 2 ? 2 * RS * B : 0));
     uint4 *sXs = reinterpret_cast<uint4 *>(p);                          // [2][C][NW] step exchange
-    uint4 *sX = sXs + 2 * C * NW;                                       // [2][C] other exchanges
+    uint4 *sWin = sXs + 2 * C * NW;                                     // [NW] the warps' leaders
+    uint4 *sX = sWin + NW;                                              // [2][C] other exchanges
     unsigned long long *sXbar = reinterpret_cast<unsigned long long *>(sX + 2 * C);   // [2], then [2] step
     unsigned long long *sXsbar = sXbar + 2;
-    uint32_t *sMisc = reinterpret_cast<uint32_t *>(sXbar + 4);          // [16]
-    unsigned long long *sRk = reinterpret_cast<unsigned long long *>(sMisc + 16);     // [NW]
+    uint32_t *sMisc = reinterpret_cast<uint32_t *>(sXbar + 4);          // [20]
+    unsigned long long *sRk = reinterpret_cast<unsigned long long *>(sMisc + 20);     // [NW]
     uint32_t *sRj = reinterpret_cast<uint32_t *>(sRk + NW);             // [NW]
     StepRec *steps = reinterpret_cast<StepRec *>(sRj + NW);             // [k], rank 0
 
     const uint32_t rank = cluster_ctarank();
     const int lane = threadIdx.x;
-    const int vl = (int)rank * T + lane;       // virtual lane: element s is atom vl + VT s
+    const int warp = lane >> 5;
+    const int fam_own = warp / (NW / NF);      // uniform in a warp
+    const uint32_t abase = At::base((int)rank * FT + lane % FT, fam_own);
     const int p_own = lane % B;                // row p' of every element of this thread
-    const int hb = lane / B;                   // column q' = 2 rank + hb + 8 s'
+    const int hb = lane % FT / B;              // column q' = CS rank + E hb + s'
     const LevelArgs &lv = a.lv;
     volatile unsigned *err = &a.ctr->error;
     volatile uint32_t *verdict = sMisc + 12;
@@ -218,8 +189,9 @@ __global__ void __launch_bounds__(kCT, 1) mp_cluster_kernel(MPArgs a) {
     if (NF == 2) {
         for (int i = threadIdx.x; i < 2 * B * CS; i += T) {
             const int tab = i / (B * CS), r = (i / CS) % B, lc = i % CS;
-            const int q = VB * (lc / TB) + TB * (int)rank + (lc % TB);
-            sCol[i] = (tab ? a.WT : a.W)[r * B + q];
+            const float2 w = (tab ? a.WT : a.W)[r * B + CS * (int)rank + lc];
+            sColH[i] = w.x;
+            sColL[i] = w.y;
         }
         for (int i = threadIdx.x; i < 2 * RS * B; i += T) {
             const int tab = i / (RS * B), r = (i / B) % RS, c = i % B;
@@ -242,7 +214,6 @@ __global__ void __launch_bounds__(kCT, 1) mp_cluster_kernel(MPArgs a) {
     unsigned max_t = 0;
     int seq = 0, sseq = 0;
     bool aborted = false;
-    const int warp = lane >> 5;
     const uint4 *xr;
 
     for (;;) {
@@ -257,89 +228,145 @@ __global__ void __launch_bounds__(kCT, 1) mp_cluster_kernel(MPArgs a) {
         const float tol = a.planes[qe.plane].tol;
         const df eps2 = df_scale(df_two_prod(tol, tol), (float)n);
         const uint32_t e0 = a.e0[leaf];
-        df En = df_from_i64((long long)e0);
         const df thrE = df_sub(eps2, df_scale(df_from_i64((long long)e0), 0x1p-32f));
         const float bandE_f = ldexpf((float)e0, -37);
         const float eps2_f = __fmul_rn(__fmul_rn(tol, tol), (float)n);
         const float S_f = sqrtf((float)e0);
         const float pre = ldexpf(S_f, -32) * 1.05f + ldexpf(S_f, -37) * 1.05f;
 
-        float ch[E], cl[E];
-        Top2 top[NG];
+        Corr<E> c;
         const float2 *cp = a.c0 + (size_t)leaf * M;
 #pragma unroll
-        for (int g = 0; g < NG; ++g) {
-            Run2 acc = run2_empty();
-#pragma unroll
-            for (int s2 = 0; s2 < G; ++s2) {
-                const int s = g * G + s2;
-                const float2 v = cp[vl + VT * s];
-                ch[s] = v.x;
-                cl[s] = DF ? v.y : 0.0f;
-                run2_fold(acc, ch[s], cl[s], (uint32_t)s);
-            }
-            top[g] = run2_top2<VT>(acc, vl);
+        for (int s = 0; s < E; s += 2) {
+            const float2 v0 = cp[At::atom(abase, s)], v1 = cp[At::atom(abase, s + 1)];
+            c.h[s / 2] = f2_make(v0.x, v1.x);
+            c.l[s / 2] = DF ? f2_make(v0.y, v1.y) : 0ull;
         }
+        Summary<E, E> sm;
+        sm.template form<0, E>(c);
 
         int t = 0, windows = 0;
         bool conv = false, tie = false;
-        const bool energy_warp = lane < 32;
-        for (;;) {
-            // (a6) accuracy test before every step, strict (identical on every CTA)
-            bool below = false;
-            if (energy_warp) {
-                below = DF ? df_lt(En, thrE) : (En.hi < eps2_f);
-                if (DF && fabsf(En.hi - thrE.hi) <= bandE_f * 1.01f + 0x1p-20f * fabsf(thrE.hi)) {
-                    if (fabs(df_to_double(En) - df_to_double(thrE)) < ldexp((double)e0, -37)) tie = true;
-                }
+        // (a6) accuracy test on the energy, strict; taken before every step
+        auto accuracy = [&](const df &e) {
+            if (DF && __builtin_expect(fabsf(e.hi - thrE.hi) <= bandE_f * 1.01f + 0x1p-20f * fabsf(thrE.hi), 0)) {
+                if (energy_in_band(e, thrE, e0)) tie = true;
             }
-            if (t == k) {
-                if (lane == 0) sMisc[10] = below ? 1u : 0u;
-                __syncthreads();
-                conv = sMisc[10] != 0u;
-                break;
-            }
+            return DF ? df_lt(e, thrE) : (e.hi < eps2_f);
+        };
+        // the energy and the verdict for step t (word 8 + (t & 1)) live in
+        // each CTA's shared memory, alike on all of them
+        if (lane == 0) {
+            const df e = df_from_i64((long long)e0);
+            sMisc[16] = __float_as_uint(e.hi);
+            sMisc[17] = __float_as_uint(e.lo);
+            sMisc[8] = accuracy(e) ? 1u : 0u;
+        }
+        bool dirty = true;                  // this warp's leader (sWin) is to be found anew (uniform in a warp)
 
-            // (a3) argmax: every warp's top-2 goes to every CTA of the
-            // cluster (lane r < C of each warp stores it into CTA r), so
-            // after one wait each CTA holds all C NW summaries and every warp
-            // reduces them alike; warp 0's entry carries the stop verdict.
-            Top2 best;
-            {
-                Top2 wb = top[0];
-#pragma unroll
-                for (int g = 1; g < NG; ++g) wb = top2_merge(wb, top[g]);
-                wb = warp_top2(wb);
-                uint4 v = pack_top2(wb);
-                if (warp == 0 && below) v.w = kStopWord;
-                const int ss = sseq & 1;
-                const uint32_t spar = (uint32_t)(sseq >> 1) & 1u;
-                ++sseq;
-                const uint32_t sbar = sh_addr(sXsbar + ss);
-                if (lane == 0) arrive_expect_tx(sbar, (uint32_t)(C * NW * sizeof(uint4)));
-                if ((lane & 31) < C) {
-                    const uint32_t r = (uint32_t)(lane & 31);
-                    st_async_peer(peer_addr(sh_addr(sXs + (ss * C + (int)rank) * NW + warp), r), v,
-                                  peer_addr(sbar, r));
-                }
-                if (lane == 0) sMisc[13 + ss] = wait_phase(sbar, spar, err) ? 1u : 0u;
-                __syncthreads();
-                if (sMisc[13 + ss] == 0u) { aborted = true; break; }
-                const uint4 *xe = sXs + ss * C * NW;
-                if (xe[rank * NW].w == kStopWord) { conv = true; break; }
-                best = (lane & 31) < C * NW ? unpack_top2(xe[lane & 31]) : top2_empty();
-                best = warp_top2(best);
+        // Sends every warp's 16 bytes to every CTA of the cluster (lane r < C
+        // of each warp stores them into CTA r); after one wait each CTA holds
+        // all C NW of them, and lane i of every warp gets the i-th.  False
+        // when the wait gave up.
+        auto share = [&](const uint4 &mine, uint4 &got) {
+            const int ss = sseq & 1;
+            const uint32_t spar = (uint32_t)(sseq >> 1) & 1u;
+            ++sseq;
+            const uint32_t sbar = sh_addr(sXsbar + ss);
+            if (lane == 0) arrive_expect_tx(sbar, (uint32_t)(C * NW * sizeof(uint4)));
+            if ((lane & 31) < C) {
+                const uint32_t r = (uint32_t)(lane & 31);
+                st_async_peer(peer_addr(sh_addr(sXs + (ss * C + (int)rank) * NW + warp), r), mine, peer_addr(sbar, r));
             }
-            if ((best.P >> 32) == 0ull) break;   // every correlation is exactly zero
-            uint32_t j1 = top2_index(best);
-            const float amax = top2_amax(best);
-            df alpha = df{top2_negative(best) ? -amax : amax, best.lo1};
-            const float window = amax * 0x1p-20f + pre;
-            if (DF && __uint_as_float(best.k2) >= amax - window) {
+            if (lane == 0) sMisc[13 + ss] = wait_phase(sbar, spar, err) ? 1u : 0u;
+            __syncthreads();
+            if (sMisc[13 + ss] == 0u) return false;
+            got = (lane & 31) < C * NW ? sXs[ss * C * NW + (lane & 31)] : make_uint4(0u, 0u, 0u, 0u);
+            return true;
+        };
+        auto window_of = [&](float amax) { return DF ? amax * 0x1p-20f + pre : 0.0f; };
+        auto contested = [&](const Lead &l) {
+            return __uint_as_float(l.k2) >= fabsf(l.hi) - window_of(fabsf(l.hi));
+        };
+        // the lowest of the cluster's candidates, and the value of atom j from
+        // its owner to every CTA; false when an exchange gave up
+        auto lowest_of = [&](uint32_t &j) {
+            if (lane == 0) sMisc[6] = kNone;
+            __syncthreads();
+            if (j != kNone) atomicMin(&sMisc[6], j);
+            __syncthreads();
+            if (!cluster_exchange<C>(sX, sXbar, verdict, seq, rank, make_uint4(sMisc[6], 0u, 0u, 0u), err, xr))
+                return false;
+            j = kNone;
+#pragma unroll
+            for (int r = 0; r < C; ++r) j = min(j, xr[r].x);
+            return true;
+        };
+        auto words_of = [&](uint32_t j, df &w) {
+            if (lane == 0) sMisc[3] = 0u;
+            __syncthreads();
+            const df own = pick_slot<E, E, 0>(c, At::slot(j));
+            if (abase + (uint32_t)B * At::slot(j) == j) {
+                sMisc[3] = 1u;
+                sMisc[4] = __float_as_uint(own.hi);
+                sMisc[5] = __float_as_uint(own.lo);
+            }
+            __syncthreads();
+            if (!cluster_exchange<C>(sX, sXbar, verdict, seq, rank, make_uint4(sMisc[3], sMisc[4], sMisc[5], 0u), err,
+                                     xr))
+                return false;
+            w = df{0.0f, 0.0f};
+#pragma unroll
+            for (int r = 0; r < C; ++r)
+                if (xr[r].x != 0u) w = df{__uint_as_float(xr[r].y), __uint_as_float(xr[r].z)};
+            return true;
+        };
+        for (;;) {
+            // (a3) argmax: the warps' leaders, merged alike everywhere; where
+            // the runner-up may lie in the leader's decision window, again
+            // from the full words (as in the single-CTA kernel)
+            uint4 got;
+            if (dirty) {
+                uint32_t M, M2;
+                bool holds;
+                warp_two(__float_as_uint(sm.top()), 0u, M, M2, holds);
+                write_lead<At, E, E>(sm, c, abase, M, holds, M2, &sWin[warp]);
+                __syncwarp();
+            }
+            dirty = false;
+            if (!share(sWin[warp], got)) { aborted = true; break; }
+            uint32_t M, M2;
+            bool holds;
+            warp_two(got.x & 0x7fffffffu, got.w, M, M2, holds);
+            Lead best{__uint_as_float(__reduce_or_sync(0xffffffffu, holds ? got.x : 0u)),
+                      __uint_as_float(__reduce_or_sync(0xffffffffu, holds ? got.y : 0u)),
+                      __reduce_or_sync(0xffffffffu, holds ? got.z : 0u), M2};
+            if (sMisc[8 + (t & 1)] != 0u) { conv = true; break; }
+            if (t == k) break;
+            const bool exact = contested(best);
+            if (__builtin_expect(exact, 0)) {
+                const Pair2 m = magnitudes_of<E>(c);
+                uint32_t A, A2;
+                warp_two(__float_as_uint(m.m1), __float_as_uint(m.m2), A, A2, holds);
+                if (!share(make_uint4(A, A2, 0u, 0u), got)) { aborted = true; break; }
+                warp_two(got.x, got.y, A, A2, holds);
+                uint32_t j = kNone;
+#pragma unroll
+                for (int s = E - 1; s >= 0; --s)
+                    if ((__float_as_uint(c.hi(s)) & 0x7fffffffu) == A) j = At::atom(abase, s);
+                df w;
+                if (!lowest_of(j) || !words_of(j, w)) { aborted = true; break; }
+                best = Lead{w.hi, w.lo, j, A2};
+            }
+            if (best.hi == 0.0f) break;          // every correlation is exactly zero
+            uint32_t j1 = best.j;
+            df alpha = df{best.hi, best.lo};
+            if (DF && __builtin_expect(exact && contested(best), 0)) {
                 // Another atom is within the window: decide in full precision
                 // over the cluster's candidates (largest magnitude, then the
                 // lowest index within 2^-32 ||y|| of it; candidates within
                 // 2^-37 ||y|| of that edge are not certified).
+                const float amax = fabsf(best.hi), window = window_of(amax);
                 ++windows;
                 const double tieC = ldexp((double)S_f, -32);
                 const double bandC = ldexp((double)S_f, -37);
@@ -347,10 +374,10 @@ __global__ void __launch_bounds__(kCT, 1) mp_cluster_kernel(MPArgs a) {
                 uint32_t mj = kNone;
 #pragma unroll
                 for (int s = 0; s < E; ++s) {
-                    if (fabsf(ch[s]) >= amax - window) {
-                        const double m = fabs((double)ch[s] + (double)cl[s]);
+                    if (fabsf(c.hi(s)) >= amax - window) {
+                        const double m = fabs((double)c.hi(s) + (double)c.lo(s));
                         const unsigned long long key = (unsigned long long)__double_as_longlong(m);
-                        if (key > mk) { mk = key; mj = (uint32_t)(vl + VT * s); }
+                        if (key > mk) { mk = key; mj = At::atom(abase, s); }
                     }
                 }
                 warp_argmax64(mk, mj);
@@ -377,81 +404,50 @@ __global__ void __launch_bounds__(kCT, 1) mp_cluster_kernel(MPArgs a) {
                 uint32_t lower = kNone;
 #pragma unroll
                 for (int s = 0; s < E; ++s) {
-                    if (fabsf(ch[s]) >= amax - window) {
-                        const double m = fabs((double)ch[s] + (double)cl[s]);
-                        const uint32_t j = (uint32_t)(vl + VT * s);
+                    if (fabsf(c.hi(s)) >= amax - window) {
+                        const double m = fabs((double)c.hi(s) + (double)c.lo(s));
+                        const uint32_t j = At::atom(abase, s);
                         if (fabs(m - edge) < bandC) tie = true;
                         if (m >= edge && j < lower) lower = j;
                     }
                 }
-                if (lane == 0) sMisc[6] = kNone;
-                __syncthreads();
-                if (lower != kNone) atomicMin(&sMisc[6], lower);
-                __syncthreads();
-                if (!cluster_exchange<C>(sX, sXbar, verdict, seq, rank, make_uint4(sMisc[6], 0u, 0u, 0u), err,
-                                         xr)) {
-                    aborted = true;
-                    break;
-                }
-                lower = kNone;
-#pragma unroll
-                for (int r = 0; r < C; ++r) lower = min(lower, xr[r].x);
-                // the owner of `lower` publishes its value
-                if (lane == 0) sMisc[3] = 0u;
-                __syncthreads();
-#pragma unroll
-                for (int s = 0; s < E; ++s)
-                    if ((uint32_t)(vl + VT * s) == lower) {
-                        sMisc[3] = 1u;
-                        sMisc[4] = __float_as_uint(ch[s]);
-                        sMisc[5] = __float_as_uint(cl[s]);
-                    }
-                __syncthreads();
-                if (!cluster_exchange<C>(sX, sXbar, verdict, seq, rank, make_uint4(sMisc[3], sMisc[4], sMisc[5], 0u),
-                                         err, xr)) {
-                    aborted = true;
-                    break;
-                }
-                float wh = 0.0f, wl = 0.0f;
-#pragma unroll
-                for (int r = 0; r < C; ++r)
-                    if (xr[r].x != 0u) {
-                        wh = __uint_as_float(xr[r].y);
-                        wl = __uint_as_float(xr[r].z);
-                    }
+                if (!lowest_of(lower) || !words_of(lower, alpha)) { aborted = true; break; }
                 j1 = lower;
-                alpha = df{wh, wl};
             }
-            if (rank == 0 && lane == 0) steps[t] = StepRec{j1, alpha.hi, alpha.lo};
-
-            // (a5) energy
-            if (energy_warp) {
-                if (DF) En = df_sub(En, df_mul(alpha, alpha));
-                else En = df{__fmaf_rn(-alpha.hi, alpha.hi, En.hi), 0.0f};
-            }
-
             // (a4) correlation update through the Gram matrix: the other
-            // family on every CTA, the chosen element on its owner
-            const bool owner = j1 % (uint32_t)VT == (uint32_t)vl;
-            if (NF == 2) {
-                const int fam1 = (int)(j1 >= (uint32_t)n);
-                const int f1 = (int)j1 - fam1 * n;
-                const int p1 = f1 % B, q1 = f1 / B;
+            // family on every CTA, the chosen element zeroed on its owner
+            const int fam1 = NF == 2 ? (int)(j1 >= (uint32_t)n) : 0;
+            const int f1 = (int)j1 - fam1 * n;
+            const int p1 = f1 % B, q1 = f1 / B;
+            const uint32_t own1 = At::owner(j1) + (uint32_t)(fam1 * FT);    // its CTA's thread, plus FT rank
+            if (NF == 2 && fam_own != fam1) {
                 // the table of the chosen family's steps: W for a DCT atom, W^T for a Haar atom
-                const int tab = fam1;
-                const uint32_t raddr = sh_addr(sRow + (size_t)tab * RS * B + (p1 % RS) * B + p_own);
+                const uint32_t raddr = sh_addr(sRow + (size_t)fam1 * RS * B + (p1 % RS) * B + p_own);
                 const float2 vp = ld_peer_f2(peer_addr(raddr, (uint32_t)(p1 / RS)));
                 const df u = DF ? df_mul(alpha, df{vp.x, vp.y}) : df{__fmul_rn(alpha.hi, vp.x), 0.0f};
-                const float2 *wcol = sCol + (size_t)tab * B * CS + q1 * CS + hb;
-                if (fam1) {
-                    top[0] = update_cols<VT, E, G, 0, TB, DF>(ch, cl, vl, u, wcol);
-                    if (owner) top[1] = zero_and_rescan<VT, E, G, G>(ch, cl, vl, j1);
-                } else {
-                    top[1] = update_cols<VT, E, G, G, TB, DF>(ch, cl, vl, u, wcol);
-                    if (owner) top[0] = zero_and_rescan<VT, E, G, 0>(ch, cl, vl, j1);
+                const int col = fam1 * B * CS + q1 * CS + E * hb;
+                update_family<E, E, 0, DF>(c, sm, u, sColH + col, sColL + col);
+                dirty = true;
+            } else {
+                if (warp == fam1 * (NW / NF)) {
+                    // (a5) the energy, the verdict for the next step and the step record
+                    df e{__uint_as_float(sMisc[16]), __uint_as_float(sMisc[17])};
+                    e = DF ? df_sub(e, df_mul(alpha, alpha)) : df{__fmaf_rn(-alpha.hi, alpha.hi, e.hi), 0.0f};
+                    const bool below = accuracy(e);
+                    if ((lane & 31) == 0) {
+                        if (rank == 0) steps[t] = StepRec{j1, alpha.hi, alpha.lo};
+                        sMisc[16] = __float_as_uint(e.hi);
+                        sMisc[17] = __float_as_uint(e.lo);
+                        sMisc[8 + ((t + 1) & 1)] = below ? 1u : 0u;
+                    }
                 }
-            } else if (owner) {
-                top[0] = zero_and_rescan<VT, E, G, 0>(ch, cl, vl, j1);
+                const uint32_t lane1 = own1 - (uint32_t)FT * rank;             // wraps on the CTAs below the owner's
+                if ((uint32_t)warp == lane1 >> 5) {
+                    const bool owner = (uint32_t)lane == lane1;
+                    zero_slot<E, E, 0>(c, owner ? (int)At::slot(j1) : -1);
+                    sm.template form<0, E>(c);
+                    dirty = true;
+                }
             }
             ++t;
         }
@@ -547,8 +543,8 @@ static cudaError_t launch_cluster_t(const MPArgs &a, int num_sms, cudaStream_t s
     constexpr int NW = kCT / 32, CS = B * kCT / (C * kCT), RS = B / C;
     (void)num_sms;
     // NF == 2: column slices 2 x b x CS and row shards 2 x RS x b double-float pairs
-    const size_t smem = (NF == 2 ? (size_t)2 * (B * CS + RS * B) * sizeof(float2) : 0) + 2 * C * NW * sizeof(uint4) +
-                        2 * C * sizeof(uint4) + 4 * sizeof(unsigned long long) + 16 * sizeof(uint32_t) +
+    const size_t smem = (NF == 2 ? (size_t)2 * (B * CS + RS * B) * sizeof(float2) : 0) + (2 * C + 1) * NW * sizeof(uint4) +
+                        2 * C * sizeof(uint4) + 4 * sizeof(unsigned long long) + 20 * sizeof(uint32_t) +
                         NW * (sizeof(unsigned long long) + sizeof(uint32_t)) + (size_t)a.lv.k * sizeof(StepRec);
     auto kern = mp_cluster_kernel<B, C, NF, DF>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
