@@ -263,12 +263,38 @@ int aqmp_synth_backward(const aqmp_code *code, int plane, const float *grad_out,
 /* Mean SSIM (Section 3; K1 = 0.01, K2 = 0.03, L = 255, 11x11 Gaussian
  * window of sigma 1.5, valid region) of `y` against the reference `x`, both
  * h x w FP32 images with `pitch` elements per row, h, w >= 11.  Window
- * sums are accumulated in double-float (~2^-46 relative), the per-window
- * formula in FP64.  *ssim (device, FP64) receives the
+ * sums and the per-window formula are evaluated in double-float (~2^-46
+ * relative).  *ssim (device, FP64) receives the
  * mean; with grad_y != NULL, grad_y (h x w, pitch) receives
  * grad_scale * d(mean SSIM)/dy. */
 int aqmp_ssim(const float *x, const float *y, int h, int w, int64_t pitch, double *ssim,
               float *grad_y, double grad_scale, void *stream);
+
+/* The two calls above for several planes at once, as one refinement step
+ * makes them: the synthesis of every listed plane into its `recon`, and the
+ * mean SSIM of `recon` against `ref` into ssim[i] (device, FP64); with
+ * want_grad, `grad` receives d(mean SSIM)/d(recon).  `workspace` (device
+ * memory, 16-byte aligned, aqmp_refine_workspace bytes; may be NULL without
+ * want_grad) holds intermediate values and may be reused once the stream has
+ * passed the call.  All images are h x w FP32 device images of their pitch
+ * (elements per row); nothing is synchronised. */
+typedef struct {
+    int     plane;
+    int     height, width;      /* >= 11 each */
+    const float *ref;
+    int64_t ref_pitch;
+    float  *recon;
+    int64_t recon_pitch;
+    float  *grad;
+    int64_t grad_pitch;
+} aqmp_refine_plane;
+int aqmp_refine_workspace(const aqmp_refine_plane *planes, int n, uint64_t *bytes);
+int aqmp_refine_forward(const aqmp_code *code, const float *alpha, const aqmp_refine_plane *planes, int n,
+                        double *ssim, int want_grad, void *workspace, void *stream);
+/* The adjoint for all of them: grad_alpha[t] = <grad, phi_{j_t}> for the atoms
+ * of the listed planes (other entries are left untouched). */
+int aqmp_refine_backward(const aqmp_code *code, const aqmp_refine_plane *planes, int n, float *grad_alpha,
+                         void *stream);
 
 /* The initial correlation of Section 2.2 step (b) for a batch of L blocks
  * of side b: c[l][j] = <y_l, phi_j> for every atom j, with y_l the

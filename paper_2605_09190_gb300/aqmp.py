@@ -76,7 +76,8 @@ EXPORTS = ["aqmp_params_default", "aqmp_encode_planes", "aqmp_encode", "aqmp_cod
            "aqmp_synth_backward", "aqmp_ssim", "aqmp_image_to_planes", "aqmp_planes_to_image",
            "aqmp_bitstream_size", "aqmp_bitstream_write", "aqmp_bitstream_parse", "aqmp_code_from_bitstream",
            "aqmp_autotune_read", "aqmp_autotune_reset", "aqmp_profile_filter", "aqmp_encode_batch",
-           "aqmp_correlate_bf16x2", "aqmp_last_device_ms", "aqmp_selftest_round"]
+           "aqmp_correlate_bf16x2", "aqmp_last_device_ms", "aqmp_selftest_round", "aqmp_refine_workspace",
+           "aqmp_refine_forward", "aqmp_refine_backward"]
 
 
 class aqmp_tune_entry(ctypes.Structure):
@@ -93,6 +94,12 @@ class aqmp_bitstream_info(ctypes.Structure):
     _fields_ = [("version", ctypes.c_int), ("color", ctypes.c_int), ("dict_id", ctypes.c_int),
                 ("n_planes", ctypes.c_int), ("min_block", ctypes.c_int), ("max_block", ctypes.c_int),
                 ("n_leaves", ctypes.c_uint64), ("n_atoms", ctypes.c_uint64)]
+
+
+class aqmp_refine_plane(ctypes.Structure):
+    _fields_ = [("plane", ctypes.c_int), ("height", ctypes.c_int), ("width", ctypes.c_int),
+                ("ref", ctypes.c_void_p), ("ref_pitch", ctypes.c_int64), ("recon", ctypes.c_void_p),
+                ("recon_pitch", ctypes.c_int64), ("grad", ctypes.c_void_p), ("grad_pitch", ctypes.c_int64)]
 
 
 class aqmp_kernel_time(ctypes.Structure):
@@ -133,6 +140,9 @@ def load_library(path: str | None = None):
         lib.aqmp_synth_forward.argtypes = [V, I, V, V, I64, V]
         lib.aqmp_synth_backward.argtypes = [V, I, V, I64, V, V]
         lib.aqmp_ssim.argtypes = [V, V, I, I, I64, V, V, ctypes.c_double, V]
+        lib.aqmp_refine_workspace.argtypes = [V, I, U64P]
+        lib.aqmp_refine_forward.argtypes = [V, V, V, I, V, I, V, V]
+        lib.aqmp_refine_backward.argtypes = [V, V, I, V, V]
         lib.aqmp_num_atoms.argtypes = [I, I]
         lib.aqmp_last_error.restype = ctypes.c_char_p
         lib.aqmp_last_device_ms.argtypes = [ctypes.POINTER(ctypes.c_double)]
@@ -496,6 +506,33 @@ def aqmp_ssim(x, y, ssim_out, grad_y=None, grad_scale: float = 1.0, stream=None)
                                     ctypes.c_void_p(grad_y.data_ptr()) if grad_y is not None else None,
                                     float(grad_scale), _stream_handle(stream)))
     return ssim_out
+
+
+def aqmp_refine_planes(rows):
+    """The C array of (plane, h, w, ref ptr, pitch, recon ptr, pitch, grad ptr, pitch) rows."""
+    return (aqmp_refine_plane * len(rows))(*rows)
+
+
+def aqmp_refine_workspace(planes) -> int:
+    n = ctypes.c_uint64()
+    _check(load_library().aqmp_refine_workspace(planes, len(planes), ctypes.byref(n)))
+    return n.value
+
+
+def aqmp_refine_forward(code: Code, alpha, planes, ssim, workspace=None, stream=None):
+    """Synthesis and mean SSIM of every plane (ssim: CUDA float64 tensor of
+    their number); with a workspace also their gradient images."""
+    _check(load_library().aqmp_refine_forward(code.handle, ctypes.c_void_p(alpha.data_ptr()), planes, len(planes),
+                                              ctypes.c_void_p(ssim.data_ptr()), 0 if workspace is None else 1,
+                                              None if workspace is None else ctypes.c_void_p(workspace.data_ptr()),
+                                              _stream_handle(stream)))
+    return ssim
+
+
+def aqmp_refine_backward(code: Code, planes, grad_alpha, stream=None):
+    _check(load_library().aqmp_refine_backward(code.handle, planes, len(planes),
+                                               ctypes.c_void_p(grad_alpha.data_ptr()), _stream_handle(stream)))
+    return grad_alpha
 
 
 # ---------------------------------------------------------------- codec stages

@@ -1,299 +1,252 @@
-// diff.cu -- refinement of the coefficients on a fixed MP support: sparse
-// synthesis (Algorithm 3) with caller coefficients and its adjoint, and the
-// mean SSIM of Section 3 with its gradient with respect to the
-// reconstruction, all on the device.
+// diff.cu -- the adjoint of the sparse synthesis (Algorithm 3 with caller
+// coefficients on a fixed MP support), for the refinement.
 //
-// Synthesis: recon[y+i][x+m] = sum_t alpha_t B[p_t][i] B[q_t][m] per leaf.
-// Adjoint: d recon / d alpha_t is the atom itself, so
-// grad alpha_t = <G_leaf, phi_t> = (B G B^T)[p_t][q_t] for the leaf's block G
-// of the incoming gradient; the block transform is computed once per leaf
-// and family (two b x b products) and gathered at the leaf's atoms.
+// Synthesis: recon[y+i][x+m] = sum_t alpha_t B[p_t][i] B[q_t][m] per leaf
+// (decode.cu).  Adjoint: d recon / d alpha_t is the atom itself, so
+// grad alpha_t = <G_leaf, phi_t> for the leaf's block G of the incoming
+// gradient = (B G B^T)[p_t][q_t]: U = B G, T = U B^T per family, then a gather
+// at the leaf's atoms.  FP32, each entry summed in ascending order.
 //
-// SSIM over the valid region with an 11 x 11 Gaussian window w = g g^T
-// (sigma 1.5), K1 = 0.01, K2 = 0.03, L = 255.  Per window:
-//   A1 = 2 mx my + C1, A2 = 2 (Exy - mx my) + C2,
-//   B1 = mx^2 + my^2 + C1, B2 = (Exx - mx^2) + (Eyy - my^2) + C2,
-//   f = A1 A2 / (B1 B2).
-// With S = mean f over the N windows, for a pixel k of y:
-//   dS/dy[k] = (1/N) sum_win w(k - win) (f_my + 2 y[k] f_Eyy + x[k] f_Exy),
-//   f_my = f (2 mx / A1 - 2 mx / A2 - 2 my / B1 + 2 my / B2),
-//   f_Exy = 2 f / A2,   f_Eyy = -f / B2,
-// i.e. the per-window partials filtered back with the (symmetric, separable)
-// window.  The window statistics and the back-filtered partials are
-// accumulated in double-float; the per-window formula runs in FP64.
+// Sides up to 32 take a warp per leaf, 64 and 128 a CTA.  A lane computes
+// tiles of 4 x 4 entries (2 x 2 at side 8, one at side 4), so 64 multiply-adds
+// share eight 16-byte loads -- one entry at a time took two loads for each
+// multiply-add and was bound by the load pipe.  Stage 1's lanes run along m
+// (rows of B broadcast, rows of G contiguous), stage 2's along p (rows of B
+// broadcast again, rows of U in a layout that spreads their 16-byte words over
+// the banks), so no transposed copy of the basis is needed.
+// 16 planes of 512x512, sides 32..8: 2.2 ms in 16 launches -> 75 us in one.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
 #include "kernels.h"
+#include "leaf_tasks.cuh"
 
 namespace aqmp {
 
 namespace {
 
-__constant__ double c_gauss[11];
+constexpr int kWarpThreads = 256;                         // of the warp-per-leaf kernel
+constexpr int kWarpFloats = 3 * 32 * 32;                  // G, U, T of side 32; sides <= 16: G, two each
+constexpr int kCtaThreads = 256;
 
-__device__ __forceinline__ int ilog2_dev(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
+template <int B>
+constexpr int tile_edge() { return B >= 16 ? 4 : B == 8 ? 2 : 1; }
 
-// One CTA per leaf: T_fam = B G B^T for the families present, then gather.
-__global__ void synth_backward_kernel(const LeafRec *leaves, unsigned long long n_leaves, const AtomRec *atoms,
-                                      uint32_t plane, const float *grad, long long pitch, float *grad_alpha,
-                                      DecodeArgs bases) {
-    extern __shared__ float sm[];
-    for (unsigned long long li = blockIdx.x; li < n_leaves; li += gridDim.x) {
-        const LeafRec L = leaves[li];
-        if (L.plane != plane || L.n_atoms == 0) continue;
-        const int b = L.b, n = b * b;
-        const float *basis = bases.basis[ilog2_dev(b)];
-        const int nfam = bases.nf;
-        float *G = sm;               // b x b gradient block, G[i][m]
-        float *U = G + n;            // B G (per family), U[p][m]
-        float *Tc = U + n;           // one family's coefficients Tc[p][q]
-        __syncthreads();
-        for (int v = threadIdx.x; v < n; v += blockDim.x) {
-            const int i = v / b, m = v - i * b;
-            G[v] = grad[(long long)(L.y + i) * pitch + L.x + m];
+// Word of U[p][m]: 16-byte words of a row exchanged by its tile row, so that
+// the tiles of a column of tiles lie in different banks.
+template <int B>
+__device__ __forceinline__ int u_at(int p, int m) {
+    return B >= 16 ? p * B + ((((m >> 2) ^ (p >> 2)) & (B / 4 - 1)) << 2) + (m & 3) : p * B + m;
+}
+
+template <int N>
+__device__ __forceinline__ void load_n(const float *src, float (&v)[N]) {
+    if constexpr (N == 4) {
+        const float4 x = *reinterpret_cast<const float4 *>(src);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else if constexpr (N == 2) {
+        const float2 x = *reinterpret_cast<const float2 *>(src);
+        v[0] = x.x; v[1] = x.y;
+    } else {
+        v[0] = *src;
+    }
+}
+
+template <int N>
+__device__ __forceinline__ void store_n(float *dst, const float (&v)[N]) {
+    if constexpr (N == 4) *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+    else if constexpr (N == 2) *reinterpret_cast<float2 *>(dst) = make_float2(v[0], v[1]);
+    else *dst = v[0];
+}
+
+// U = Bf G, thread `t` of NT.
+template <int B, int NT>
+__device__ __forceinline__ void stage1(const float *Bf, const float *G, float *U, int t) {
+    constexpr int E = tile_edge<B>(), TB = B / E;
+    for (int tile = t; tile < TB * TB; tile += NT) {
+        const int p0 = tile / TB * E, m0 = tile % TB * E;
+        float s[E][E];
+#pragma unroll
+        for (int r = 0; r < E; ++r)
+#pragma unroll
+            for (int c = 0; c < E; ++c) s[r][c] = 0.0f;
+#pragma unroll 4
+        for (int i = 0; i < B; i += 4) {
+            float b[E][4], g[4][E];
+#pragma unroll
+            for (int r = 0; r < E; ++r) load_n<4>(Bf + (p0 + r) * B + i, b[r]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) load_n<E>(G + (i + k) * B + m0, g[k]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int r = 0; r < E; ++r)
+#pragma unroll
+                    for (int c = 0; c < E; ++c) s[r][c] = __fmaf_rn(b[r][k], g[k][c], s[r][c]);
         }
-        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < E; ++r) store_n<E>(U + u_at<B>(p0 + r, m0), s[r]);
+    }
+}
+
+// T[q][p] = (U Bf^T)[p][q].
+template <int B, int NT>
+__device__ __forceinline__ void stage2(const float *Bf, const float *U, float *T, int t) {
+    constexpr int E = tile_edge<B>(), TB = B / E;
+    for (int tile = t; tile < TB * TB; tile += NT) {
+        const int p0 = tile % TB * E, q0 = tile / TB * E;
+        float s[E][E];                                     // [q][p]
+#pragma unroll
+        for (int r = 0; r < E; ++r)
+#pragma unroll
+            for (int c = 0; c < E; ++c) s[c][r] = 0.0f;
+#pragma unroll 4
+        for (int m = 0; m < B; m += 4) {
+            float u[E][4], b[E][4];
+#pragma unroll
+            for (int r = 0; r < E; ++r) load_n<4>(U + u_at<B>(p0 + r, m), u[r]);
+#pragma unroll
+            for (int c = 0; c < E; ++c) load_n<4>(Bf + (q0 + c) * B + m, b[c]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int r = 0; r < E; ++r)
+#pragma unroll
+                    for (int c = 0; c < E; ++c) s[c][r] = __fmaf_rn(u[r][k], b[c][k], s[c][r]);
+        }
+#pragma unroll
+        for (int c = 0; c < E; ++c) store_n<E>(T + (q0 + c) * B + p0, s[c]);
+    }
+}
+
+template <int NT>
+__device__ __forceinline__ void sync_group() {
+    if (NT <= 32) __syncwarp();
+    else __syncthreads();
+}
+
+// One leaf on NT threads; sm: 3 b^2 floats (5 b^2 up to side 16, where the two
+// families run side by side on half of the warp each).
+template <int B, int NT>
+__device__ __forceinline__ void adjoint_leaf(const AdjointArgs &a, const LeafRec &L, float *sm, int t) {
+    constexpr int n = B * B, LG = B == 4 ? 2 : B == 8 ? 3 : B == 16 ? 4 : B == 32 ? 5 : B == 64 ? 6 : 7;
+    constexpr bool BOTH = B <= 16;
+    if (L.n_atoms == 0) return;
+    const int nfam = a.bases.nf, img = (int)(L.plane - a.grad.plane);
+    const long long pitch = a.grad.pitch[img];
+    const float *src = a.grad.img[img] + (long long)L.y * pitch + L.x;
+    float *G = sm, *U = G + n, *T = U + (BOTH ? 2 * n : n);
+#pragma unroll 8
+    for (int v = t; v < n; v += NT) G[v] = src[(long long)(v / B) * pitch + v % B];
+    sync_group<NT>();
+    const float *basis = a.bases.basis[LG] + (nfam == 1 ? a.bases.single_family * n : 0);
+    const AtomRec *atoms = a.atoms + L.atom_off;
+    float *out = a.grad_alpha + L.atom_off;
+    if constexpr (BOTH) {
+        const int fam = t / (NT / 2), ft = t % (NT / 2);
+        if (fam < nfam) stage1<B, NT / 2>(basis + fam * n, G, U + fam * n, ft);
+        sync_group<NT>();
+        if (fam < nfam) stage2<B, NT / 2>(basis + fam * n, U + fam * n, T + fam * n, ft);
+        sync_group<NT>();
+        for (int i = t; i < L.n_atoms; i += NT) {
+            const uint32_t j = atoms[i].j;
+            if (j < (uint32_t)(nfam * n)) out[i] = T[j];       // T[fam][q][p] at fam n + q b + p
+        }
+    } else {
         for (int fam = 0; fam < nfam; ++fam) {
-            const float *B = basis + (nfam == 1 ? bases.single_family : fam) * b * b;
-            for (int v = threadIdx.x; v < n; v += blockDim.x) {          // U = B G
-                const int p = v / b, m = v - p * b;
-                float s = 0.0f;
-                for (int i = 0; i < b; ++i) s = __fmaf_rn(B[p * b + i], G[i * b + m], s);
-                U[v] = s;
+            stage1<B, NT>(basis + fam * n, G, U, t);
+            sync_group<NT>();
+            stage2<B, NT>(basis + fam * n, U, T, t);
+            sync_group<NT>();
+            for (int i = t; i < L.n_atoms; i += NT) {
+                const uint32_t f = atoms[i].j - (uint32_t)(fam * n);
+                if (f < (uint32_t)n) out[i] = T[f];
             }
-            __syncthreads();
-            for (int v = threadIdx.x; v < n; v += blockDim.x) {          // T = U B^T
-                const int p = v / b, q = v - p * b;
-                float s = 0.0f;
-                for (int m = 0; m < b; ++m) s = __fmaf_rn(U[p * b + m], B[q * b + m], s);
-                Tc[v] = s;
-            }
-            __syncthreads();
-            for (int t = threadIdx.x; t < L.n_atoms; t += blockDim.x) {    // this family's atoms
-                const uint32_t j = atoms[L.atom_off + t].j;
-                const int fa = nfam == 2 ? (int)(j >= (uint32_t)n) : 0;
-                if (fa != fam) continue;
-                const int f = (int)j - (nfam == 2 ? fa * n : 0);
-                grad_alpha[L.atom_off + t] = Tc[(f % b) * b + (f / b)];
-            }
-            __syncthreads();
         }
     }
+    sync_group<NT>();
 }
 
-// The 11-tap passes run in double-float on the FP32 pipes (GB300's FP64
-// rate is a small fraction of its FP32 rate): each tap adds g v with the
-// weight g as a (hi, lo) pair and v a pixel, an exact pixel product, or a
-// stored pair, so the window sums keep ~2^-46 relative accuracy and
-// E[x^2] - mu^2 is formed in FP64 from them without losing the variance.
-// Intermediate planes hold (hi, lo) float pairs in the 8-byte slots.
-__constant__ float2 c_gauss_df[11];
-
-__device__ __forceinline__ df gw(int j) {
-    const float2 g = c_gauss_df[j];
-    return df{-g.x, -g.y};                          // negated: s - (-g) v = s + g v
-}
-
-__device__ __forceinline__ df df_of(double d) {
-    const float hi = (float)d;
-    return df{hi, (float)(d - (double)hi)};
-}
-
-// Horizontal 11-tap pass of the five products (x, y, x^2, y^2, x y) over the
-// valid columns: H[k][row][a] for a < w - 10.
-__global__ void ssim_hpass_kernel(const float *x, const float *y, int h, int w, long long pitch, float2 *H) {
-    const int wo = w - 10;
-    const long long plane = (long long)h * wo;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < plane;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(idx / wo), a = (int)(idx - (long long)r * wo);
-        df sx{0.0f, 0.0f}, sy = sx, sxx = sx, syy = sx, sxy = sx;
-#pragma unroll
-        for (int j = 0; j < 11; ++j) {
-            const df g = gw(j);
-            const float xv = x[(long long)r * pitch + a + j], yv = y[(long long)r * pitch + a + j];
-            sx = df_sub_mul(sx, g, df{xv, 0.0f});
-            sy = df_sub_mul(sy, g, df{yv, 0.0f});
-            sxx = df_sub_mul(sxx, g, df_two_prod(xv, xv));
-            syy = df_sub_mul(syy, g, df_two_prod(yv, yv));
-            sxy = df_sub_mul(sxy, g, df_two_prod(xv, yv));
-        }
-        H[idx] = make_float2(sx.hi, sx.lo);
-        H[plane + idx] = make_float2(sy.hi, sy.lo);
-        H[2 * plane + idx] = make_float2(sxx.hi, sxx.lo);
-        H[3 * plane + idx] = make_float2(syy.hi, syy.lo);
-        H[4 * plane + idx] = make_float2(sxy.hi, sxy.lo);
+__device__ __forceinline__ void plane_range(const AdjointArgs &a, unsigned long long (&range)[2]) {
+    const int warp = threadIdx.x >> 5;
+    if (warp < 2) {
+        const uint32_t plane = a.grad.plane + (uint32_t)(warp ? a.grad.n_planes : 0);
+        const unsigned long long at = first_of_plane(a.leaves, a.n_leaves, plane);
+        if ((threadIdx.x & 31) == 0) range[warp] = at;
     }
-}
-
-// Vertical pass, SSIM per window, its partials (scaled) and the mean.  The
-// window formula runs in FP64 from the double-float sums, with one division.
-__global__ void ssim_window_kernel(const float2 *H, int h, int w, double *P, double *sum, double gscale) {
-    const int wo = w - 10, ho = h - 10;
-    const long long hplane = (long long)h * wo, wins = (long long)ho * wo;
-    const double C1 = (0.01 * 255.0) * (0.01 * 255.0), C2 = (0.03 * 255.0) * (0.03 * 255.0);
-    double local = 0.0;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < wins;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(idx / wo), a = (int)(idx - (long long)r * wo);
-        df m[5];
-#pragma unroll
-        for (int k = 0; k < 5; ++k) m[k] = df{0.0f, 0.0f};
-#pragma unroll
-        for (int i = 0; i < 11; ++i) {
-            const df g = gw(i);
-            const long long o = (long long)(r + i) * wo + a;
-#pragma unroll
-            for (int k = 0; k < 5; ++k) {
-                const float2 v = H[k * hplane + o];
-                m[k] = df_sub_mul(m[k], g, df{v.x, v.y});
-            }
-        }
-        const double mx = df_to_double(m[0]), my = df_to_double(m[1]);
-        const double exx = df_to_double(m[2]), eyy = df_to_double(m[3]), exy = df_to_double(m[4]);
-        const double A1 = 2 * mx * my + C1, A2 = 2 * (exy - mx * my) + C2;
-        const double B1 = mx * mx + my * my + C1, B2 = (exx - mx * mx) + (eyy - my * my) + C2;
-        const double A12 = A1 * A2, B12 = B1 * B2;
-        const double r1 = 1.0 / (A12 * B12);                 // 1 / (A1 A2 B1 B2)
-        const double f = A12 * A12 * r1;                      // A1 A2 / (B1 B2)
-        local += f;
-        if (P) {
-            const double iA1 = A2 * B12 * r1, iA2 = A1 * B12 * r1, iB1 = A12 * B2 * r1, iB2 = A12 * B1 * r1;
-            P[idx] = gscale * f * (2 * mx * iA1 - 2 * mx * iA2 - 2 * my * iB1 + 2 * my * iB2);   // f_my
-            P[wins + idx] = gscale * (-f * iB2);                                              // f_Eyy
-            P[2 * wins + idx] = gscale * (2 * f * iA2);                                       // f_Exy
-        }
-    }
-    // block sum, one atomic per block
-    __shared__ double red[32];
-    for (int off = 16; off > 0; off >>= 1) local += __shfl_xor_sync(0xffffffffu, local, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = local;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        double v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (threadIdx.x == 0) atomicAdd(sum, v / (double)wins);
-    }
 }
 
-// Back through the vertical pass: V[k][row][a] = sum_i g[i] P[k][row - i][a]
-// over the windows whose first row is row - i (full height, valid columns).
-__global__ void ssim_vback_kernel(const double *P, int h, int w, float2 *V) {
-    const int wo = w - 10, ho = h - 10;
-    const long long wins = (long long)ho * wo, vplane = (long long)h * wo;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < vplane;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(idx / wo), a = (int)(idx - (long long)r * wo);
-        df s0{0.0f, 0.0f}, s1 = s0, s2 = s0;
-#pragma unroll
-        for (int i = 0; i < 11; ++i) {
-            const int wr = r - i;
-            if (wr < 0 || wr >= ho) continue;
-            const df g = gw(i);
-            const long long o = (long long)wr * wo + a;
-            s0 = df_sub_mul(s0, g, df_of(P[o]));
-            s1 = df_sub_mul(s1, g, df_of(P[wins + o]));
-            s2 = df_sub_mul(s2, g, df_of(P[2 * wins + o]));
-        }
-        V[idx] = make_float2(s0.hi, s0.lo);
-        V[vplane + idx] = make_float2(s1.hi, s1.lo);
-        V[2 * vplane + idx] = make_float2(s2.hi, s2.lo);
-    }
+// Leaves of side <= 32, a warp each.
+__global__ void __launch_bounds__(kWarpThreads) adjoint_warp_kernel(const __grid_constant__ AdjointArgs a) {
+    extern __shared__ __align__(16) float sm_all[];
+    __shared__ unsigned long long range[2];
+    plane_range(a, range);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *sm = sm_all + warp * kWarpFloats;
+    for_tiles(
+        a.leaves, range[0], (unsigned)(range[1] - range[0]), 1u, blockIdx.x + gridDim.x * (unsigned)warp,
+        gridDim.x * (kWarpThreads / 32), [](int b) { return b <= 32 ? 1 : 0; },
+        [&](const LeafRec &L, unsigned long long, int) {
+            switch (L.b) {
+                case 4: adjoint_leaf<4, 32>(a, L, sm, lane); break;
+                case 8: adjoint_leaf<8, 32>(a, L, sm, lane); break;
+                case 16: adjoint_leaf<16, 32>(a, L, sm, lane); break;
+                case 32: adjoint_leaf<32, 32>(a, L, sm, lane); break;
+                default: break;
+            }
+        });
 }
 
-// Back through the horizontal pass and the products:
-// grad_y[r][c] = G1 + 2 y G2 + x G3 with G_k[r][c] = sum_j g[j] V[k][r][c - j].
-__global__ void ssim_hback_kernel(const float2 *V, const float *x, const float *y, int h, int w, long long pitch,
-                                  float *grad) {
-    const int wo = w - 10;
-    const long long vplane = (long long)h * wo, npix = (long long)h * w;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < npix;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(idx / w), c = (int)(idx - (long long)r * w);
-        df g1{0.0f, 0.0f}, g2 = g1, g3 = g1;
-#pragma unroll
-        for (int j = 0; j < 11; ++j) {
-            const int a = c - j;
-            if (a < 0 || a >= wo) continue;
-            const df g = gw(j);
-            const long long o = (long long)r * wo + a;
-            const float2 v1 = V[o], v2 = V[vplane + o], v3 = V[2 * vplane + o];
-            g1 = df_sub_mul(g1, g, df{v1.x, v1.y});
-            g2 = df_sub_mul(g2, g, df{v2.x, v2.y});
-            g3 = df_sub_mul(g3, g, df{v3.x, v3.y});
+// Leaves of side 64 and 128, a CTA each: leaves blockIdx.x + gridDim.x i, 256
+// of them looked over at a time.
+__global__ void __launch_bounds__(kCtaThreads) adjoint_cta_kernel(const __grid_constant__ AdjointArgs a) {
+    extern __shared__ __align__(16) float sm_all[];
+    __shared__ unsigned long long range[2];
+    __shared__ unsigned list[kCtaThreads], found;
+    plane_range(a, range);
+    const unsigned count = (unsigned)(range[1] - range[0]);
+    for (unsigned long long base = blockIdx.x; base < count; base += (unsigned long long)gridDim.x * kCtaThreads) {
+        if (threadIdx.x == 0) found = 0u;
+        __syncthreads();
+        const unsigned long long at = base + (unsigned long long)gridDim.x * threadIdx.x;
+        if (at < count && a.leaves[range[0] + at].b >= 64) list[atomicAdd(&found, 1u)] = (unsigned)at;
+        __syncthreads();
+        for (unsigned i = 0; i < found; ++i) {
+            const LeafRec L = a.leaves[range[0] + list[i]];
+            if (L.b == 64) adjoint_leaf<64, kCtaThreads>(a, L, sm_all, (int)threadIdx.x);
+            else if (L.b == 128) adjoint_leaf<128, kCtaThreads>(a, L, sm_all, (int)threadIdx.x);
         }
-        const float xv = x[(long long)r * pitch + c], yv = y[(long long)r * pitch + c];
-        // g1 + 2 y g2 + x g3
-        df t = df_sub_mul(g1, df{-2.0f * yv, 0.0f}, g2);
-        t = df_sub_mul(t, df{-xv, 0.0f}, g3);
-        grad[(long long)r * pitch + c] = __fadd_rn(t.hi, t.lo);
+        __syncthreads();
     }
 }
 
 }  // namespace
 
-cudaError_t upload_gauss11(cudaStream_t st) {
-    double g[11], s = 0.0;
-    for (int i = 0; i < 11; ++i) {
-        const double r = i - 5.0;
-        g[i] = exp(-(r * r) / (2.0 * 1.5 * 1.5));
-        s += g[i];
+cudaError_t launch_synth_backward(const AdjointArgs &a, int num_sms, cudaStream_t st) {
+    if (a.n_leaves == 0) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    const float *const *basis = a.bases.basis;
+    if (basis[2] || basis[3] || basis[4] || basis[5]) {
+        constexpr size_t smem = sizeof(float) * kWarpFloats * (kWarpThreads / 32);
+        e = cudaFuncSetAttribute(adjoint_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        unsigned long long blocks = (a.n_leaves + kWarpThreads / 32 - 1) / (kWarpThreads / 32);
+        if (blocks > (unsigned long long)num_sms * 2) blocks = (unsigned long long)num_sms * 2;
+        adjoint_warp_kernel<<<(unsigned)blocks, kWarpThreads, smem, st>>>(a);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    for (int i = 0; i < 11; ++i) g[i] /= s;
-    float2 gf[11];
-    for (int i = 0; i < 11; ++i) {
-        gf[i].x = (float)g[i];
-        gf[i].y = (float)(g[i] - (double)gf[i].x);
+    if (basis[6] || basis[7]) {
+        const size_t side = basis[7] ? 128 : 64, smem = sizeof(float) * 3 * side * side;
+        e = cudaFuncSetAttribute(adjoint_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        unsigned long long blocks = a.n_leaves;
+        const unsigned long long cap = (unsigned long long)num_sms * (basis[7] ? 1 : 4);
+        if (blocks > cap) blocks = cap;
+        adjoint_cta_kernel<<<(unsigned)blocks, kCtaThreads, smem, st>>>(a);
+        e = cudaGetLastError();
     }
-    cudaError_t e = cudaMemcpyToSymbolAsync(c_gauss, g, sizeof g, 0, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return e;
-    return cudaMemcpyToSymbolAsync(c_gauss_df, gf, sizeof gf, 0, cudaMemcpyHostToDevice, st);
-}
-
-cudaError_t launch_synth_forward(const LeafRec *leaves, unsigned long long n_leaves, const AtomRec *atoms,
-                                 const float *alpha, uint32_t plane, float *out, long long pitch,
-                                 const DecodeArgs &bases, int num_sms, cudaStream_t st) {
-    // the decoder with caller coefficients (decode.cu)
-    DecodeArgs a = bases;
-    a.leaves = leaves;
-    a.n_leaves = n_leaves;
-    a.atoms = atoms;
-    a.plane = plane;
-    a.out = out;
-    a.out_pitch = pitch;
-    return launch_decode_alpha(a, alpha, num_sms, st);
-}
-
-cudaError_t launch_synth_backward(const LeafRec *leaves, unsigned long long n_leaves, const AtomRec *atoms,
-                                  uint32_t plane, const float *grad, long long pitch, float *grad_alpha,
-                                  const DecodeArgs &bases, int max_side, int num_sms, cudaStream_t st) {
-    if (n_leaves == 0) return cudaSuccess;
-    const size_t smem = sizeof(float) * (size_t)max_side * max_side * 3;   // G, U, Tc
-    cudaError_t e = cudaFuncSetAttribute(synth_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    long long blocks = (long long)n_leaves;
-    if (blocks > (long long)num_sms * 8) blocks = (long long)num_sms * 8;
-    synth_backward_kernel<<<(unsigned)blocks, 256, smem, st>>>(leaves, n_leaves, atoms, plane, grad, pitch,
-                                                                grad_alpha, bases);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_ssim(const float *x, const float *y, int h, int w, long long pitch, double *H, double *P,
-                        double *V, double *sum, float *grad, double gscale, int num_sms, cudaStream_t st) {
-    const unsigned grid = (unsigned)num_sms * 8;
-    float2 *Hf = reinterpret_cast<float2 *>(H), *Vf = reinterpret_cast<float2 *>(V);   // (hi, lo) in 8-byte slots
-    ssim_hpass_kernel<<<grid, 256, 0, st>>>(x, y, h, w, pitch, Hf);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const long long wins = (long long)(h - 10) * (w - 10);
-    const double scale = grad ? gscale / (double)wins : 0.0;
-    ssim_window_kernel<<<grid, 256, 0, st>>>(Hf, h, w, grad ? P : nullptr, sum, scale);
-    if ((e = cudaGetLastError()) != cudaSuccess || !grad) return e;
-    ssim_vback_kernel<<<grid, 256, 0, st>>>(P, h, w, Vf);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    ssim_hback_kernel<<<grid, 256, 0, st>>>(Vf, x, y, h, w, pitch, grad);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace aqmp

@@ -377,7 +377,6 @@ struct Ctx {
     std::map<int, std::unique_ptr<Dict>> dicts;
     DeviceBuf planes, staging, queues, Y, e0, c0, counters, ssim_ws, Y8, inv_sl, omp_L, mu_buf, ebound, fbq;
     DeviceBuf leaves_ws, atoms_ws, lo_ws, atom_leaf, cells, perm, new_off, order_status;   // emission -> canonical order
-    bool gauss_ready = false;
     Tuner tuner;
     Counters *host_ctr = nullptr;             // pinned
     cudaMemPool_t out_pool = nullptr;         // encode outputs (aqmp_code arrays)
@@ -1310,6 +1309,20 @@ int aqmp_code_copy(const aqmp_code *code, aqmp_leaf *leaves, aqmp_atom *atoms, f
     return AQMP_OK;
 }
 
+// Basis tables of every side a code uses, for the synthesis kernels.
+static int code_bases(Ctx *c, const aqmp_code *code, cudaStream_t st, Bases *a) {
+    *a = Bases{};
+    a->nf = num_families(code->dict_id);
+    a->single_family = 0;
+    for (int b = code->min_block; b <= code->max_block; b *= 2) {
+        Dict *d;
+        int rc = get_dict(c, b, code->dict_id, st, &d, false);
+        if (rc) return rc;
+        a->basis[ilog2(b)] = d->d.basis;
+    }
+    return AQMP_OK;
+}
+
 int aqmp_decode(const aqmp_code *code, int plane, float *out, int64_t out_pitch, int out_is_device, void *stream) {
     g_last_error.clear();
     if (!code || !out || plane < 0 || plane >= (int)code->shapes.size()) return fail(AQMP_E_ARG, "bad argument");
@@ -1324,14 +1337,7 @@ int aqmp_decode(const aqmp_code *code, int plane, float *out, int64_t out_pitch,
     a.leaves = code->leaves;
     a.n_leaves = code->n_leaves;
     a.atoms = code->atoms;
-    a.plane = (uint32_t)plane;
-    a.nf = num_families(code->dict_id);
-    a.single_family = 0;
-    for (int b = code->min_block; b <= code->max_block; b *= 2) {
-        Dict *d;
-        if ((rc = get_dict(c, b, code->dict_id, st, &d, false))) return rc;
-        a.basis[ilog2(b)] = d->d.basis;
-    }
+    if ((rc = code_bases(c, code, st, &a.bases))) return rc;
     float *dst = out;
     long long pitch = out_pitch;
     void *tmp = nullptr;
@@ -1340,8 +1346,10 @@ int aqmp_decode(const aqmp_code *code, int plane, float *out, int64_t out_pitch,
         dst = (float *)tmp;
         pitch = w;
     }
-    a.out = dst;
-    a.out_pitch = pitch;
+    a.out.plane = (uint32_t)plane;
+    a.out.n_planes = 1;
+    a.out.img[0] = dst;
+    a.out.pitch[0] = pitch;
     cudaError_t e = g_prof.run(kname("decode", code->max_block), st, [&] { return launch_decode(a, c->num_sms, st); });
     if (e == cudaSuccess && !out_is_device)
         e = cudaMemcpy2DAsync(out, sizeof(float) * out_pitch, dst, sizeof(float) * w, sizeof(float) * w, h,
@@ -1368,16 +1376,32 @@ int aqmp_code_device(const aqmp_code *code, const aqmp_leaf **leaves, const aqmp
     return AQMP_OK;
 }
 
-// Basis tables of every side a code uses, for the synthesis kernels.
-static int code_bases(Ctx *c, const aqmp_code *code, cudaStream_t st, DecodeArgs *a) {
-    *a = DecodeArgs{};
-    a->nf = num_families(code->dict_id);
-    a->single_family = 0;
-    for (int b = code->min_block; b <= code->max_block; b *= 2) {
-        Dict *d;
-        int rc = get_dict(c, b, code->dict_id, st, &d, false);
-        if (rc) return rc;
-        a->basis[ilog2(b)] = d->d.basis;
+// The synthesis of planes[0 .. n) (images `img` of `pitch`) or, with `adjoint`,
+// its adjoint: one launch for each run of consecutive planes.
+static int synth_planes(Ctx *c, const aqmp_code *code, int n, const int *planes, float *const *img,
+                        const int64_t *pitch, const float *alpha, float *grad_alpha, cudaStream_t st) {
+    DecodeArgs fwd{};
+    AdjointArgs adj{};
+    int rc;
+    if ((rc = code_bases(c, code, st, &fwd.bases))) return rc;
+    fwd.leaves = adj.leaves = code->leaves;
+    fwd.n_leaves = adj.n_leaves = code->n_leaves;
+    fwd.atoms = adj.atoms = code->atoms;
+    fwd.alpha = alpha;
+    adj.bases = fwd.bases;
+    adj.grad_alpha = grad_alpha;
+    PlaneImages &im = grad_alpha ? adj.grad : fwd.out;
+    for (int i = 0; i < n;) {
+        im.plane = (uint32_t)planes[i];
+        im.n_planes = 0;
+        do {
+            im.img[im.n_planes] = img[i];
+            im.pitch[im.n_planes++] = pitch[i];
+            ++i;
+        } while (i < n && im.n_planes < kRefinePlanes && planes[i] == planes[i - 1] + 1);
+        CK(g_prof.run(kname(grad_alpha ? "synth_bwd" : "synth_fwd", code->max_block), st, [&] {
+            return grad_alpha ? launch_synth_backward(adj, c->num_sms, st) : launch_decode(fwd, c->num_sms, st);
+        }));
     }
     return AQMP_OK;
 }
@@ -1391,14 +1415,7 @@ int aqmp_synth_forward(const aqmp_code *code, int plane, const float *alpha, flo
     int rc;
     if ((rc = get_ctx(&c))) return rc;
     std::lock_guard<std::mutex> lock(c->mu);
-    cudaStream_t st = (cudaStream_t)stream;
-    DecodeArgs bases;
-    if ((rc = code_bases(c, code, st, &bases))) return rc;
-    CK(g_prof.run(kname("synth_fwd", code->max_block), st, [&] {
-        return launch_synth_forward(code->leaves, code->n_leaves, code->atoms, alpha, (uint32_t)plane, out,
-                                    out_pitch, bases, c->num_sms, st);
-    }));
-    return AQMP_OK;
+    return synth_planes(c, code, 1, &plane, &out, &out_pitch, alpha, nullptr, (cudaStream_t)stream);
 }
 
 int aqmp_synth_backward(const aqmp_code *code, int plane, const float *grad_out, int64_t pitch, float *grad_alpha,
@@ -1411,14 +1428,34 @@ int aqmp_synth_backward(const aqmp_code *code, int plane, const float *grad_out,
     int rc;
     if ((rc = get_ctx(&c))) return rc;
     std::lock_guard<std::mutex> lock(c->mu);
-    cudaStream_t st = (cudaStream_t)stream;
-    DecodeArgs bases;
-    if ((rc = code_bases(c, code, st, &bases))) return rc;
-    CK(g_prof.run(kname("synth_bwd", code->max_block), st, [&] {
-        return launch_synth_backward(code->leaves, code->n_leaves, code->atoms, (uint32_t)plane, grad_out, pitch,
-                                     grad_alpha, bases, code->max_block, c->num_sms, st);
-    }));
-    return AQMP_OK;
+    float *img = const_cast<float *>(grad_out);                  // read only by the adjoint
+    return synth_planes(c, code, 1, &plane, &img, &pitch, nullptr, grad_alpha, (cudaStream_t)stream);
+}
+
+// Bytes of the per-window partials of one h x w image.
+static size_t ssim_partial_bytes(int h, int w) {
+    return ((sizeof(float4) + sizeof(float2)) * (size_t)(h - 10) * (w - 10) + 255) & ~(size_t)255;
+}
+
+static void ssim_plane(SsimPlane &p, const float *x, int64_t x_pitch, const float *y, int64_t y_pitch, int h, int w,
+                       double *sum, float *grad, int64_t grad_pitch, double grad_scale, void *partials) {
+    p = SsimPlane{};
+    p.x = x;
+    p.x_pitch = x_pitch;
+    p.y = y;
+    p.y_pitch = y_pitch;
+    p.h = h;
+    p.w = w;
+    p.sum = sum;
+    if (!grad) return;
+    const size_t wins = (size_t)(h - 10) * (w - 10);
+    const double scale = grad_scale / (double)wins;
+    p.grad = grad;
+    p.grad_pitch = grad_pitch;
+    p.scale.hi = (float)scale;
+    p.scale.lo = (float)(scale - (double)p.scale.hi);
+    p.P4 = (float4 *)partials;
+    p.P2 = (float2 *)(p.P4 + wins);
 }
 
 int aqmp_ssim(const float *x, const float *y, int h, int w, int64_t pitch, double *ssim, float *grad_y,
@@ -1430,17 +1467,99 @@ int aqmp_ssim(const float *x, const float *y, int h, int w, int64_t pitch, doubl
     if ((rc = get_ctx(&c))) return rc;
     std::lock_guard<std::mutex> lock(c->mu);
     cudaStream_t st = (cudaStream_t)stream;
-    if (!c->gauss_ready) {
-        CK(upload_gauss11(st));
-        c->gauss_ready = true;
-    }
-    const size_t hw = (size_t)h * (w - 10), win = (size_t)(h - 10) * (w - 10);
-    if ((rc = c->ssim_ws.reserve(sizeof(double) * (5 * hw + 3 * win + 3 * hw)))) return rc;
-    double *H = (double *)c->ssim_ws.p, *P = H + 5 * hw, *V = P + 3 * win;
+    if (grad_y && (rc = c->ssim_ws.reserve(ssim_partial_bytes(h, w)))) return rc;
+    SsimArgs a{};
+    a.n = 1;
+    ssim_plane(a.p[0], x, pitch, y, pitch, h, w, ssim, grad_y, pitch, grad_scale, c->ssim_ws.p);
     CK(cudaMemsetAsync(ssim, 0, sizeof(double), st));
     CK(g_prof.run(grad_y ? "ssim_fwd_bwd" : "ssim_fwd", st,
-                  [&] { return launch_ssim(x, y, h, w, pitch, H, P, V, ssim, grad_y, grad_scale, c->num_sms, st); }));
+                  [&] { return launch_ssim(a, grad_y != nullptr, c->num_sms, st); }));
     return AQMP_OK;
+}
+
+static int check_refine(const aqmp_code *code, const aqmp_refine_plane *planes, int n) {
+    if (!code || !planes || n <= 0) return fail(AQMP_E_ARG, "bad argument");
+    for (int i = 0; i < n; ++i) {
+        const aqmp_refine_plane &p = planes[i];
+        if (p.plane < 0 || p.plane >= (int)code->shapes.size()) return fail(AQMP_E_ARG, "plane %d: no such plane", i);
+        if (p.height < 11 || p.width < 11) return fail(AQMP_E_ARG, "plane %d: smaller than the SSIM window", i);
+    }
+    return AQMP_OK;
+}
+
+int aqmp_refine_workspace(const aqmp_refine_plane *planes, int n, uint64_t *bytes) {
+    g_last_error.clear();
+    if (!planes || n <= 0 || !bytes) return fail(AQMP_E_ARG, "bad argument");
+    *bytes = 0;
+    for (int i = 0; i < n; ++i) {
+        if (planes[i].height < 11 || planes[i].width < 11) return fail(AQMP_E_ARG, "plane %d: smaller than the SSIM window", i);
+        *bytes += ssim_partial_bytes(planes[i].height, planes[i].width);
+    }
+    return AQMP_OK;
+}
+
+int aqmp_refine_forward(const aqmp_code *code, const float *alpha, const aqmp_refine_plane *planes, int n,
+                        double *ssim, int want_grad, void *workspace, void *stream) {
+    g_last_error.clear();
+    int rc = check_refine(code, planes, n);
+    if (rc) return rc;
+    if (!alpha || !ssim || (want_grad && (!workspace || ((uintptr_t)workspace & 15)))) return fail(AQMP_E_ARG, "bad argument");
+    std::vector<int> id(n);
+    std::vector<float *> recon(n);
+    std::vector<int64_t> pitch(n);
+    for (int i = 0; i < n; ++i) {
+        const aqmp_refine_plane &p = planes[i];
+        const int w = code->shapes[p.plane].second;
+        if (p.height < code->shapes[p.plane].first) return fail(AQMP_E_ARG, "plane %d: fewer rows than the plane", i);
+        if (!p.ref || !p.recon || (want_grad && !p.grad)) return fail(AQMP_E_ARG, "plane %d: NULL image", i);
+        if (p.ref_pitch < p.width || p.recon_pitch < std::max(w, p.width) || (want_grad && p.grad_pitch < p.width))
+            return fail(AQMP_E_ARG, "plane %d: pitch below width", i);
+        id[i] = p.plane;
+        recon[i] = p.recon;
+        pitch[i] = p.recon_pitch;
+    }
+    Ctx *c;
+    if ((rc = get_ctx(&c))) return rc;
+    std::lock_guard<std::mutex> lock(c->mu);
+    cudaStream_t st = (cudaStream_t)stream;
+    if ((rc = synth_planes(c, code, n, id.data(), recon.data(), pitch.data(), alpha, nullptr, st))) return rc;
+    CK(cudaMemsetAsync(ssim, 0, sizeof(double) * n, st));
+    unsigned char *ws = (unsigned char *)workspace;
+    for (int i0 = 0; i0 < n; i0 += kRefinePlanes) {
+        SsimArgs a{};
+        a.n = std::min(n - i0, kRefinePlanes);
+        for (int i = 0; i < a.n; ++i) {
+            const aqmp_refine_plane &p = planes[i0 + i];
+            ssim_plane(a.p[i], p.ref, p.ref_pitch, p.recon, p.recon_pitch, p.height, p.width, ssim + i0 + i,
+                       want_grad ? p.grad : nullptr, p.grad_pitch, 1.0, ws);
+            if (want_grad) ws += ssim_partial_bytes(p.height, p.width);
+        }
+        CK(g_prof.run(want_grad ? "ssim_fwd_bwd" : "ssim_fwd", st,
+                      [&] { return launch_ssim(a, want_grad != 0, c->num_sms, st); }));
+    }
+    return AQMP_OK;
+}
+
+int aqmp_refine_backward(const aqmp_code *code, const aqmp_refine_plane *planes, int n, float *grad_alpha,
+                         void *stream) {
+    g_last_error.clear();
+    int rc = check_refine(code, planes, n);
+    if (rc) return rc;
+    if (!grad_alpha) return fail(AQMP_E_ARG, "bad argument");
+    std::vector<int> id(n);
+    std::vector<float *> grad(n);
+    std::vector<int64_t> pitch(n);
+    for (int i = 0; i < n; ++i) {
+        if (!planes[i].grad || planes[i].grad_pitch < code->shapes[planes[i].plane].second)
+            return fail(AQMP_E_ARG, "plane %d: bad gradient image", i);
+        id[i] = planes[i].plane;
+        grad[i] = planes[i].grad;
+        pitch[i] = planes[i].grad_pitch;
+    }
+    Ctx *c;
+    if ((rc = get_ctx(&c))) return rc;
+    std::lock_guard<std::mutex> lock(c->mu);
+    return synth_planes(c, code, n, id.data(), grad.data(), pitch.data(), nullptr, grad_alpha, (cudaStream_t)stream);
 }
 
 int aqmp_selftest_wait(int limit_ms, void *stream) {

@@ -166,32 +166,66 @@ cudaError_t launch_corr_tc_fp8(const CorrArgs &a, const float *inv_sl, cudaStrea
 bool corr_tc_available();
 cudaError_t launch_wait_selftest(Counters *ctr, unsigned long long limit_ns, cudaStream_t st);
 
-// Decoder (decode.cu): one plane's leaves -> float image.
+// The planes [plane, plane + n_planes) of a code and one image for each, as
+// the decoder and the synthesis adjoint take them in one launch.
+constexpr int kRefinePlanes = 32;
+struct PlaneImages {
+    uint32_t plane;
+    int n_planes;                        // 1 .. kRefinePlanes
+    float *img[kRefinePlanes];
+    long long pitch[kRefinePlanes];      // elements per row
+};
+
+// FP32 1-D bases of the sides a code uses.
+struct Bases {
+    const float *basis[8];       // per level log2(b): [2][b][b] FP32 bases (NULL: no leaf of that side)
+    int nf;                      // 2: DCT+Haar, 1: single family
+    int single_family;           // its slot in `basis` (when nf == 1)
+};
+
+// Decoder (decode.cu): the planes' leaves -> float images; alpha, if not NULL,
+// holds caller coefficients in place of the code's.
 struct DecodeArgs {
     const LeafRec *leaves;
     unsigned long long n_leaves;
     const AtomRec *atoms;
-    uint32_t plane;
-    float *out;
-    long long out_pitch;
-    const float *basis[8];       // per level log2(b): [2][b][b] FP32 bases
-    int nf;                      // 2: DCT+Haar, 1: single family
-    int single_family;           // 0: DCT, 1: Haar (when nf == 1)
+    const float *alpha;
+    Bases bases;
+    PlaneImages out;
 };
 cudaError_t launch_decode(const DecodeArgs &a, int num_sms, cudaStream_t st);
-// The same with caller coefficients alpha[atom] in place of the code's.
-cudaError_t launch_decode_alpha(const DecodeArgs &a, const float *alpha, int num_sms, cudaStream_t st);
 
-// Refinement on a fixed support (diff.cu).
-cudaError_t upload_gauss11(cudaStream_t st);
-cudaError_t launch_synth_forward(const LeafRec *leaves, unsigned long long n_leaves, const AtomRec *atoms,
-                                 const float *alpha, uint32_t plane, float *out, long long pitch,
-                                 const DecodeArgs &bases, int num_sms, cudaStream_t st);
-cudaError_t launch_synth_backward(const LeafRec *leaves, unsigned long long n_leaves, const AtomRec *atoms,
-                                  uint32_t plane, const float *grad, long long pitch, float *grad_alpha,
-                                  const DecodeArgs &bases, int max_side, int num_sms, cudaStream_t st);
-cudaError_t launch_ssim(const float *x, const float *y, int h, int w, long long pitch, double *H, double *P,
-                        double *V, double *sum, float *grad, double gscale, int num_sms, cudaStream_t st);
+// Adjoint of the synthesis (diff.cu): grad_alpha of the planes' atoms from the
+// gradient images in `grad`.
+struct AdjointArgs {
+    const LeafRec *leaves;
+    unsigned long long n_leaves;
+    const AtomRec *atoms;
+    float *grad_alpha;
+    Bases bases;
+    PlaneImages grad;
+};
+cudaError_t launch_synth_backward(const AdjointArgs &a, int num_sms, cudaStream_t st);
+
+// Mean SSIM and its gradient (ssim.cu) of up to kRefinePlanes images.
+struct SsimPlane {
+    const float *x, *y;
+    float *grad;
+    long long x_pitch, y_pitch, grad_pitch;
+    int h, w;
+    df scale;                    // of the gradient
+    float4 *P4;                  // [(h-10)(w-10)] per-window partials f_my, f_Eyy (high words, low words)
+    float2 *P2;                  // [(h-10)(w-10)] f_Exy
+    double *sum;
+    unsigned tile0, tiles_x;     // filled by the launch
+};
+struct SsimArgs {
+    SsimPlane p[kRefinePlanes];
+    int n;
+    df c1, c2;                                       // filled by the launch, as are the window's
+    unsigned long long gh[11], ngh[11], gl[11];      // weights: high word, its negative, low word, twice each
+};
+cudaError_t launch_ssim(SsimArgs &a, bool grad, int num_sms, cudaStream_t st);
 
 // Level-0 queue from the plane descriptors (gather.cu).
 cudaError_t launch_seed_roots(const PlaneDesc *planes, int n_planes, int max_block,

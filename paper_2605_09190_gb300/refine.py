@@ -24,31 +24,32 @@ class SynthesisSSIM(torch.autograd.Function):
     def forward(ctx, alpha, code, refs):
         # When alpha needs a gradient, the SSIM kernels return d SSIM / d y
         # in the same pass (the window statistics are computed once); the
-        # backward only scales it and runs the synthesis adjoint.
+        # backward only scales it and runs the synthesis adjoint.  All planes
+        # go through one launch of each kernel.
         want = ctx.needs_input_grad[0]
-        grads, vals = [], []
-        for plane, ref in refs:
-            out = torch.empty_like(ref)
-            aqmp.aqmp_synth_forward(code, plane, alpha, out)
-            s = torch.zeros((), dtype=torch.float64, device=ref.device)
-            if want:
-                gy = torch.empty_like(out)
-                aqmp.aqmp_ssim(ref, out, s, gy, 1.0)
-                grads.append(gy)
-            else:
-                aqmp.aqmp_ssim(ref, out, s)
-            vals.append(s)
-        ctx.code, ctx.refs, ctx.grads = code, refs, grads
+        dev = alpha.device
+        at = [0]
+        for _, ref in refs:
+            at.append(at[-1] + ref.shape[0] * ref.shape[1])
+        recon = torch.empty(at[-1], dtype=torch.float32, device=dev)
+        grad = torch.empty_like(recon) if want else None
+        y0, g0 = recon.data_ptr(), grad.data_ptr() if want else None
+        planes = aqmp.aqmp_refine_planes([
+            (plane, ref.shape[0], ref.shape[1], ref.data_ptr(), ref.stride(0), y0 + 4 * o, ref.shape[1],
+             g0 + 4 * o if want else None, ref.shape[1]) for (plane, ref), o in zip(refs, at)])
+        ssim = torch.empty(len(refs), dtype=torch.float64, device=dev)
+        work = torch.empty(aqmp.aqmp_refine_workspace(planes), dtype=torch.uint8, device=dev) if want else None
+        aqmp.aqmp_refine_forward(code, alpha, planes, ssim, work)
+        ctx.code, ctx.planes, ctx.images = code, planes, grad
         ctx.n_alpha = alpha.shape[0]
-        return torch.stack(vals).mean()
+        return ssim.mean()
 
     @staticmethod
     def backward(ctx, grad):
         grad_alpha = torch.zeros(ctx.n_alpha, dtype=torch.float32, device=grad.device)
-        for (plane, _), gy in zip(ctx.refs, ctx.grads):
-            aqmp.aqmp_synth_backward(ctx.code, plane, gy, grad_alpha)
+        aqmp.aqmp_refine_backward(ctx.code, ctx.planes, grad_alpha)
         # the mean over planes and the upstream gradient, on the device
-        return grad_alpha * (grad / len(ctx.refs)).to(torch.float32), None, None
+        return grad_alpha * (grad / len(ctx.planes)).to(torch.float32), None, None
 
 
 def synthesis_ssim(alpha, code, refs):
