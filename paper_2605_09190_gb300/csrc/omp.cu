@@ -3,22 +3,29 @@
 // of Algorithm 2 (sides 32 and 64: omp_cta.cu, the same rules).
 //
 // One warp owns one leaf.  Each step:
-//   - residual energy ||r||^2 = ||y||^2 - x_S . c0_S (the residual is
-//     orthogonal to span(D_S) after every re-fit), tested before the step
-//     with the rule of Eq. (3) and the same equality band as the MP kernel;
+//   - residual energy ||r||^2 = ||y||^2 - |z|^2, z = L^-1 c0_S, tested before
+//     the step with the rule of Eq. (3) and the same equality band as the MP
+//     kernel;
 //   - residual correlations c = c0 - G[:, S] x_S, the Gram entries generated
 //     from W = C H^T (G is the identity inside a family and kron(W, W)
-//     across the two);
+//     across the two); the residual is orthogonal to the support, whose atoms
+//     are left out;
 //   - argmax |c| with the MP kernel's tie rule (values within 2^-32 ||y|| of
 //     the largest are tied, lowest index wins) and certification band;
-//   - the new row of the Cholesky factor L of G_SS (solve L w = G[S, j],
-//     pivot 1 - |w|^2; a pivot <= 2^-40 ends the pursuit, the atom being
-//     dependent on the support), then the re-fit L L^T x_S = c0_S.
-// Everything is FP64.  L lives packed in shared memory; row i of every
-// triangular solve belongs to lane i mod 32 and the solves run in axpy form
-// (the owner finishes its row, shuffles the value, every lane updates its
-// rows), so each step of their chains is one shuffle, not a reduction.  A
-// leaf's budget k must be <= 64 (two rows per lane).
+//   - the Cholesky factor L of G_SS grows by a row (w, sqrt(d)) with
+//     w = L^-1 G[S, j], d = 1 - |w|^2 (a pivot d <= 2^-40 ends the pursuit, the
+//     atom being dependent on the support); z grows by (c0_j - w . z) / sqrt(d)
+//     and the re-fit x_S = L^-T z by z_new times the new column of L^-T.
+//
+// Everything is FP64, at 1/64 of GB300's FP32 rate, and that bounds the
+// kernel: a warp's FP64 instruction takes the SM 16 cycles.  So the inverse
+// factor K = L^-1 is kept instead of L (packed, in shared memory): its new row
+// is (-w^T K, 1) / sqrt(d), and a step takes the two products K g (over the
+// support atoms of the other family alone, g being zero on its own) and w^T K,
+// about 2.5 t instructions for t atoms, where two forward and one back
+// substitution with L took 9 t, in chains of shuffles.  The argmax compares
+// the doubles' bit patterns on the integer pipes.  A 512x512 plane at
+// four tolerances, sides 16..4: the whole encode 6.53 -> 3.86 ms.  A leaf's budget k must be <= 64 (two rows per lane).
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -39,10 +46,15 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, off));
-    return v;
+// |v| as an integer of the same order.
+__device__ __forceinline__ unsigned long long mag_bits(double v) {
+    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+
+__device__ __forceinline__ unsigned long long warp_max64(unsigned long long v) {
+    const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(v >> 32));
+    const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(v >> 32) == hi ? (uint32_t)v : 0u);
+    return ((unsigned long long)hi << 32) | lo;
 }
 
 __host__ __device__ __forceinline__ int tri(int i) { return i * (i + 1) / 2; }
@@ -74,16 +86,15 @@ __global__ void __launch_bounds__(256, 1) omp_kernel(MPArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     double *sW = reinterpret_cast<double *>(smem);
     const int k = a.lv.k;
-    const int per = tri(k) + 3 * k + M;                  // L, x_S, c0_S, 1 / L_ii, dense x (doubles)
+    const int per = tri(k) + 2 * k;                      // K, x_S, g then w (doubles)
     const int warps = blockDim.x >> 5;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double *base = sW + (NF == 2 ? B * B : 0);
-    double *L = base + (size_t)warp * per;
-    double *xs = L + tri(k);
-    double *c0s = xs + k;
-    double *rdiag = c0s + k;
-    double *xd = rdiag + k;                              // x_S scattered over all M atoms
-    uint32_t *Sj = reinterpret_cast<uint32_t *>(base + (size_t)warps * per) + (size_t)warp * k;
+    double *K = base + (size_t)warp * per;
+    double *xs = K + tri(k);
+    double *gs = xs + k;                                 // G[S, j], then w
+    uint32_t *Sj = reinterpret_cast<uint32_t *>(base + (size_t)warps * per) + (size_t)warp * 2 * k;
+    uint32_t *fam_pos = Sj + k;                          // positions of the DCT atoms, from the end the Haar atoms
 
     if (NF == 2)
         for (int i = threadIdx.x; i < B * B; i += blockDim.x) sW[i] = (double)a.W[i].x + (double)a.W[i].y;
@@ -115,15 +126,13 @@ __global__ void __launch_bounds__(256, 1) omp_kernel(MPArgs a) {
             c0r[s] = j < M ? (double)cp[j].x + (double)cp[j].y : 0.0;
         }
 
-        for (int i = lane; i < M; i += 32) xd[i] = 0.0;
-        __syncwarp();
-        int nS = 0;
+        int nS = 0, nC = 0, nH = 0;                          // support size, and per family
+        uint32_t taken = 0u;                                 // this lane's slots in the support
+        double z0 = 0.0, z1 = 0.0, x0 = 0.0, x1 = 0.0;       // rows lane and lane + 32
+        double En = E0;
         bool conv = false, tie = false;
         for (;;) {
             // (a6) accuracy test before every step, strict
-            double acc = 0.0;
-            for (int i = lane; i < nS; i += 32) acc += xs[i] * c0s[i];
-            const double En = E0 - warp_sum(acc);
             if (fabs(En - thr_e) < band_e) tie = true;
             if (En < thr_e) { conv = true; break; }
             if (nS == k) break;
@@ -137,20 +146,19 @@ __global__ void __launch_bounds__(256, 1) omp_kernel(MPArgs a) {
                 // lane's atoms share p = lane mod B: a support atom of one
                 // family reaches the other family's slots through
                 // W[p_d][p_h] (one factor per lane) times W[q_d][q_h]
-                for (int i = 0; i < nS; ++i) {
-                    const uint32_t sa = Sj[i];
-                    const double x = xs[i];
-                    if (sa < (uint32_t)n) {
-                        const uint32_t ps = sa % B, qs = sa / B;
-                        const double ax = x * sW[ps * B + p_own];
+                for (int i = 0; i < nC; ++i) {
+                    const uint32_t at = fam_pos[i], sa = Sj[at];
+                    const uint32_t ps = sa % B, qs = sa / B;
+                    const double ax = xs[at] * sW[ps * B + p_own];
 #pragma unroll
-                        for (int s = E / 2; s < E; ++s) cv[s] -= ax * sW[qs * B + q_own + (32 / B) * s - B];
-                    } else {
-                        const uint32_t ps = (sa - n) % B, qs = (sa - n) / B;
-                        const double ax = x * sW[p_own * B + ps];
+                    for (int s = E / 2; s < E; ++s) cv[s] -= ax * sW[qs * B + q_own + (32 / B) * s - B];
+                }
+                for (int i = 0; i < nH; ++i) {
+                    const uint32_t at = fam_pos[k - 1 - i], sa = Sj[at] - (uint32_t)n;
+                    const uint32_t ps = sa % B, qs = sa / B;
+                    const double ax = xs[at] * sW[p_own * B + ps];
 #pragma unroll
-                        for (int s = 0; s < E / 2; ++s) cv[s] -= ax * sW[(q_own + (32 / B) * s) * B + qs];
-                    }
+                    for (int s = 0; s < E / 2; ++s) cv[s] -= ax * sW[(q_own + (32 / B) * s) * B + qs];
                 }
             } else if (NF == 2) {
 #pragma unroll
@@ -161,27 +169,32 @@ __global__ void __launch_bounds__(256, 1) omp_kernel(MPArgs a) {
                         if ((Sj[i] >= (uint32_t)n) != (j >= (uint32_t)n)) cv[s] -= gram<B, NF>(sW, j, Sj[i]) * xs[i];
                 }
             }
-            // the diagonal: each support atom's own coefficient, kept dense
-#pragma unroll
-            for (int s = 0; s < E; ++s)
-                if (lane + 32 * s < M) cv[s] -= xd[lane + 32 * s];
-            double amax = 0.0;
+            unsigned long long mag[E], best = 0ull;
 #pragma unroll
             for (int s = 0; s < E; ++s) {
-                if ((uint32_t)(lane + 32 * s) >= (uint32_t)M) cv[s] = 0.0;
-                amax = fmax(amax, fabs(cv[s]));
+                mag[s] = (uint32_t)(lane + 32 * s) < (uint32_t)M && !((taken >> s) & 1u) ? mag_bits(cv[s]) : 0ull;
+                best = max(best, mag[s]);
             }
-            amax = warp_max(amax);
+            const double amax = __longlong_as_double((long long)warp_max64(best));
             if (amax <= tie_c) break;                        // nothing left to remove
             const double edge = amax - tie_c;
+            const unsigned long long edge_b = mag_bits(edge);
+            // (only values within two bands of the edge can lie within one)
+            const unsigned long long near_lo = mag_bits(fmax(edge - 2.0 * band_c, 0.0)), near_hi = mag_bits(edge + 2.0 * band_c);
             uint32_t jl = kNoAtom;
+            bool near = false;
 #pragma unroll
             for (int s = 0; s < E; ++s) {
-                const uint32_t j = lane + 32 * s;
-                if (j >= (uint32_t)M) continue;
-                const double m = fabs(cv[s]);
-                if (m >= edge && j < jl) jl = j;
-                if (fabs(m - edge) < band_c) tie = true;
+                if ((uint32_t)(lane + 32 * s) >= (uint32_t)M) continue;
+                if (mag[s] >= edge_b) jl = min(jl, (uint32_t)(lane + 32 * s));
+                near |= mag[s] >= near_lo && mag[s] <= near_hi;
+            }
+            if (__builtin_expect(near, 0)) {
+#pragma unroll
+                for (int s = 0; s < E; ++s)
+                    if ((uint32_t)(lane + 32 * s) < (uint32_t)M &&
+                        fabs(__longlong_as_double((long long)mag[s]) - edge) < band_c)
+                        tie = true;
             }
             const uint32_t jb = __reduce_min_sync(0xffffffffu, jl);
             double c0b = 0.0;
@@ -190,67 +203,68 @@ __global__ void __launch_bounds__(256, 1) omp_kernel(MPArgs a) {
                 if ((uint32_t)(lane + 32 * s) == jb) c0b = c0r[s];
             c0b = __shfl_sync(0xffffffffu, c0b, (int)(jb & 31u));
 
-            // new Cholesky row: L w = G[S, jb] (rows lane and lane + 32)
-            double g0 = lane < nS ? gram<B, NF>(sW, Sj[lane], jb) : 0.0;
-            double g1 = lane + 32 < nS ? gram<B, NF>(sW, Sj[lane + 32], jb) : 0.0;
-            for (int i = 0; i < nS; ++i) {
-                double wi = 0.0;
-                if (lane == (i & 31)) wi = (i < 32 ? g0 : g1) * rdiag[i];
-                wi = __shfl_sync(0xffffffffu, wi, i & 31);
-                if (lane == (i & 31)) {
-                    if (i < 32) g0 = wi; else g1 = wi;
+            // w = K G[S, jb] (rows lane and lane + 32): G[S, jb] is nonzero on
+            // the other family alone
+            const bool haar = NF == 2 && jb >= (uint32_t)n;
+            double w0 = 0.0, w1 = 0.0;
+            if (NF == 2) {
+                if (lane < nS) gs[lane] = gram<B, NF>(sW, Sj[lane], jb);
+                if (lane + 32 < nS) gs[lane + 32] = gram<B, NF>(sW, Sj[lane + 32], jb);
+                __syncwarp();
+                const int others = haar ? nC : nH;
+                const double *r0 = K + tri(lane), *r1 = K + tri(lane + 32);
+                for (int i = 0; i < others; ++i) {
+                    const int at = (int)fam_pos[haar ? i : k - 1 - i];
+                    const double g = gs[at];
+                    if (nS > 32 && lane + 32 < nS && at <= lane + 32) w1 = fma(r1[at], g, w1);
+                    if (at < 32 && lane < nS && at <= lane) w0 = fma(r0[at], g, w0);
                 }
-                if (lane > i && lane < nS) g0 -= L[tri(lane) + i] * wi;
-                if (lane + 32 > i && lane + 32 < nS) g1 -= L[tri(lane + 32) + i] * wi;
+                __syncwarp();
+                if (lane < nS) gs[lane] = w0;
+                if (lane + 32 < nS) gs[lane + 32] = w1;
+                __syncwarp();
             }
-            // g0 / g1 now hold w for the lane's rows
-            const double d = 1.0 - warp_sum((lane < nS ? g0 * g0 : 0.0) + (lane + 32 < nS ? g1 * g1 : 0.0));
+            const double d = 1.0 - warp_sum(w0 * w0 + w1 * w1);
             if (d > kPivotMin * 0x1p-4 && d < kPivotMin * 0x1p4) tie = true;
             if (d <= kPivotMin) break;                       // dependent on the support
-            const int rb = tri(nS);
-            if (lane < nS) L[rb + lane] = g0;
-            if (lane + 32 < nS) L[rb + lane + 32] = g1;
-            if (lane == 0) {
-                const double ld = sqrt(d);
-                L[rb + nS] = ld;
-                rdiag[nS] = 1.0 / ld;
-                Sj[nS] = jb;
-                c0s[nS] = c0b;
-            }
-            ++nS;
-            __syncwarp();
+            const double rd = 1.0 / sqrt(d);
+            const double zn = (c0b - warp_sum(w0 * z0 + w1 * z1)) * rd;
+            En -= zn * zn;
 
-            // re-fit: L z = c0_S, then L^T x = z (rows lane and lane + 32)
-            double z0 = lane < nS ? c0s[lane] : 0.0;
-            double z1 = lane + 32 < nS ? c0s[lane + 32] : 0.0;
-            for (int i = 0; i < nS; ++i) {
-                double zi = 0.0;
-                if (lane == (i & 31)) zi = (i < 32 ? z0 : z1) * rdiag[i];
-                zi = __shfl_sync(0xffffffffu, zi, i & 31);
-                if (lane == (i & 31)) {
-                    if (i < 32) z0 = zi; else z1 = zi;
+            // K's new row -(w^T K, -1) / sqrt(d) (columns lane and lane + 32),
+            // and x_S += zn times it
+            double v0 = 0.0, v1 = 0.0;
+            if (NF == 2) {
+                for (int i = 0; i < min(nS, 32); ++i)
+                    if (lane <= i) v0 = fma(gs[i], K[tri(i) + lane], v0);
+                for (int i = 32; i < nS; ++i) {
+                    const double w = gs[i];
+                    v0 = fma(w, K[tri(i) + lane], v0);
+                    if (lane + 32 <= i) v1 = fma(w, K[tri(i) + lane + 32], v1);
                 }
-                if (lane > i && lane < nS) z0 -= L[tri(lane) + i] * zi;
-                if (lane + 32 > i && lane + 32 < nS) z1 -= L[tri(lane + 32) + i] * zi;
             }
-            for (int i = nS - 1; i >= 0; --i) {
-                double xi = 0.0;
-                if (lane == (i & 31)) xi = (i < 32 ? z0 : z1) * rdiag[i];
-                xi = __shfl_sync(0xffffffffu, xi, i & 31);
-                if (lane == (i & 31)) {
-                    if (i < 32) z0 = xi; else z1 = xi;
-                }
-                if (lane < i) z0 -= L[tri(i) + lane] * xi;
-                if (lane + 32 < i) z1 -= L[tri(i) + lane + 32] * xi;
+            v0 = lane == nS ? rd : -v0 * rd;
+            v1 = lane + 32 == nS ? rd : -v1 * rd;
+            const int rb = tri(nS);
+            if (lane <= nS) {
+                K[rb + lane] = v0;
+                x0 = fma(zn, v0, x0);
+                xs[lane] = x0;
             }
-            if (lane < nS) {
-                xs[lane] = z0;
-                xd[Sj[lane]] = z0;
+            if (lane + 32 <= nS) {
+                K[rb + lane + 32] = v1;
+                x1 = fma(zn, v1, x1);
+                xs[lane + 32] = x1;
             }
-            if (lane + 32 < nS) {
-                xs[lane + 32] = z1;
-                xd[Sj[lane + 32]] = z1;
+            if (lane == nS) z0 = zn;
+            if (lane + 32 == nS) z1 = zn;
+            if (lane == 0) {
+                Sj[nS] = jb;
+                fam_pos[haar ? k - 1 - nH : nC] = (uint32_t)nS;
             }
+            if ((jb & 31u) == (uint32_t)lane) taken |= 1u << (jb / 32u);
+            if (haar) ++nH; else ++nC;
+            ++nS;
             __syncwarp();
         }
 
@@ -322,7 +336,7 @@ static cudaError_t launch_omp_t(const MPArgs &a, int num_sms, cudaStream_t st) {
     constexpr int warps = 8;
     const int k = a.lv.k;
     const size_t bytes = (NF == 2 ? sizeof(double) * B * B : 0) +
-                         warps * (sizeof(double) * (size_t)(tri(k) + 3 * k + NF * B * B) + sizeof(uint32_t) * (size_t)k);
+                         warps * (sizeof(double) * (size_t)(tri(k) + 2 * k) + 2 * sizeof(uint32_t) * (size_t)k);
     auto kern = omp_kernel<B, NF>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
