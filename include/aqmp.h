@@ -104,9 +104,11 @@ extern "C" {
                                       budget per leaf of at most 64 atoms at
                                       sides 4..16 and 1024 at sides 32 and 64
                                       (else AQMP_E_UNSUPPORTED).  Sides 32 and
-                                      64 keep a Cholesky factor of up to
-                                      k(k+1)/2 doubles per SM in device
-                                      memory (4.2 MB at k = 1024). */
+                                      64 keep the inverse Cholesky factor of
+                                      each leaf in flight (at most one per SM)
+                                      in device memory, by rows and by columns:
+                                      k(k+1)/2 + k^2 doubles (12.6 MB at
+                                      k = 1024). */
 /* Autotuning: kernel choices that leave the result unchanged bit for bit
  * are measured on the first calls of each configuration and the fastest
  * is kept for the life of the process: the initial correlation on the

@@ -870,14 +870,14 @@ int aqmp_encode_planes(const aqmp_params *params, const aqmp_plane *planes, int 
     CK(cudaMallocFromPoolAsync((void **)&code->alpha_lo, sizeof(float) * std::max<unsigned long long>(1, atom_cap),
                                c->out_pool, st));
     if ((rc = c->counters.reserve(sizeof(Counters)))) return rc;
-    // OMP at sides 32 and 64: a packed Cholesky factor per resident CTA
+    // OMP at sides 32 and 64: the inverse factor of each leaf in flight
     unsigned long long omp_doubles = 0;
     if (omp)
         for (int l = 0; l < nlev; ++l) {
             const int b = P.max_block >> l;
             if (b < 32) continue;
             const int kb = (int)std::max<long long>(1, (long long)b * b * P.cap_num / P.cap_den);
-            omp_doubles = std::max(omp_doubles, omp_cta_workspace_doubles(kb, c->num_sms));
+            omp_doubles = std::max(omp_doubles, omp_cta_workspace_doubles(kb, c->num_sms, cap[l]));
         }
     if (omp_doubles && (rc = c->omp_L.reserve(sizeof(double) * omp_doubles))) return rc;
 

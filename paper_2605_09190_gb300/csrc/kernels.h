@@ -25,8 +25,9 @@ struct MPArgs {
     unsigned long long atom_cap;
     CellMap cells;               // emitted leaves are marked here
     Counters *ctr;
-    // OMP at sides 32 and 64: one packed Cholesky factor of up to k(k+1)/2
-    // doubles per CTA, omp_slots of them (omp_L_doubles in all)
+    // OMP at sides 32 and 64: the inverse factor of a leaf in flight, by rows
+    // (packed) and by columns; omp_slots is the device's SMs, the most leaves
+    // in flight (omp_L_doubles in all, see omp_cta_workspace_doubles)
     double *omp_L;
     int omp_slots;
     unsigned long long omp_L_doubles;
@@ -57,12 +58,12 @@ bool mp_has_variant(int b, int nf);
 cudaError_t launch_mp_cluster(const MPArgs &a, int nf, bool double_float, int num_sms, cudaStream_t st);
 
 // Orthogonal Matching Pursuit of one level: sides 4, 8, 16 with a warp per
-// leaf (omp.cu), sides 32 and 64 with a CTA per leaf and the Cholesky factor
-// in the omp_L slots (omp_cta.cu); budget k <= omp_max_budget(b) (0: side not
+// leaf (omp.cu), sides 32 and 64 with one to eight CTAs per leaf and the inverse
+// factor in the omp_L slots (omp_cta.cu); budget k <= omp_max_budget(b) (0: side not
 // served); same arguments and outputs as the MP kernel (the coefficients
 // emitted are the final least-squares values).
 int omp_max_budget(int b);
-unsigned long long omp_cta_workspace_doubles(int k, int slots);
+unsigned long long omp_cta_workspace_doubles(int k, int sms, unsigned long long leaves);
 cudaError_t launch_omp(const MPArgs &a, int nf, int num_sms, cudaStream_t st);
 int omp_cta_max_budget();
 cudaError_t launch_omp_cta(const MPArgs &a, int nf, cudaStream_t st);
