@@ -21,7 +21,6 @@
 
 #include "common.cuh"
 #include "kernels.h"
-#include "haar_rows.cuh"
 #include "sep.cuh"
 
 namespace aqmp {
@@ -55,9 +54,8 @@ template <int B>
 constexpr int sep_threads() { return B >= 128 ? 768 : 256; }
 
 // Shared-memory layout of one CTA (G leaves): the centred pixels, their
-// even and odd column halves, and the Z~ region, which the Haar pass reuses
-// for its summed-area table.  A Haar-only launch (HO) keeps the pixels and
-// the table alone.
+// even and odd column halves, and the Z~ region, which the Haar pass reuses.
+// A Haar-only launch (HO) keeps that pass's arrays alone.
 template <int B, bool HO = false>
 struct SepSmem {
     static constexpr int n = B * B, H = B / 2, G = sep_group<B>();
@@ -65,27 +63,54 @@ struct SepSmem {
     static constexpr int YS = B + 4;                           // row stride of the pixels (bytes): the
                                                                // transposing stores hit distinct banks
     static constexpr size_t yt = 0;                            // int8  [G][i][YS]
-    static constexpr size_t ys = (G * B * YS + 15) & ~15;      // int16 [G][parity][i < H][m]
+    static constexpr size_t ys = HO ? 0 : (G * B * YS + 15) & ~15;      // int16 [G][parity][i < H][m]
     static constexpr size_t z = ys + (HO ? 0 : ((2 * G * n + 15) & ~15));   // Limbs2 [G][p][RS] / int [G][RS][RS]
-    static constexpr size_t zbytes = HO ? ((sizeof(int) * G * RS * RS + 15) & ~15) : sizeof(Limbs2) * G * B * RS;
+    // the Haar pass: K [G][p][RS] (int), the first transform [G][p][DS] (int16), sums of 16 values [c][G * B] (int)
+    static constexpr int CH = B < 16 ? B : 16, C = B / CH, DS = B + 2;
+    static constexpr size_t d1 = sizeof(int) * G * B * RS, part = d1 + ((sizeof(int16_t) * G * B * DS + 15) & ~15),
+                            hbytes = part + (C > 1 ? sizeof(int) * C * G * B : 0);
+    static constexpr size_t zbytes = HO ? ((hbytes + 15) & ~15) : sizeof(Limbs2) * G * B * RS;
     static constexpr int E = 1 + ilog2(B);                     // Haar scale classes: row 0, scales 1 .. b/2
-    static constexpr size_t hrow = z + zbytes;                 // int4 [B]: s, h, class, sign
-    static constexpr size_t ptab = hrow + sizeof(int4) * B;    // ulonglong2 [E][E]: fL(c1) fL(c2), int128
-    static constexpr size_t bytes = ptab + sizeof(ulonglong2) * E * E;
-    static_assert(sizeof(int) * RS * RS <= sizeof(Limbs2) * B * RS, "table fits the Z~ region");
+    static constexpr size_t ptab = z + zbytes;                 // int4 [E][E]: the limbs of -fL(c1) fL(c2)
+    static constexpr size_t bytes = ptab + sizeof(int4) * E * E;
+    static_assert(hbytes <= sizeof(Limbs2) * G * B * RS, "the Haar pass fits the Z~ region");
 };
 
 __device__ __forceinline__ long long bf_value(int2 w) { return (long long)w.y * (1ll << 24) + w.x; }
 
-// P K for 0 <= P < 2^96 (as 64-bit halves lo, hi < 2^32) and |K| < 2^31:
-// three 32 x 32 -> 64-bit products joined in int128.
-__device__ __forceinline__ __int128 mul_u96_i32(const ulonglong2 &P, int K) {
-    const unsigned k = (unsigned)(K < 0 ? -K : K);
-    const unsigned long long a0 = (unsigned long long)(unsigned)P.x * k;
-    const unsigned long long a1 = (unsigned long long)(unsigned)(P.x >> 32) * k;
-    const unsigned long long a2 = (unsigned long long)(unsigned)P.y * k;
-    const unsigned __int128 m = (unsigned __int128)a0 + ((unsigned __int128)a1 << 32) + ((unsigned __int128)a2 << 64);
-    return K < 0 ? -(__int128)m : (__int128)m;
+// The Haar class of a row: 0 for row 0, 1 + log2 of the scale's first row.
+__device__ __forceinline__ int haar_class(int r) { return 32 - __clz(r); }
+
+// Unnormalised Haar transform (row 0 the sum, row r >= 1 the sum over its
+// first half minus that over its second) of CH values in v, in place of a
+// part of a longer row: put(level row offset, value) for all but the sum,
+// which is returned.  c is the part's number of C: the rows of scale s that
+// lie in the part are B / s + c CH / s + t.
+template <int B, int CH, typename V, typename Put>
+__device__ __forceinline__ V haar_part(V (&v)[CH], int c, Put put) {
+#pragma unroll
+    for (int s = 2; s <= CH; s *= 2) {
+#pragma unroll
+        for (int t = 0; t < CH / s; ++t) {
+            const V x = v[2 * t], y = v[2 * t + 1];
+            put(B / s + c * (CH / s) + t, x - y);
+            v[t] = x + y;
+        }
+    }
+    return v[0];
+}
+
+// Row r < C of the transform from the C parts' sums at s[0], s[stride], ...
+template <int C>
+__device__ __forceinline__ int haar_join(const int *s, int stride, int r) {
+    const int len = r == 0 ? C : C >> (31 - __clz(r));           // parts under the row
+    const int at = r == 0 ? 0 : (r - (1 << (31 - __clz(r)))) * len;
+    int sum = 0;
+    for (int i = 0; i < len; ++i) {
+        const int x = s[(at + i) * stride];
+        sum += r != 0 && 2 * i >= len ? -x : x;
+    }
+    return sum;
 }
 
 // One CTA handles G leaves at a time (grid-stride over the leaves).
@@ -98,13 +123,17 @@ __device__ __forceinline__ __int128 mul_u96_i32(const ulonglong2 &P, int K) {
 // exact integers.  |Z~+-| < 2^60, so zh < 2^28 and every limb sum over
 // b/2 <= 64 terms stays below 2^61.
 //
-// Haar family: row p of Bf is constant on each of two dyadic halves
-// (haar_halves), fL on the first and s_p fL on the second (s_p = +1 for row
-// 0, -1 otherwise), and fL depends only on the row's scale.  So T~[p][q] =
-// fL(p) fL(q) K with K = LL + s_q LR + s_p RL + s_p s_q RR, the sums of y~
-// over the four half-by-half rectangles, read from the summed-area table of
-// y~ (|entries| <= 2^21, |K| <= 2^21); the products fL(c1) fL(c2) of the
-// 1 + log2 b scale classes are formed once per CTA in int128.
+// Haar family: row p of Bf is +fL on its first half and -fL on its second
+// (row 0: fL throughout), and fL depends only on the row's scale.  So
+// T~[p][q] = fL(p) fL(q) K[p][q] with K the integer 2-D Haar transform of y~
+// (|K| <= 2^21): one pass of sums and differences along i, one along m, two
+// additions per value each, in parts of 16 per thread.  The products
+// fL(c1) fL(c2) of the 1 + log2 b scale classes are formed once per CTA and
+// kept negated in three signed 32-bit limbs (2^95 fits with that sign), so
+// T + the rounding's bias is a chain of three 32-bit multiply-adds.  The
+// integer work of an output is now the smaller part of it beside the rounding.
+// Side 64, 50 910 leaves, this family alone: HAAR_FIGURES (a summed-area table,
+// nine reads and an int128 product per output, before).
 template <int B, bool HO>
 __global__ void __launch_bounds__(sep_threads<B>())
 corr_sep_simt_kernel(int nf, int fam0, int fmask, int Kpad, const int2 *__restrict__ Bs, const int2 *__restrict__ BsT,
@@ -119,44 +148,40 @@ corr_sep_simt_kernel(int nf, int fam0, int fmask, int Kpad, const int2 *__restri
     int8_t *yt = reinterpret_cast<int8_t *>(smem + L::yt);
     int16_t *ys = reinterpret_cast<int16_t *>(smem + L::ys);
     Limbs2 *Z = reinterpret_cast<Limbs2 *>(smem + L::z);
-    int *S = reinterpret_cast<int *>(smem + L::z);
 
-    constexpr int nt = sep_threads<B>(), nw = nt / 32, E = L::E;
-    int4 *hrow = reinterpret_cast<int4 *>(smem + L::hrow);
-    ulonglong2 *ptab = reinterpret_cast<ulonglong2 *>(smem + L::ptab);
+    constexpr int nt = sep_threads<B>(), E = L::E;
+    int4 *ptab = reinterpret_cast<int4 *>(smem + L::ptab);
 
     const long long count = count_dev ? (long long)*count_dev : fixed_count;
     const int M = nf * n;
     const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
     if ((nf == 2 || fam0 == 1) && ((fmask >> 1) & 1)) {
-        // the Haar rows' supports and classes, and the class products
+        // the class products
         const int2 *Bh = Bs + (size_t)n;
-        for (int r = tid; r < B; r += nt) {
-            int sr, hr;
-            haar_halves(r, B, sr, hr);
-            const int cls = r == 0 ? 0 : 1 + (31 - __clz(B / (2 * hr)));
-            hrow[r] = make_int4(sr, hr, cls, r == 0 ? 1 : -1);
-        }
         for (int e = tid; e < E * E; e += nt) {
             const int c1 = e / E, c2 = e - c1 * E;
             const int r1 = c1 == 0 ? 0 : 1 << (c1 - 1), r2 = c2 == 0 ? 0 : 1 << (c2 - 1);   // first row of the class
-            const unsigned __int128 P = (unsigned __int128)((__int128)bf_value(Bh[r1 * B]) * bf_value(Bh[r2 * B]));
-            ptab[e] = make_ulonglong2((unsigned long long)P, (unsigned long long)(P >> 64));
+            const __int128 P = -(__int128)bf_value(Bh[r1 * B]) * bf_value(Bh[r2 * B]);
+            const int32_t l0 = (int32_t)(uint32_t)(unsigned __int128)P;
+            const long long P1 = (long long)((P - l0) >> 32);
+            const int32_t l1 = (int32_t)(uint32_t)(unsigned long long)P1;
+            ptab[e] = make_int4(l0, l1, (int32_t)((P1 - l1) >> 32), 0);
         }
         __syncthreads();
     }
     for (long long base = (long long)blockIdx.x * G; base < count; base += (long long)gridDim.x * G) {
         const int live = (int)min((long long)G, count - base);
-        // centred pixels, transposed so that the contractions read consecutive m
-        for (int o = tid; o < G * n; o += nt) {
-            const int g = o / n, v = o - g * n;
-            const int m = v / B, i = v - m * B;
-            int8_t y = 0;
-            if (g < live) y = (int8_t)__bfloat162float(Y[(base + g) * Kpad + v]);
-            yt[(g * B + i) * YS + m] = y;
+        if constexpr (!HO) {
+            // centred pixels, transposed so that the contractions read consecutive m
+            for (int o = tid; o < G * n; o += nt) {
+                const int g = o / n, v = o - g * n;
+                const int m = v / B, i = v - m * B;
+                int8_t y = 0;
+                if (g < live) y = (int8_t)__bfloat162float(Y[(base + g) * Kpad + v]);
+                yt[(g * B + i) * YS + m] = y;
+            }
+            __syncthreads();
         }
-        __syncthreads();
         for (int f = 0; f < nf; ++f) {
             const int F = nf == 2 ? f : fam0;
             if (!((fmask >> F) & 1)) continue;                   // uniform
@@ -234,65 +259,82 @@ corr_sep_simt_kernel(int nf, int fam0, int fmask, int Kpad, const int2 *__restri
                 }
                 }
             } else {
-                // summed-area table S[i][m] = sum of y~ over [0, i) x [0, m):
-                // prefix sums along m (one warp per row), then along i (one
-                // warp per column; stride RS = 1 mod 32 keeps it conflict-free)
-                for (int o = tid; o < G * RS; o += nt) {
-                    const int g = o / RS, e = o - g * RS;
-                    S[g * RS * RS + e] = 0;                            // row 0
-                    S[g * RS * RS + e * RS] = 0;                       // column 0
-                }
-                for (int row = warp; row < G * B; row += nw) {
-                    const int g = row / B, i = row - g * B;
-                    int carry = 0;
-                    for (int c = 0; c < B; c += 32) {
-                        int v = c + lane < B ? (int)yt[(g * B + i) * YS + c + lane] : 0;
-#pragma unroll
-                        for (int d = 1; d < 32; d <<= 1) {
-                            const int u = __shfl_up_sync(0xffffffffu, v, d);
-                            if (lane >= d) v += u;
-                        }
-                        if (c + lane < B) S[g * RS * RS + (i + 1) * RS + c + lane + 1] = carry + v;
-                        carry += __shfl_sync(0xffffffffu, v, 31);
-                    }
-                }
-                __syncthreads();
-                for (int col = warp; col < G * B; col += nw) {
-                    const int g = col / B, m = col - g * B + 1;
-                    int carry = 0;
-                    for (int c = 0; c < B; c += 32) {
-                        int *at = S + g * RS * RS + (c + lane + 1) * RS + m;
-                        int v = c + lane < B ? *at : 0;
-#pragma unroll
-                        for (int d = 1; d < 32; d <<= 1) {
-                            const int u = __shfl_up_sync(0xffffffffu, v, d);
-                            if (lane >= d) v += u;
-                        }
-                        if (c + lane < B) *at = carry + v;
-                        carry += __shfl_sync(0xffffffffu, v, 31);
-                    }
-                }
-                __syncthreads();
-                // T~[g][p][q], p lane-fastest
-                for (int o = tid; o < G * n; o += nt) {
-                    const int g = o / n, r = o - g * n;
-                    const int q = r / B, p = r - q * B;
-                    const int4 hp = hrow[p], hq = hrow[q];
-                    const int *Sg = S + g * RS * RS;
-                    const int *r0 = Sg + hp.x * RS, *r1 = r0 + hp.y * RS, *r2 = r1 + hp.y * RS;
-                    const int m0 = hq.x, m1 = hq.x + hq.y, m2 = hq.x + 2 * hq.y;
-                    const int s00 = r0[m0], s01 = r0[m1], s02 = r0[m2];
-                    const int s10 = r1[m0], s11 = r1[m1], s12 = r1[m2];
-                    const int s20 = r2[m0], s21 = r2[m1], s22 = r2[m2];
-                    const int LL = s11 - s01 - s10 + s00, LR = s12 - s02 - s11 + s01;
-                    const int RL = s21 - s11 - s20 + s10, RR = s22 - s12 - s21 + s11;
-                    const int K = (LL + hq.w * LR) + hp.w * (RL + hq.w * RR);
-                    __int128 T = mul_u96_i32(ptab[hp.z * E + hq.z], K);
-                    // rows r >= 1 sum to zero (halves of equal length and
-                    // opposite values), so only (0, 0) has a centring term
-                    if ((p | q) == 0) T += (__int128)(128ll * R[0]) * R[0];
+                constexpr int CH = L::CH, C = L::C, DS = L::DS, rows = G * B;
+                int *K = reinterpret_cast<int *>(smem + L::z);                       // [G][p][RS]
+                int16_t *D1 = reinterpret_cast<int16_t *>(smem + L::z + L::d1);      // [G][p][DS]
+                int *part = reinterpret_cast<int *>(smem + L::z + L::part);
+                // along i, straight from the gathered pixels (y~ at m b + i), in
+                // exact floats: lanes take consecutive m
+                for (int o = tid; o < rows * C; o += nt) {
+                    const int row = o % rows, c = o / rows, g = row / B, m = row % B;
+                    uint32_t x[CH / 2] = {};
                     if (g < live) {
-                        const df c = int128_to_df(T);
+                        const __nv_bfloat16 *src = Y + (base + g) * Kpad + m * B + c * CH;
+                        if constexpr (CH == 4) {
+                            const uint2 u = *reinterpret_cast<const uint2 *>(src);
+                            x[0] = u.x, x[1] = u.y;
+                        } else {
+#pragma unroll
+                            for (int w = 0; w < CH / 8; ++w) {
+                                const uint4 u = reinterpret_cast<const uint4 *>(src)[w];
+                                x[4 * w] = u.x, x[4 * w + 1] = u.y, x[4 * w + 2] = u.z, x[4 * w + 3] = u.w;
+                            }
+                        }
+                    }
+                    float v[CH];
+#pragma unroll
+                    for (int w = 0; w < CH / 2; ++w) {
+                        v[2 * w] = __uint_as_float(x[w] << 16);
+                        v[2 * w + 1] = __uint_as_float(x[w] & 0xffff0000u);
+                    }
+                    int16_t *dst = D1 + g * B * DS + m;
+                    auto as_int = [](float f) { return __float_as_int(__fadd_rn(f, 12582912.0f)); };   // + 0x4B400000
+                    const float sum = haar_part<B, CH>(v, c, [&](int p, float f) { dst[p * DS] = (int16_t)as_int(f); });
+                    if (C > 1) part[c * rows + row] = as_int(sum) - 0x4B400000;
+                    else dst[0] = (int16_t)as_int(sum);
+                }
+                if (C > 1) {
+                    __syncthreads();
+                    for (int o = tid; o < rows * C; o += nt) {
+                        const int row = o % rows, r = o / rows;
+                        D1[((row / B) * B + r) * DS + row % B] = (int16_t)haar_join<C>(part + row, rows, r);
+                    }
+                }
+                __syncthreads();
+                // along m: lanes take consecutive p
+                for (int o = tid; o < rows * C; o += nt) {
+                    const int row = o % rows, c = o / rows;
+                    const int32_t *src = reinterpret_cast<const int32_t *>(D1 + row * DS + c * CH);
+                    int *dst = K + row * RS;
+                    int v[CH];
+#pragma unroll
+                    for (int w = 0; w < CH / 2; ++w) {
+                        const int x = src[w];
+                        v[2 * w] = (int)(int16_t)x;
+                        v[2 * w + 1] = x >> 16;
+                    }
+                    const int sum = haar_part<B, CH>(v, c, [&](int q, int x) { dst[q] = x; });
+                    if (C > 1) part[c * rows + row] = sum;
+                    else dst[0] = sum;
+                }
+                __syncthreads();
+                if (C > 1) {
+                    for (int o = tid; o < rows * C; o += nt)
+                        K[(o % rows) * RS + o / rows] = haar_join<C>(part + o % rows, rows, o / rows);
+                    __syncthreads();
+                }
+                // T[g][p][q], p lane-fastest and the same in every turn of a thread
+                const int p = tid % B, cp = haar_class(p) * E;
+                for (int o = tid; o < G * n; o += nt) {
+                    const int q = o / B % B, g = o / n;
+                    int k = -K[(g * B + p) * RS + q];
+                    if ((p | q) == 0) k -= 128 * n;             // centring: rows r >= 1 sum to zero, R[0] = b fL(0)
+                    const int4 l = ptab[cp + haar_class(q)];
+                    const long long x0 = mul_wide(l.x, k) + (long long)kDigitBiasLo;
+                    const long long x1 = mul_wide(l.y, k) + (x0 >> 32);
+                    const long long x2 = mul_wide(l.z, k) + (long long)kDigitBiasHi + (x1 >> 32);
+                    if (g < live) {
+                        const df c = biased_to_df((uint32_t)x0, (uint32_t)x1, (uint32_t)x2, (uint32_t)(x2 >> 32));
                         out[(base + g) * M + q * B + p] = make_float2(c.hi, c.lo);
                     }
                 }
