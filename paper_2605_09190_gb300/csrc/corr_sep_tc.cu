@@ -3,34 +3,46 @@
 // per family as the SIMT twin (corr_sep.cu), rounded the same way, so both
 // give identical bits.
 //
+// A CTA takes two leaves at a time: 128 rows of a tile are (leaf, row), and
+// every value ends in the lane and the thread that uses it.
+//
 // Digits.  Bf = sum_{s<6} d_s 2^(8s) with balanced digits |d_s| <= 128 (the
 // top one <= 181), all exact BF16 values, as are the centred pixels.
-//   Stage 1 (per leaf and family): Z~^T[m][p] = sum_i y~[i][m] Bf[p][i].
-//     A = [d_2u rows p ; d_2u+1 rows p] (128 rows, K = i) from shared memory,
-//     B = the leaf's pixels (rows m, K = i), one FP32 accumulator per digit
-//     pair u: lane (s parity, p), column m.  |d y~| sums over 64 terms stay
-//     below 2^24: exact.
-//   Z~ (|Z~| < 2^59) is assembled exactly in int64 from the six digit sums
-//   (the two parities meet through shared memory) and split into eight
-//   balanced base-2^8 digits e_t, written into tensor memory as the A operand
-//   of stage 2: tile v holds [e_2v rows p ; e_2v+1 rows p] (K = m).
-//   Stage 2: T~[p][q] = sum_{t,s} 2^(8(t+s)) sum_m e_t[p][m] d_s[q][m].
-//     A = tile v (tensor memory), B = d_s rows q (shared memory, 32 q per
-//     pass), accumulated into column block 2v + s: lane half h of block c
-//     then holds the digit diagonal t + s = c + h, the sum of at most three
-//     digit products (one per tile v with 0 <= c - 2v < 6), each below
-//     128 x 181 x 64 < 2^20.5 in magnitude: below 2^22, exact.
-//   The epilogue reads each diagonal (an exact FP32 integer), joins
-//   adjacent diagonals in one 32-bit multiply-add and those pairs in int64
-//   groups, then in int128 (the base-2^8 Horner scheme), the two lane
-//   halves meet through shared memory, and T = T~ + 128 R[p] R[q] is
-//   rounded once into a double-float (int128_to_df).
+//   Fold (DCT-II).  Row q of Bf equals (-1)^q times its mirror image, so row m
+//   of the pixels becomes y~[m] + y~[63-m] (m < 32) or y~[m] - y~[63-m]
+//   (m >= 32), in place: at most 256 in magnitude, exact BF16.  The even rows
+//   of Bf need the first 32 only, the odd ones the last 32: half of stage 2.
+//   Stage 1: Z~^T[m][p] = sum_i y~[i][m] Bf[p][i].  A = the pixels (rows
+//     (leaf, m), K = i), B = the digits (rows (parity of p, s, p / 2)): lane
+//     (leaf, m) holds the six digit sums of each p, each below 256 x 181 x 64
+//     < 2^22 in magnitude: exact.  They are joined in int64 with the centring
+//     term 128 R[p] of each pixel row (R[p] the row sums of Bf; a difference
+//     has none) and split into eight balanced base-2^8 digits e_t, written to
+//     shared memory as stage 2's A operand: rows (leaf, p), K = m, M-major, so
+//     that a lane's row m is a row of 64 p there.
+//   Stage 2: T[p][q] = sum_{t,s} 2^(8(t+s)) sum_m e_t[p][m] d_s[q][m], 32 q of
+//     one parity at a time.  B = the digits d_0 .. d_5 of those q stacked (192
+//     rows), so that one MMA with A = e_t adds into the columns of the digit
+//     diagonals t .. t + 5 (32 columns each): the sum of at most six digit
+//     products, each below 128 x 181 x 32: below 2^22, exact.  Without the fold
+//     (the Haar family) K = 64, and the bound holds since a Haar row of 64
+//     nonzero entries is a power of two, with one nonzero digit.
+//   The epilogue joins the 13 diagonals of an output: adjacent ones in one
+//   32-bit multiply-add on their biased bit patterns (no wrap), those as
+//   disjoint words of two 128-bit numbers, and biased_to_df rounds the sum
+//   plus one constant for all biases.
 //
-// One CTA per SM (16 warps, all 512 TMEM columns: A tiles 0..127, stage-1
-// accumulators 128..319, stage-2 accumulators 128..511), persistent over the
-// leaves; thread 0 issues the TMA loads and the MMAs, all threads drain.
-// Every wait is bounded by a timer; on expiry the kernel records
-// AQMP_E_TIMEOUT, frees its TMEM and returns.
+// What bounds it: the instructions of the epilogue and of the digit split
+// (about 105 an output and 35 a value of Z~), which therefore overlap the MMAs where they can:
+// a pass's outputs are rounded and stored while the next pass or the next
+// pair's stage 1 runs.  Side 64, DCT-II family, 50 910 leaves: 4.60 -> 1.51
+// ms (one leaf at a time with two digits in the 128 rows, halves that met
+// through shared memory and 24 accumulators an output, before).
+//
+// One CTA per SM (16 warps, all 512 TMEM columns: stage 1 in 0..383, stage 2
+// in 0..415), persistent over the pairs; thread 0 issues the TMA loads and the
+// MMAs, all threads drain.  Every wait is bounded by a timer; on expiry the
+// kernel records AQMP_E_TIMEOUT, frees its TMEM and returns.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
@@ -47,51 +59,90 @@ namespace septc {
 constexpr int kB = 64;                        // block side served here
 constexpr int kThreads = 512;                 // 16 warps: 4 per TMEM lane quarter
 constexpr int kTmemCols = 512;
-constexpr int kColA = 0;                      // stage-2 A tiles: 4 x 32 columns
-constexpr int kColD = 128;                    // accumulators
-constexpr int kTileBd = 128 * 128;            // bytes: 128 rows x 128 B (two digits of one family)
 constexpr int kTileY = 64 * 128;              // bytes: 64 rows (m) x 64 BF16 (i)
-constexpr int kOffBd = 0;                     // 6 tiles: (family, digit pair)
-constexpr int kOffY = kOffBd + 6 * kTileBd;   // 2 buffers
-constexpr int kOffX = kOffY + 2 * kTileY;     // exchange: 64 KB
-constexpr int kBytesX = 64 * 1024;
-constexpr int kOffBar = kOffX + kBytesX;      // barriers: Bd, Y[2], MMA
+constexpr int kTileE = 64 * 128;              // bytes: 64 rows (m) x 64 BF16 (p) of one leaf and digit
+constexpr int kDigitRows = 6 * 64;            // rows of one family: (parity, s, p / 2)
+constexpr int kOffD = 0;
+constexpr int kOffE = kOffD + kDigitRows * 128;          // [digit t][leaf]
+constexpr int kOffY = kOffE + 8 * 2 * kTileE;            // [buffer][leaf]
+constexpr int kOffCen = kOffY + 2 * 2 * kTileY;          // centring terms by p
+constexpr int kOffBar = kOffCen + 8 * kB;                // barriers: digits, Y[2], MMA
 constexpr int kOffMisc = kOffBar + 8 * 8;
 constexpr int kSmemBytes = kOffMisc + 16 + 1024;
 
-// Stage 1: M = 128, N = 64; stage 2: M = 128, N = 32; BF16 x BF16 -> F32.
-constexpr uint32_t kIdesc1 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(64 >> 3) << 17) |
-                             ((uint32_t)(128 >> 4) << 24);
-constexpr uint32_t kIdesc2 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(32 >> 3) << 17) |
-                             ((uint32_t)(128 >> 4) << 24);
+// M = 128, N columns; BF16 x BF16 -> F32; A K-major, or M-major in stage 2.
+constexpr uint32_t idesc(int n, bool a_m_major) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | (a_m_major ? 1u << 15 : 0u) | ((uint32_t)(n >> 3) << 17) |
+           ((uint32_t)(128 >> 4) << 24);
+}
+
+// M-major tile: rows k of 64 M values (128 bytes, 128-byte swizzle), groups of
+// 8 k 1024 bytes apart; the second 64 M values one leaf's tile further.
+__device__ __forceinline__ unsigned long long smem_desc_m_major(uint32_t addr) {
+    unsigned long long d = 0;
+    d |= (unsigned long long)((addr & 0x3ffffu) >> 4);
+    d |= (unsigned long long)(kTileE >> 4) << 16;
+    d |= (unsigned long long)(1024 >> 4) << 32;
+    d |= (unsigned long long)1 << 46;
+    d |= (unsigned long long)2 << 61;
+    return d;
+}
+
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
+}
+
+__device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// Two FP32 integers of magnitude below 2^22 as a 2^8 + b + kPairBias, without
+// wrapping; one as a + kOneBias.
+constexpr uint32_t kOneBias = 0x4B400000u, kPairBias = (uint32_t)(257ull * kOneBias);
+__device__ __forceinline__ uint32_t biased_one(uint32_t bits) {
+    return __float_as_uint(__fadd_rn(__uint_as_float(bits), 12582912.0f));
+}
+__device__ __forceinline__ uint32_t biased_pair(uint32_t a_bits, uint32_t b_bits) {
+    return biased_one(a_bits) * 256u + biased_one(b_bits);
+}
+
+// Byte t of two words' numbers, each minus 128, as two BF16: 128 + the low
+// seven bits, less 128 where the byte's top bit is set and 256 where not.
+__device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1, int byte) {
+    const uint32_t w = __byte_perm(w0, w1, (uint32_t)(byte | ((4 + byte) << 8)) * 0x11u);
+    const uint32_t x = (w & 0x007f007fu) | 0x43004300u, c = (~w & 0x00800080u) | 0xC300C300u;
+    uint32_t d;
+    asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(x), "r"(c));
+    return d;
+}
 
 }  // namespace septc
 
 // Y map: the gathered leaves viewed as [capacity * 64 rows][64] BF16 (row m of
-// leaf l at row 64 l + m, K = i); Bd map: [6 * 128 rows][64] BF16, tile (F, u)
-// at row 128 (3 F + u).
+// leaf l at row 64 l + m, K = i); digit map: [2 * 384 rows][64] BF16, the rows
+// of family F from 384 F.
 __global__ void __launch_bounds__(septc::kThreads, 1)
-corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmBd, int nf,
-                   int fam0, int fmask, const long long *__restrict__ Rs, const unsigned *count_dev,
-                   long long fixed_count, float2 *__restrict__ c0, Counters *ctr) {
+corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmD, int F, int M,
+                   int off, const long long *__restrict__ Rs, const unsigned *count_dev, long long fixed_count,
+                   float2 *__restrict__ c0, Counters *ctr) {
     using namespace septc;
-    constexpr int n = kB * kB;
     const long long count = count_dev ? (long long)*count_dev : fixed_count;
-    if ((long long)blockIdx.x >= count) return;                  // uniform
-    const int M = nf * n;
+    const long long pairs = (count + 1) / 2;
+    if ((long long)blockIdx.x >= pairs) return;                  // uniform
+    const bool fold = F == 0;
 
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     unsigned char *gbase = smem_raw + (base - raw);
-    const uint32_t sBd = base + kOffBd, sY = base + kOffY, sBar = base + kOffBar;
-    const uint32_t barBd = sBar, barY0 = sBar + 8, barY1 = sBar + 16, barMma = sBar + 24;
-    long long *X = reinterpret_cast<long long *>(gbase + kOffX);
+    const uint32_t sD = base + kOffD, sE = base + kOffE, sY = base + kOffY, sBar = base + kOffBar;
+    const uint32_t barD = sBar, barY0 = sBar + 8, barY1 = sBar + 16, barMma = sBar + 24;
+    unsigned long long *cen = reinterpret_cast<unsigned long long *>(gbase + kOffCen);
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(gbase + kOffMisc);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) {
-        mbar_init(barBd, 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        mbar_init(barD, 1);
         mbar_init(barY0, 1);
         mbar_init(barY1, 1);
         mbar_init(barMma, 1);
@@ -102,216 +153,198 @@ corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constan
                      ::"r"(smem_u32(tmem_holder)), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    // the centring of Z~'s rows: 128 R[p], twice that for a sum of two rows
+    if (tid < kB) cen[tid] = (unsigned long long)(Rs[F * kB + tid] * (fold ? 256 : 128));
     fence_before();
     __syncthreads();
     fence_after();
     const uint32_t tmem = *tmem_holder;
 
-    // the six digit tiles once, the first leaf's pixels
-    if (threadIdx.x == 0) {
-        mbar_expect_tx(barBd, 6 * kTileBd);
-        for (int t = 0; t < 6; ++t) tma_load_2d(sBd + t * kTileBd, &tmBd, barBd, 0, 128 * t);
-        mbar_expect_tx(barY0, kTileY);
-        tma_load_2d(sY, &tmY, barY0, 0, (int)(64 * blockIdx.x));
+    auto load_pair = [&](long long pair, int buf) {
+        const uint32_t bar = buf ? barY1 : barY0;
+        mbar_expect_tx(bar, 2 * kTileY);
+        for (int l = 0; l < 2; ++l)                              // a row past the end reads zeros
+            tma_load_2d(sY + (2 * buf + l) * kTileY, &tmY, bar, 0, (int)(64 * (2 * pair + l)));
+    };
+    // the digits once, the first pair's pixels
+    if (tid == 0) {
+        mbar_expect_tx(barD, kDigitRows * 128);
+        for (int t = 0; t < 3; ++t) tma_load_2d(sD + t * 128 * 128, &tmD, barD, 0, kDigitRows * F + 128 * t);
+        load_pair(blockIdx.x, 0);
     }
-    bool ok = __syncthreads_and(mbar_wait(barBd, 0)) != 0;
+    bool ok = __syncthreads_and(mbar_wait(barD, 0)) != 0;
 
     // TMEM lane quarter of this warp and the column group it drains
     const int quarter = warp & 3, cg = warp >> 2;
-    const int row = quarter * 32 + lane;                          // TMEM lane = tile row
+    const int row = quarter * 32 + lane, half = row >> 6, r64 = row & 63;      // (leaf, m) or (leaf, p)
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-    const int par = row >> 6, p = row & 63;
+    const bool difference = fold && (quarter & 1);                             // rows m >= 32
     uint32_t mma_phase = 0, y_phase[2] = {0u, 0u};
+    uint32_t T[8][4];                                                          // biased words, 8 q of a pass
+
+    // rounds and stores the outputs q = 2 (8 cg + j) + par of a pair
+    auto finish = [&](long long pair, int par) {
+        const long long leaf = 2 * pair + half;
+        if (leaf >= count) return;
+        float2 *out = c0 + leaf * M + off + (2 * 8 * cg + par) * kB + r64;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const df v = biased_to_df(T[j][0], T[j][1], T[j][2], T[j][3]);
+            out[2 * j * kB] = make_float2(v.hi, v.lo);
+        }
+    };
+
     int it = 0;
-    for (long long leaf = blockIdx.x; ok && leaf < count; leaf += gridDim.x, ++it) {
+    long long pending = -1;
+    for (long long pair = blockIdx.x; ok && pair < pairs; pair += gridDim.x, ++it) {
         const int buf = it & 1;
-        const uint32_t barY = buf ? barY1 : barY0;
-        ok = __syncthreads_and(mbar_wait(barY, y_phase[buf])) != 0;
+        ok = __syncthreads_and(mbar_wait(buf ? barY1 : barY0, y_phase[buf])) != 0;
         y_phase[buf] ^= 1u;
         if (!ok) break;
-        // prefetch the next leaf into the other buffer (its last reader
-        // finished with the previous iteration's barriers)
-        if (threadIdx.x == 0 && leaf + gridDim.x < count) {
-            const uint32_t nb = buf ? barY0 : barY1;
-            mbar_expect_tx(nb, kTileY);
-            tma_load_2d(sY + (buf ^ 1) * kTileY, &tmY, nb, 0, (int)(64 * (leaf + gridDim.x)));
+        // prefetch the next pair into the other buffer (its last reader, the
+        // previous pair's stage 1, has been waited for)
+        if (tid == 0 && pair + gridDim.x < pairs) load_pair(pair + gridDim.x, buf ^ 1);
+        if (fold) {
+            // rows m and 63 - m, one 16-byte chunk a thread (the swizzle places
+            // chunk j of row m at j ^ (m mod 8))
+            const int l = tid >> 8, m = (tid >> 3) & 31, j = tid & 7;
+            unsigned char *t = gbase + kOffY + (2 * buf + l) * kTileY;
+            uint4 *pa = reinterpret_cast<uint4 *>(t + m * 128 + ((j ^ (m & 7)) << 4));
+            uint4 *pb = reinterpret_cast<uint4 *>(t + (63 - m) * 128 + ((j ^ (7 - (m & 7))) << 4));
+            uint4 x = *pa, y = *pb;
+            auto both = [](uint32_t &u, uint32_t &v) {
+                uint32_t s, d;
+                asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(s) : "r"(u), "r"(v));
+                asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(v), "r"(u));
+                u = s;
+                v = d;
+            };
+            both(x.x, y.x);
+            both(x.y, y.y);
+            both(x.z, y.z);
+            both(x.w, y.w);
+            *pa = x;
+            *pb = y;
+            fence_async();
         }
-        const uint32_t yaddr = sY + buf * kTileY;
-        for (int f = 0; f < nf && ok; ++f) {
-            const int F = nf == 2 ? f : fam0;
-            if (!((fmask >> F) & 1)) continue;                   // uniform
-            // ---- stage 1: Z~^T[m][p], one accumulator per digit pair u
-            if (threadIdx.x == 0) {
-                fence_after();
-                for (int u = 0; u < 3; ++u) {
-                    const unsigned long long ad = smem_desc(sBd + (3 * F + u) * kTileBd);
-                    const unsigned long long bd = smem_desc(yaddr);
+        fence_before();
+        __syncthreads();
+        // ---- stage 1
+        if (tid == 0) {
+            fence_after();
+            const unsigned long long ad = smem_desc(sY + 2 * buf * kTileY), bd = smem_desc(sD);
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        mma_ss(tmem + kColD + 64 * u, ad + 2ull * kk, bd + 2ull * kk, kIdesc1, kk > 0 ? 1u : 0u);
+            for (int par = 0; par < 2; ++par)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+                    mma_ss(tmem + 192 * par, ad + 2ull * kk, bd + (unsigned long long)(par * 192 * 128 >> 4) + 2ull * kk,
+                           idesc(192, false), kk > 0 ? 1u : 0u);
+            mma_commit(barMma);
+        }
+        if (pending >= 0) finish(pending, 1);
+        ok = __syncthreads_and(mbar_wait(barMma, mma_phase)) != 0;
+        mma_phase ^= 1u;
+        if (!ok) break;
+        fence_after();
+        // ---- drain 1: p = 16 cg + 8 h + (0 .. 7), one chunk of each digit's row
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t a[2][6][4];
+#pragma unroll
+            for (int par = 0; par < 2; ++par)
+#pragma unroll
+                for (int sd = 0; sd < 6; ++sd) tmem_ld4(lane_base + 192 * par + 32 * sd + 8 * cg + 4 * h, a[par][sd]);
+            wait_ld();
+            uint32_t e[8][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                uint32_t lo[2], hi[2];
+#pragma unroll
+                for (int par = 0; par < 2; ++par) {
+                    // Z~ + 128 in every byte, the biases of the three pairs removed
+                    constexpr unsigned long long kC =
+                        0x8080808080808080ull - (unsigned long long)kPairBias * 0x100010001ull;
+                    const unsigned long long c = kC + (difference ? 0ull : cen[16 * cg + 8 * h + 2 * i + par]);
+                    const unsigned long long z =
+                        (unsigned long long)biased_pair(a[par][1][i], a[par][0][i]) +
+                        ((unsigned long long)biased_pair(a[par][3][i], a[par][2][i]) << 16) +
+                        ((unsigned long long)biased_pair(a[par][5][i], a[par][4][i]) << 32) + c;
+                    lo[par] = (uint32_t)z;
+                    hi[par] = (uint32_t)(z >> 32);
+                }
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    e[t][i] = digit_pair(lo[0], lo[1], t);
+                    e[4 + t][i] = digit_pair(hi[0], hi[1], t);
+                }
+            }
+            unsigned char *dst = gbase + kOffE + half * kTileE + r64 * 128 + (((2 * cg + h) ^ (r64 & 7)) << 4);
+#pragma unroll
+            for (int t = 0; t < 8; ++t)
+                *reinterpret_cast<uint4 *>(dst + t * 2 * kTileE) = make_uint4(e[t][0], e[t][1], e[t][2], e[t][3]);
+        }
+        fence_async();
+        fence_before();
+        __syncthreads();
+        // ---- stage 2, the q of one parity a pass
+#pragma unroll 1
+        for (int par = 0; par < 2 && ok; ++par) {
+            if (tid == 0) {
+                fence_after();
+                const int k0 = fold ? 2 * par : 0, k1 = fold ? k0 + 2 : 4;
+                for (int kk = k0; kk < k1; ++kk) {
+                    const uint32_t more = kk > k0 ? 1u : 0u;
+                    const unsigned long long ad = smem_desc_m_major(sE) + 128ull * kk;
+                    const unsigned long long bd = smem_desc(sD + par * 192 * 128) + 2ull * kk;
+                    constexpr unsigned long long kStepE = 2 * kTileE >> 4;
+                    // digits 0 and 6 meet every diagonal but the last first
+                    mma_ss(tmem, ad, bd, idesc(192, true), more);
+                    mma_ss(tmem + 192, ad + 6 * kStepE, bd, idesc(192, true), more);
+                    mma_ss(tmem + 224, ad + 7 * kStepE, bd, idesc(160, true), 1u);
+                    mma_ss(tmem + 384, ad + 7 * kStepE, bd + (5 * 32 * 128 >> 4), idesc(32, true), more);
+                    for (int t = 1; t < 6; ++t) mma_ss(tmem + 32 * t, ad + t * kStepE, bd, idesc(192, true), 1u);
                 }
                 mma_commit(barMma);
             }
+            if (par == 1) finish(pair, 0);
             ok = __syncthreads_and(mbar_wait(barMma, mma_phase)) != 0;
             mma_phase ^= 1u;
             if (!ok) break;
             fence_after();
-            // ---- drain 1: this thread's parity sum Z_par[p][m] for its 16 m
-            // (lane row = (parity, p), columns m = 16 cg + j); X is stored
-            // m-major so that the lanes of a warp (consecutive p) hit
-            // consecutive words
-            {
-                uint32_t r0[16], r1[16], r2[16];
-                const uint32_t col = kColD + 16 * cg;
-                tmem_ld16(lane_base + col, r0);
-                tmem_ld16(lane_base + col + 64, r1);
-                tmem_ld16(lane_base + col + 128, r2);
+            // ---- drain 2: q = 2 (8 cg + j) + par, 13 diagonals each
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t a[13][4];
+#pragma unroll
+                for (int c = 0; c < 13; ++c) tmem_ld4(lane_base + 32 * c + 8 * cg + 4 * h, a[c]);
                 wait_ld();
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const long long z = (long long)small_int(r0[j]) + (long long)small_int(r1[j]) * 65536ll +
-                                        (long long)small_int(r2[j]) * 4294967296ll;
-                    X[(par * 64 + 16 * cg + j) * 64 + p] = z;
+                for (int i = 0; i < 4; ++i) {
+                    typedef unsigned __int128 u128;
+                    constexpr u128 kPairs = (u128)kPairBias * ((((u128)1 << 48 | (u128)1 << 32) | ((u128)1 << 16 | 1)) |
+                                                               ((u128)1 << 80 | (u128)1 << 64));
+                    constexpr u128 kC = (((u128)kDigitBiasHi << 64) | kDigitBiasLo) - kPairs - ((u128)kOneBias << 96);
+                    const u128 even = (u128)biased_pair(a[1][i], a[0][i]) | (u128)biased_pair(a[5][i], a[4][i]) << 32 |
+                                      (u128)biased_pair(a[9][i], a[8][i]) << 64 | (u128)biased_one(a[12][i]) << 96;
+                    const u128 odd = (u128)biased_pair(a[3][i], a[2][i]) << 16 |
+                                     (u128)biased_pair(a[7][i], a[6][i]) << 48 |
+                                     (u128)biased_pair(a[11][i], a[10][i]) << 80;
+                    const u128 t = even + odd + kC;
+                    T[4 * h + i][0] = (uint32_t)t;
+                    T[4 * h + i][1] = (uint32_t)(t >> 32);
+                    T[4 * h + i][2] = (uint32_t)(t >> 64);
+                    T[4 * h + i][3] = (uint32_t)(t >> 96);
                 }
-            }
-            __syncthreads();
-            // both parities of Z~[p][m] -> eight balanced digits; this lane keeps
-            // the digits of its own parity (tile v = t / 2, lane half = t mod 2).
-            // With z' = Z~ + sum_{t<7} 128 2^(8t), digit t < 7 is byte t of z'
-            // minus 128 and digit 7 is z' >> 56: no carry chain between digits.
-            {
-                uint32_t packed[4][8];
-#pragma unroll
-                for (int j2 = 0; j2 < 8; ++j2) {
-                    int32_t dig[2][4];
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int m = 16 * cg + 2 * j2 + e;
-                        const long long zz = X[(0 * 64 + m) * 64 + p] + X[(1 * 64 + m) * 64 + p] * 256ll +
-                                             0x80808080808080ll;
-                        const uint32_t lo = (uint32_t)zz, hi = (uint32_t)((unsigned long long)zz >> 32);
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            const int t = 2 * v + par;
-                            int32_t d;
-                            if (t == 7) d = (int32_t)(zz >> 56);
-                            else if (t < 4) d = (int32_t)((lo >> (8 * t)) & 255u) - 128;
-                            else d = (int32_t)((hi >> (8 * (t - 4))) & 255u) - 128;
-                            dig[e][v] = d;
-                        }
-                    }
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) packed[v][j2] = bf16_bits(dig[0][v]) | (bf16_bits(dig[1][v]) << 16);
-                }
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    // 8 packed columns (16 values of m)
-                    asm volatile(
-                        "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                        ::"r"(lane_base + kColA + 32 * v + 8 * cg), "r"(packed[v][0]), "r"(packed[v][1]),
-                          "r"(packed[v][2]), "r"(packed[v][3]), "r"(packed[v][4]), "r"(packed[v][5]),
-                          "r"(packed[v][6]), "r"(packed[v][7])
-                        : "memory");
-                }
-                wait_st();
             }
             fence_before();
             __syncthreads();
-            // ---- stage 2, 32 values of q per pass
-            for (int c = 0; c < 2 && ok; ++c) {
-                if (threadIdx.x == 0) {
-                    fence_after();
-                    uint32_t written = 0u;
-                    for (int v = 0; v < 4; ++v)
-                        for (int s = 0; s < 6; ++s) {
-                            const int cb = 2 * v + s;
-                            const uint32_t btile = sBd + (3 * F + (s >> 1)) * kTileBd + (s & 1) * (64 * 128) +
-                                                   c * (32 * 128);
-                            const unsigned long long bd = smem_desc(btile);
-#pragma unroll
-                            for (int kk = 0; kk < 4; ++kk) {
-                                const uint32_t acc = ((written >> cb) & 1u) | (kk > 0 ? 1u : 0u);
-                                mma_ts(tmem + kColD + 32 * cb, tmem + kColA + 32 * v + 8 * kk, bd + 2ull * kk,
-                                       kIdesc2, acc);
-                            }
-                            written |= 1u << cb;
-                        }
-                    mma_commit(barMma);
-                }
-                // the row sums this lane's outputs need, fetched while the MMAs run
-                const long long rowsum_p = Rs[F * kB + p];
-                long long rowsum_q[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) rowsum_q[j] = Rs[F * kB + 32 * c + 8 * cg + 4 * par + j];
-                ok = __syncthreads_and(mbar_wait(barMma, mma_phase)) != 0;
-                mma_phase ^= 1u;
-                if (!ok) break;
-                fence_after();
-                // ---- drain 2: lane (half hh, p), 8 values of q; block cb holds the
-                // diagonal cb + hh.  Horner in base 2^8 over three groups of four
-                // blocks (each exact in an int64: |D| < 2^22), the groups joined
-                // in int128; then the lanes of the two halves add their sums.
-                const int hh = par;
-                long long grp[3][8];
-#pragma unroll
-                for (int g = 2; g >= 0; --g) {
-                    uint32_t r[4][8];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const uint32_t ta = lane_base + kColD + 32 * (4 * g + 3 - k) + 8 * cg;
-                        asm volatile(
-                            "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                            : "=r"(r[k][0]), "=r"(r[k][1]), "=r"(r[k][2]), "=r"(r[k][3]), "=r"(r[k][4]),
-                              "=r"(r[k][5]), "=r"(r[k][6]), "=r"(r[k][7])
-                            : "r"(ta));
-                    }
-                    wait_ld();
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        // r[k] holds block 4g + 3 - k: two adjacent diagonals meet in
-                        // one 32-bit multiply-add on their biased bit patterns (the
-                        // bias cancels modulo 2^32 and |pair| < 2^31), two pairs in
-                        // one 64-bit multiply-add
-                        const int32_t hi2 = pair8(r[0][j], r[1][j]);        // blocks 4g+3, 4g+2
-                        const int32_t lo2 = pair8(r[2][j], r[3][j]);        // blocks 4g+1, 4g
-                        grp[g][j] = (long long)hi2 * 65536ll + (long long)lo2;
-                    }
-                }
-                fence_before();
-                __syncthreads();                  // X is free (drain 1 done), D read
-                __int128 *XT = reinterpret_cast<__int128 *>(X);
-                // lanes of half hh finalise q = 8 cg + [4 hh, 4 hh + 4) of the pass;
-                // they hand over the other four (stored j-major: consecutive p,
-                // consecutive words)
-                __int128 mine[4];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const __int128 sum = ((__int128)grp[2][j] * ((__int128)1 << 64) +
-                                          (__int128)grp[1][j] * ((__int128)1 << 32) + (__int128)grp[0][j]) *
-                                         (hh ? (__int128)256 : (__int128)1);
-                    if ((j >> 2) != hh) XT[(size_t)((cg * 2 + hh) * 8 + j) * 64 + p] = sum;
-                    else mine[j & 3] = sum;
-                }
-                __syncthreads();
-                const long long rp128 = 128ll * rowsum_p;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if ((j >> 2) == hh) {
-                        const __int128 other = XT[(size_t)((cg * 2 + 1 - hh) * 8 + j) * 64 + p];
-                        const int q = 32 * c + 8 * cg + j;
-                        const __int128 T = mine[j & 3] + other + (__int128)rp128 * rowsum_q[j & 3];
-                        const df v = int128_to_df(T);
-                        c0[leaf * M + (nf == 2 ? f * n : 0) + q * kB + p] = make_float2(v.hi, v.lo);
-                    }
-                }
-                fence_before();
-                __syncthreads();
-            }
         }
+        pending = pair;
     }
+    if (ok && pending >= 0) finish(pending, 1);
     fence_before();
     __syncthreads();
-    if (threadIdx.x == 0 && !ok && ctr) raise_error(ctr, kDevErrTimeout, 12u);
+    if (tid == 0 && !ok && ctr) raise_error(ctr, kDevErrTimeout, 12u);
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
@@ -327,13 +360,20 @@ cudaError_t launch_corr_sep_tc(const CorrArgs &a, cudaStream_t st) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const unsigned grid = (unsigned)(rows < sms ? rows : sms);
+    const long long pairs = (rows + 1) / 2;
+    const unsigned grid = (unsigned)(pairs < sms ? pairs : sms);
     e = cudaFuncSetAttribute(corr_sep_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, septc::kSmemBytes);
     if (e != cudaSuccess) return e;
-    corr_sep_tc_kernel<<<grid, septc::kThreads, septc::kSmemBytes, st>>>(
-        *reinterpret_cast<const CUtensorMap *>(a.tmap_Ysep), *reinterpret_cast<const CUtensorMap *>(d.tmap_sepd),
-        d.nf, d.fam0, a.fmask ? a.fmask : 3, d.Rs, a.count, a.fixed_count, a.c0, a.ctr);
-    return cudaGetLastError();
+    const int n = septc::kB * septc::kB, fmask = a.fmask ? a.fmask : 3;
+    for (int f = 0; f < d.nf && e == cudaSuccess; ++f) {
+        const int F = d.nf == 2 ? f : d.fam0;
+        if (!((fmask >> F) & 1)) continue;
+        corr_sep_tc_kernel<<<grid, septc::kThreads, septc::kSmemBytes, st>>>(
+            *reinterpret_cast<const CUtensorMap *>(a.tmap_Ysep), *reinterpret_cast<const CUtensorMap *>(d.tmap_sepd), F,
+            d.nf * n, f * n, d.Rs, a.count, a.fixed_count, a.c0, a.ctr);
+        e = cudaGetLastError();
+    }
+    return e;
 }
 
 }  // namespace aqmp

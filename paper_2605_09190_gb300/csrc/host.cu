@@ -272,9 +272,8 @@ Profiler g_prof;
 std::string kname(const char *k, int b) { return std::string(k) + "_b" + std::to_string(b); }
 
 // The exact separable correlation on the tensor-core path: the DCT-II family
-// on the tensor cores, the Haar family on the SIMT pipes, where its rows' two
-// constant halves reduce it to a summed-area computation with no contraction
-// left to speed up.  Bit for bit the SIMT kernel's result for both families.
+// on the tensor cores, the Haar family on the SIMT pipes, where it is two
+// passes of sums and differences with no contraction left to speed up.  Bit for bit the SIMT kernel's result for both families.
 cudaError_t corr_sep_hybrid(const CorrArgs &ca, int b, cudaStream_t st) {
     const DictDev &d = *ca.d;
     const bool dct = d.nf == 2 || d.fam0 == 0, haar = d.nf == 2 || d.fam0 == 1;
@@ -507,9 +506,8 @@ int get_dict(Ctx *c, int b, int dict_id, cudaStream_t st, Dict **out, bool table
             CK(cudaMemcpyAsync(d.Bs, limbs.data(), sizeof(int32_t) * limbs.size(), cudaMemcpyHostToDevice, st));
             CK(cudaMemcpyAsync(d.Rs, rows.data(), sizeof(long long) * rows.size(), cudaMemcpyHostToDevice, st));
             if (corr_sep_tc_available(b, d.nf)) {
-                // balanced base-2^8 digits d_s of Bf (s = 0..5) as BF16, in six
-                // 128-row tiles (family F, digit pair u): row r of tile (F, u)
-                // is row r mod b of digit 2u + r / b
+                // balanced base-2^8 digits d_s of Bf (s = 0..5) as BF16, 6 b rows
+                // a family: row r of digit s at (r mod 2, s, r / 2)
                 std::vector<__nv_bfloat16> dg(6 * 2 * bb);
                 for (int F = 0; F < 2; ++F)
                     for (int r = 0; r < b; ++r)
@@ -518,8 +516,8 @@ int get_dict(Ctx *c, int b, int dict_id, cudaStream_t st, Dict **out, bool table
                             for (int sd = 0; sd < 6; ++sd) {
                                 long long dv = sd < 5 ? ((f + 128) & 255) - 128 : f;
                                 f = (f - dv) >> 8;
-                                const int u = sd >> 1, half = sd & 1;
-                                dg[((size_t)(3 * F + u) * 2 * b + half * b + r) * b + col] = __float2bfloat16((float)dv);
+                                const size_t at = (size_t)F * 6 * b + (r & 1) * 3 * b + sd * (b / 2) + (r >> 1);
+                                dg[at * b + col] = __float2bfloat16((float)dv);
                             }
                         }
                 if ((rc0 = Dn->sepd.reserve(sizeof(__nv_bfloat16) * dg.size()))) return rc0;
@@ -1104,7 +1102,13 @@ int aqmp_encode_planes(const aqmp_params *params, const aqmp_plane *planes, int 
             cf.count = &ctr->fb_count[l];
             cf.mu = nullptr;
             cf.ebound = nullptr;
-            CK(g_prof.run(kname("corr_fb", b), st, [&] { return launch_corr_sep_tc(cf, st); }));
+            CK(g_prof.run(kname("corr_fb", b), st, [&] {
+                CorrArgs cd = cf;
+                cd.fmask = 1;
+                const cudaError_t e1 = launch_corr_sep_tc(cd, st);
+                cd.fmask = 2;
+                return e1 != cudaSuccess ? e1 : launch_corr_sep_simt(cd, st);
+            }));
             MPArgs mf = ma;
             mf.lv.queue = (const QueueEntry *)c->fbq.p;
             mf.lv.count = &ctr->fb_count[l];

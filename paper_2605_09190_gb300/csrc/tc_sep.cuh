@@ -1,6 +1,5 @@
 // tc_sep.cuh -- the tcgen05 / TMA / mbarrier helpers of the separable
-// tensor-core correlation kernels (corr_sep_tc.cu, corr_sepbf_tc.cu), and the
-// exact conversions of FP32 digit sums into integers.
+// tensor-core correlation kernels (corr_sep_tc.cu, corr_sepbf_tc.cu).
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -103,41 +102,10 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         : "r"(taddr));
 }
 
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-        "%14, %15, %16};"
-        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-          "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-        : "memory");
-}
-
 __device__ __forceinline__ void wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// An FP32 value holding an integer of magnitude below 2^22, as an int32
-// (the integer lands in the low mantissa bits of x + 1.5 2^23).
-__device__ __forceinline__ int32_t small_int(uint32_t bits) {
-    return __float_as_int(__fadd_rn(__uint_as_float(bits), 12582912.0f)) - 0x4B400000;
-}
-
-// a 2^8 + b for two FP32 values holding integers of magnitude below 2^22:
-// their biased bit patterns (x + 1.5 2^23) combined in 32-bit arithmetic,
-// the bias removed once; exact as |a 2^8 + b| < 2^31.
-__device__ __forceinline__ int32_t pair8(uint32_t a_bits, uint32_t b_bits) {
-    const uint32_t ab = (uint32_t)__float_as_int(__fadd_rn(__uint_as_float(a_bits), 12582912.0f));
-    const uint32_t bb = (uint32_t)__float_as_int(__fadd_rn(__uint_as_float(b_bits), 12582912.0f));
-    return (int32_t)(ab * 256u + bb - 257u * 0x4B400000u);
-}
-
-// The BF16 bits of a small integer |e| <= 256 (exact: at most 8 significant
-// bits, so the FP32 value's low 16 bits are zero).
-__device__ __forceinline__ uint32_t bf16_bits(int32_t e) {
-    const float f = __fsub_rn(__int_as_float(0x4B400000 + e), 12582912.0f);   // (float)e, exact
-    return __float_as_uint(f) >> 16;
-}
 
 }  // namespace septc
 }  // namespace aqmp
