@@ -597,6 +597,17 @@ def aqmp_bitstream_parse(data: bytes):
     return d, [(int(shapes[2 * i]), int(shapes[2 * i + 1])) for i in range(info.n_planes)], leaves, atoms
 
 
+def _bitstream_head(data: bytes):
+    """The header's part of aqmp_bitstream_parse: (info dict, shapes)."""
+    lib = load_library()
+    info = aqmp_bitstream_info()
+    _check(lib.aqmp_bitstream_parse(data, len(data), ctypes.byref(info), None, None, None))
+    shapes = np.zeros(2 * max(1, info.n_planes), np.int32)
+    _check(lib.aqmp_bitstream_parse(data, len(data), ctypes.byref(info), shapes.ctypes.data, None, None))
+    d = {k: getattr(info, k) for k, _ in aqmp_bitstream_info._fields_}
+    return d, [(int(shapes[2 * i]), int(shapes[2 * i + 1])) for i in range(info.n_planes)]
+
+
 def aqmp_code_from_bitstream(data: bytes) -> Code:
     out = ctypes.c_void_p()
     _check(load_library().aqmp_code_from_bitstream(data, len(data), ctypes.byref(out)))
@@ -626,12 +637,12 @@ def decompress(blob: bytes, stream=None):
     an (h, w, C) uint8 CUDA tensor."""
     import torch
     data = zlib.decompress(blob)
-    info, shapes, _, _ = aqmp_bitstream_parse(data)
-    if len(set(shapes)) != 1:
-        raise ValueError("planes of different sizes do not form one image")
-    h, w = shapes[0]
-    code = aqmp_code_from_bitstream(data)
+    code = aqmp_code_from_bitstream(data)                # the one parse of the leaves and atoms
     try:
+        info, shapes = _bitstream_head(data)
+        if len(set(shapes)) != 1:
+            raise ValueError("planes of different sizes do not form one image")
+        h, w = shapes[0]
         planes = torch.empty((info["n_planes"], h, w), dtype=torch.float32, device="cuda")
         for c in range(info["n_planes"]):
             aqmp_decode(code, c, planes[c], stream)

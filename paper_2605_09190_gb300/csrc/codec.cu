@@ -72,6 +72,7 @@ struct Reader {
     }
     float f32() { uint32_t v = u32(); float f; std::memcpy(&f, &v, 4); return f; }
     uint32_t varint() {
+        if (ok && p < end && *p < 0x80u) return *p++;
         uint32_t v = 0;
         for (int shift = 0; shift < 35; shift += 7) {
             const uint8_t b = u8();
@@ -149,7 +150,8 @@ int parse(const uint8_t *buf, uint64_t len, aqmp_bitstream_info &info, std::vect
     L->reserve(info.n_leaves);
     A->reserve(info.n_atoms);
     struct Node { uint32_t y, x, b; };
-    std::vector<Node> stack;
+    Node stack[3 * 8 + 1];                          // three siblings a level on the way down, kMaxSide / 1 at the most
+    static_assert(kMaxSide <= 128, "the stack's depth");
     const int maxlev = log2i(mb / nb);
     for (uint32_t p = 0; p < np; ++p) {
         const PlaneHead &h = heads[p];
@@ -160,10 +162,10 @@ int parse(const uint8_t *buf, uint64_t len, aqmp_bitstream_info &info, std::vect
         uint32_t next = 0;
         for (uint32_t ry = 0; ry < h.h / mb; ++ry) {
             for (uint32_t rx = 0; rx < h.w / mb; ++rx) {
-                stack.assign(1, Node{ry * (uint32_t)mb, rx * (uint32_t)mb, (uint32_t)mb});
-                while (!stack.empty()) {
-                    Node n = stack.back();
-                    stack.pop_back();
+                int depth = 0;
+                stack[depth++] = Node{ry * (uint32_t)mb, rx * (uint32_t)mb, (uint32_t)mb};
+                while (depth > 0) {
+                    const Node n = stack[--depth];
                     if (next >= h.n_leaves) return set_error(AQMP_E_ARG, "malformed bitstream: too few leaves");
                     const int lev = levels[next];
                     if (lev > maxlev) return set_error(AQMP_E_ARG, "malformed bitstream: bad leaf size");
@@ -171,10 +173,10 @@ int parse(const uint8_t *buf, uint64_t len, aqmp_bitstream_info &info, std::vect
                     if (b > n.b) return set_error(AQMP_E_ARG, "malformed bitstream: leaf larger than its node");
                     if (b < n.b) {
                         const uint32_t c = n.b / 2;
-                        stack.push_back(Node{n.y + c, n.x + c, c});     // BR
-                        stack.push_back(Node{n.y + c, n.x, c});         // BL
-                        stack.push_back(Node{n.y, n.x + c, c});         // TR
-                        stack.push_back(Node{n.y, n.x, c});             // TL, visited next
+                        stack[depth++] = Node{n.y + c, n.x + c, c};     // BR
+                        stack[depth++] = Node{n.y + c, n.x, c};         // BL
+                        stack[depth++] = Node{n.y, n.x + c, c};         // TR
+                        stack[depth++] = Node{n.y, n.x, c};             // TL, visited next
                         continue;
                     }
                     LeafRec rec{};
@@ -200,16 +202,30 @@ int parse(const uint8_t *buf, uint64_t len, aqmp_bitstream_info &info, std::vect
             atoms += t;
         }
         if (atoms != h.n_atoms) return set_error(AQMP_E_ARG, "malformed bitstream: atom count mismatch");
+        // indices and coefficients are plain arrays: one check of the length, one pass
+        if ((uint64_t)(r.end - r.p) < 6 * atoms) return set_error(AQMP_E_ARG, "malformed bitstream: truncated");
+        const uint8_t *pj = r.p, *pa = r.p + 2 * atoms;
+        r.p += 6 * atoms;
         const size_t a0 = A->size();
         A->resize(a0 + atoms);
-        for (uint64_t i = 0; i < atoms; ++i) (*A)[a0 + i].j = r.u16();
-        for (uint64_t i = 0; i < atoms; ++i) (*A)[a0 + i].alpha = r.f32();
-        if (!r.ok) return set_error(AQMP_E_ARG, "malformed bitstream: truncated");
+        AtomRec *a = A->data() + a0;
         for (size_t i = first; i < L->size(); ++i) {
             const LeafRec &rec = (*L)[i];
             const uint32_t m = (uint32_t)(info.dict_id == AQMP_DICT_DCT_HAAR ? 2 : 1) * rec.b * rec.b;
-            for (uint32_t t = 0; t < rec.n_atoms; ++t)
-                if ((*A)[rec.atom_off + t].j >= m) return set_error(AQMP_E_ARG, "malformed bitstream: atom index");
+            const uint32_t na = rec.n_atoms;
+            uint32_t top = 0;
+            for (uint32_t t = 0; t < na; ++t) {
+                const uint32_t j = (uint32_t)pj[2 * t] | ((uint32_t)pj[2 * t + 1] << 8);
+                const uint32_t v = (uint32_t)pa[4 * t] | ((uint32_t)pa[4 * t + 1] << 8) |
+                                   ((uint32_t)pa[4 * t + 2] << 16) | ((uint32_t)pa[4 * t + 3] << 24);
+                a[t].j = j;
+                std::memcpy(&a[t].alpha, &v, 4);
+                top = std::max(top, j);
+            }
+            if (na > 0 && top >= m) return set_error(AQMP_E_ARG, "malformed bitstream: atom index");
+            pj += 2 * na;
+            pa += 4 * na;
+            a += na;
         }
     }
     if (r.p != r.end) return set_error(AQMP_E_ARG, "malformed bitstream: trailing bytes");

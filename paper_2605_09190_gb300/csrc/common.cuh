@@ -126,4 +126,15 @@ __device__ __forceinline__ void raise_error(Counters *ctr, unsigned code, unsign
 constexpr unsigned kDevErrQueueOverflow = 6;
 constexpr unsigned kDevErrTimeout = 7;
 
+// Byte `byte` of w0 and of w1, each minus 128, as two BF16 (w0's in the low
+// half): 128 + the low seven bits, less 128 where the byte's top bit is set
+// and 256 where not, all exact.
+__device__ __forceinline__ uint32_t bytes_less_128(uint32_t w0, uint32_t w1, int byte) {
+    const uint32_t w = __byte_perm(w0, w1, (uint32_t)(byte | ((4 + byte) << 8)) * 0x11u);
+    const uint32_t x = (w & 0x007f007fu) | 0x43004300u, c = (~w & 0x00800080u) | 0xC300C300u;
+    uint32_t d;
+    asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(x), "r"(c));
+    return d;
+}
+
 }  // namespace aqmp

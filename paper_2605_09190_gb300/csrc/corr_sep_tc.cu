@@ -106,16 +106,6 @@ __device__ __forceinline__ uint32_t biased_pair(uint32_t a_bits, uint32_t b_bits
     return biased_one(a_bits) * 256u + biased_one(b_bits);
 }
 
-// Byte t of two words' numbers, each minus 128, as two BF16: 128 + the low
-// seven bits, less 128 where the byte's top bit is set and 256 where not.
-__device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1, int byte) {
-    const uint32_t w = __byte_perm(w0, w1, (uint32_t)(byte | ((4 + byte) << 8)) * 0x11u);
-    const uint32_t x = (w & 0x007f007fu) | 0x43004300u, c = (~w & 0x00800080u) | 0xC300C300u;
-    uint32_t d;
-    asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(x), "r"(c));
-    return d;
-}
-
 }  // namespace septc
 
 // Y map: the gathered leaves viewed as [capacity * 64 rows][64] BF16 (row m of
@@ -274,8 +264,8 @@ corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constan
                 }
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
-                    e[t][i] = digit_pair(lo[0], lo[1], t);
-                    e[4 + t][i] = digit_pair(hi[0], hi[1], t);
+                    e[t][i] = bytes_less_128(lo[0], lo[1], t);
+                    e[4 + t][i] = bytes_less_128(hi[0], hi[1], t);
                 }
             }
             unsigned char *dst = gbase + kOffE + half * kTileE + r64 * 128 + (((2 * cg + h) ^ (r64 & 7)) << 4);
