@@ -106,6 +106,79 @@ __device__ __forceinline__ uint32_t biased_pair(uint32_t a_bits, uint32_t b_bits
     return biased_one(a_bits) * 256u + biased_one(b_bits);
 }
 
+// Z~ + 128 in every byte from its six digit sums; c the centring term.
+__device__ __forceinline__ unsigned long long join_digits(uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t a4,
+                                                          uint32_t a5, unsigned long long c) {
+    constexpr unsigned long long kC = 0x8080808080808080ull - (unsigned long long)kPairBias * 0x100010001ull;
+    return (unsigned long long)biased_pair(a1, a0) + ((unsigned long long)biased_pair(a3, a2) << 16) +
+           ((unsigned long long)biased_pair(a5, a4) << 32) + (kC + c);
+}
+
+// The words of T + the rounding's bias from output i's 13 diagonals.
+__device__ __forceinline__ void join_diagonals(const uint32_t (&a)[13][4], int i, uint32_t (&T)[4]) {
+    typedef unsigned __int128 u128;
+    constexpr u128 kPairs = (u128)kPairBias * ((((u128)1 << 48 | (u128)1 << 32) | ((u128)1 << 16 | 1)) |
+                                               ((u128)1 << 80 | (u128)1 << 64));
+    constexpr u128 kC = (((u128)kDigitBiasHi << 64) | kDigitBiasLo) - kPairs - ((u128)kOneBias << 96);
+    const u128 even = (u128)biased_pair(a[1][i], a[0][i]) | (u128)biased_pair(a[5][i], a[4][i]) << 32 |
+                      (u128)biased_pair(a[9][i], a[8][i]) << 64 | (u128)biased_one(a[12][i]) << 96;
+    const u128 odd = (u128)biased_pair(a[3][i], a[2][i]) << 16 | (u128)biased_pair(a[7][i], a[6][i]) << 48 |
+                     (u128)biased_pair(a[11][i], a[10][i]) << 80;
+    const u128 t = even + odd + kC;
+    T[0] = (uint32_t)t;
+    T[1] = (uint32_t)(t >> 32);
+    T[2] = (uint32_t)(t >> 64);
+    T[3] = (uint32_t)(t >> 96);
+}
+
+// The 13 diagonals of 8 columns from column `col` of each 32, joined.
+__device__ __forceinline__ void drain_diagonals(uint32_t lane_base, int col, uint32_t (&T)[8][4]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t a[13][4];
+#pragma unroll
+        for (int c = 0; c < 13; ++c) tmem_ld4(lane_base + 32 * c + col + 4 * h, a[c]);
+        wait_ld();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) join_diagonals(a, i, T[4 * h + i]);
+    }
+}
+
+// x + y and y - x of two 16-byte chunks of BF16, in place.
+__device__ __forceinline__ void fold_chunks(uint4 *pa, uint4 *pb) {
+    uint4 x = *pa, y = *pb;
+    auto both = [](uint32_t &u, uint32_t &v) {
+        uint32_t s, d;
+        asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(s) : "r"(u), "r"(v));
+        asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(v), "r"(u));
+        u = s;
+        v = d;
+    };
+    both(x.x, y.x);
+    both(x.y, y.y);
+    both(x.z, y.z);
+    both(x.w, y.w);
+    *pa = x;
+    *pb = y;
+}
+
+// Stage 2's MMAs over the 16-wide steps k0 .. k1: every digit tile of E
+// against the six stacked digits at D (192 rows), into the diagonals' columns.
+__device__ __forceinline__ void issue_stage2(uint32_t tmem, uint32_t sE, uint32_t sD, int k0, int k1) {
+    for (int kk = k0; kk < k1; ++kk) {
+        const uint32_t more = kk > k0 ? 1u : 0u;
+        const unsigned long long ad = smem_desc_m_major(sE) + 128ull * kk;
+        const unsigned long long bd = smem_desc(sD) + 2ull * kk;
+        constexpr unsigned long long kStepE = 2 * kTileE >> 4;
+        // digits 0 and 6 meet every diagonal but the last first
+        mma_ss(tmem, ad, bd, idesc(192, true), more);
+        mma_ss(tmem + 192, ad + 6 * kStepE, bd, idesc(192, true), more);
+        mma_ss(tmem + 224, ad + 7 * kStepE, bd, idesc(160, true), 1u);
+        mma_ss(tmem + 384, ad + 7 * kStepE, bd + (5 * 32 * 128 >> 4), idesc(32, true), more);
+        for (int t = 1; t < 6; ++t) mma_ss(tmem + 32 * t, ad + t * kStepE, bd, idesc(192, true), 1u);
+    }
+}
+
 }  // namespace septc
 
 // Y map: the gathered leaves viewed as [capacity * 64 rows][64] BF16 (row m of
@@ -201,20 +274,7 @@ corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constan
             unsigned char *t = gbase + kOffY + (2 * buf + l) * kTileY;
             uint4 *pa = reinterpret_cast<uint4 *>(t + m * 128 + ((j ^ (m & 7)) << 4));
             uint4 *pb = reinterpret_cast<uint4 *>(t + (63 - m) * 128 + ((j ^ (7 - (m & 7))) << 4));
-            uint4 x = *pa, y = *pb;
-            auto both = [](uint32_t &u, uint32_t &v) {
-                uint32_t s, d;
-                asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(s) : "r"(u), "r"(v));
-                asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(v), "r"(u));
-                u = s;
-                v = d;
-            };
-            both(x.x, y.x);
-            both(x.y, y.y);
-            both(x.z, y.z);
-            both(x.w, y.w);
-            *pa = x;
-            *pb = y;
+            fold_chunks(pa, pb);
             fence_async();
         }
         fence_before();
@@ -251,14 +311,9 @@ corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constan
                 uint32_t lo[2], hi[2];
 #pragma unroll
                 for (int par = 0; par < 2; ++par) {
-                    // Z~ + 128 in every byte, the biases of the three pairs removed
-                    constexpr unsigned long long kC =
-                        0x8080808080808080ull - (unsigned long long)kPairBias * 0x100010001ull;
-                    const unsigned long long c = kC + (difference ? 0ull : cen[16 * cg + 8 * h + 2 * i + par]);
                     const unsigned long long z =
-                        (unsigned long long)biased_pair(a[par][1][i], a[par][0][i]) +
-                        ((unsigned long long)biased_pair(a[par][3][i], a[par][2][i]) << 16) +
-                        ((unsigned long long)biased_pair(a[par][5][i], a[par][4][i]) << 32) + c;
+                        join_digits(a[par][0][i], a[par][1][i], a[par][2][i], a[par][3][i], a[par][4][i], a[par][5][i],
+                                    difference ? 0ull : cen[16 * cg + 8 * h + 2 * i + par]);
                     lo[par] = (uint32_t)z;
                     hi[par] = (uint32_t)(z >> 32);
                 }
@@ -281,19 +336,7 @@ corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constan
         for (int par = 0; par < 2 && ok; ++par) {
             if (tid == 0) {
                 fence_after();
-                const int k0 = fold ? 2 * par : 0, k1 = fold ? k0 + 2 : 4;
-                for (int kk = k0; kk < k1; ++kk) {
-                    const uint32_t more = kk > k0 ? 1u : 0u;
-                    const unsigned long long ad = smem_desc_m_major(sE) + 128ull * kk;
-                    const unsigned long long bd = smem_desc(sD + par * 192 * 128) + 2ull * kk;
-                    constexpr unsigned long long kStepE = 2 * kTileE >> 4;
-                    // digits 0 and 6 meet every diagonal but the last first
-                    mma_ss(tmem, ad, bd, idesc(192, true), more);
-                    mma_ss(tmem + 192, ad + 6 * kStepE, bd, idesc(192, true), more);
-                    mma_ss(tmem + 224, ad + 7 * kStepE, bd, idesc(160, true), 1u);
-                    mma_ss(tmem + 384, ad + 7 * kStepE, bd + (5 * 32 * 128 >> 4), idesc(32, true), more);
-                    for (int t = 1; t < 6; ++t) mma_ss(tmem + 32 * t, ad + t * kStepE, bd, idesc(192, true), 1u);
-                }
+                issue_stage2(tmem, sE, sD + par * 192 * 128, fold ? 2 * par : 0, fold ? 2 * par + 2 : 4);
                 mma_commit(barMma);
             }
             if (par == 1) finish(pair, 0);
@@ -302,30 +345,7 @@ corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constan
             if (!ok) break;
             fence_after();
             // ---- drain 2: q = 2 (8 cg + j) + par, 13 diagonals each
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                uint32_t a[13][4];
-#pragma unroll
-                for (int c = 0; c < 13; ++c) tmem_ld4(lane_base + 32 * c + 8 * cg + 4 * h, a[c]);
-                wait_ld();
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    typedef unsigned __int128 u128;
-                    constexpr u128 kPairs = (u128)kPairBias * ((((u128)1 << 48 | (u128)1 << 32) | ((u128)1 << 16 | 1)) |
-                                                               ((u128)1 << 80 | (u128)1 << 64));
-                    constexpr u128 kC = (((u128)kDigitBiasHi << 64) | kDigitBiasLo) - kPairs - ((u128)kOneBias << 96);
-                    const u128 even = (u128)biased_pair(a[1][i], a[0][i]) | (u128)biased_pair(a[5][i], a[4][i]) << 32 |
-                                      (u128)biased_pair(a[9][i], a[8][i]) << 64 | (u128)biased_one(a[12][i]) << 96;
-                    const u128 odd = (u128)biased_pair(a[3][i], a[2][i]) << 16 |
-                                     (u128)biased_pair(a[7][i], a[6][i]) << 48 |
-                                     (u128)biased_pair(a[11][i], a[10][i]) << 80;
-                    const u128 t = even + odd + kC;
-                    T[4 * h + i][0] = (uint32_t)t;
-                    T[4 * h + i][1] = (uint32_t)(t >> 32);
-                    T[4 * h + i][2] = (uint32_t)(t >> 64);
-                    T[4 * h + i][3] = (uint32_t)(t >> 96);
-                }
-            }
+            drain_diagonals(lane_base, 8 * cg, T);
             fence_before();
             __syncthreads();
         }
@@ -339,17 +359,266 @@ corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constan
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
-bool corr_sep_tc_available(int b, int) { return b == septc::kB; }
+// ------------------------------------------------------------- side 128
+//
+// The DCT-II family, one leaf at a time: the 128 rows of stage 1's tile are the
+// folded pixel rows m (64 sums, 64 differences), K = i = 128, and the digit
+// sums stay below 128 x 256 x 128 = 2^22 (the top digit is at most 32).  The
+// digits e_t of one class of rows (128 p, K = 64 m) fill 128 KB, so the classes
+// b = 0, 1 (the even and the odd q) go one after the other, and stage 1's
+// products are formed for one parity a of p at a time (384 columns), of which a
+// class's half of the rows is drained.  Stage 2 as at side 64, 32 of the class's
+// q a pass; its digit sums reach 0.99 x 2^22 for the rows there are (checked
+// when the table is made).
+//   The six digits of all 128 rows take 192 KB: they come through one 48 KB
+// buffer, as (parity of the row, half of K) chunks.  Class b takes (1 - b, 1 - b)
+// first, which the class before left there, then (1 - b, b), (b, 1 - b) and
+// (b, b), which is also stage 2's operand.
+//   A 17th warp loads and issues, so that the 16 that drain round and store a
+// pass's outputs meanwhile.  M is ordered (p / 16, a, p' mod 8), p' = p / 2, so
+// that a thread writes whole chunks and a warp's 32 outputs are contiguous.
+// 3072 leaves: 0.62 ms; both families of the SIMT twin took 3.65 ms, bound by
+// the wide integer multiply-adds, and the Haar family alone takes 0.24.
+namespace septc {
+constexpr int kThreads128 = 17 * 32;
+constexpr int kChunk = 384 * 128;                                // bytes of a digit chunk
+constexpr int kOffE128 = 0;
+constexpr int kOffD128 = kOffE128 + 8 * 2 * kTileE;
+constexpr int kOffY128 = kOffD128 + kChunk;                      // [half of K][128 rows]
+constexpr int kOffCen128 = kOffY128 + 2 * 128 * 128;
+constexpr int kOffBar128 = kOffCen128 + 8 * 128;                 // digits, pixels, producer's, drainers', back
+constexpr int kOffMisc128 = kOffBar128 + 8 * 8;
+constexpr int kSmemBytes128 = kOffMisc128 + 16 + 1024;
+}  // namespace septc
+
+// Y map: [capacity * 128 rows][128] BF16 in boxes of 128 rows x 64; digit map:
+// [2 * 768 rows][128] BF16, row (a, q half, s, q mod 32 of the parity) of a family.
+__global__ void __launch_bounds__(septc::kThreads128, 1)
+corr_sep_tc128_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmD, int M,
+                      const long long *__restrict__ Rs, const unsigned *count_dev, long long fixed_count,
+                      float2 *__restrict__ c0, Counters *ctr) {
+    using namespace septc;
+    constexpr int b = 128;
+    const long long count = count_dev ? (long long)*count_dev : fixed_count;
+    if ((long long)blockIdx.x >= count) return;                  // uniform
+
+    extern __shared__ unsigned char smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    unsigned char *gbase = smem_raw + (base - raw);
+    const uint32_t sE = base + kOffE128, sD = base + kOffD128, sY = base + kOffY128, sBar = base + kOffBar128;
+    const uint32_t barD = sBar, barY = sBar + 8, barP = sBar + 16, barA = sBar + 24, barC = sBar + 32;
+    unsigned long long *cen = reinterpret_cast<unsigned long long *>(gbase + kOffCen128);
+    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(gbase + kOffMisc128);
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        mbar_init(barD, 1);
+        mbar_init(barY, 1);
+        mbar_init(barP, 1);
+        mbar_init(barA, 1);
+        mbar_init(barC, 16);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_holder)), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid < b) cen[tid] = (unsigned long long)(Rs[tid] * 256);      // of a sum of two rows
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *tmem_holder;
+    bool ok = true;
+
+    if (warp == 16) {
+        if (lane == 0) {
+            uint32_t phD = 0, phP = 0, phC = 0;
+            auto load_digits = [&](int a, int kh) {
+                mbar_expect_tx(barD, kChunk);
+                for (int t = 0; t < 3; ++t) tma_load_2d(sD + t * 128 * 128, &tmD, barD, 64 * kh, 384 * a + 128 * t);
+            };
+            auto load_pixels = [&](long long leaf) {
+                mbar_expect_tx(barY, 2 * 128 * 128);
+                for (int kh = 0; kh < 2; ++kh) tma_load_2d(sY + kh * 128 * 128, &tmY, barY, 64 * kh, (int)(128 * leaf));
+            };
+            auto wait = [&](uint32_t bar, uint32_t &phase) {
+                ok = ok && mbar_wait(bar, phase);
+                phase ^= 1u;
+                return ok;
+            };
+            // stage 1 over one half of K
+            auto stage1 = [&](int kh, uint32_t acc, uint32_t bar) {
+                fence_after();
+                const unsigned long long ad = smem_desc(sY + kh * 128 * 128), bd = smem_desc(sD);
+                for (int qh = 0; qh < 2; ++qh)
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        mma_ss(tmem + 192 * qh, ad + 2ull * kk, bd + (unsigned long long)(qh * 192 * 128 >> 4) + 2ull * kk,
+                               idesc(192, false), kk > 0 ? 1u : acc);
+                mma_commit(bar);
+            };
+            load_digits(1, 1);
+            load_pixels(blockIdx.x);
+            bool fresh = true;
+            for (long long leaf = blockIdx.x; ok && leaf < count; leaf += gridDim.x) {
+                for (int cls = 0; cls < 2 && ok; ++cls) {
+                    if (!wait(barC, phC)) break;                  // pixels folded, accumulators drained
+                    if (fresh && !wait(barD, phD)) break;
+                    fresh = false;
+                    stage1(1 - cls, 0u, barP);                    // chunk (1 - cls, 1 - cls)
+                    if (!wait(barP, phP)) break;
+                    load_digits(1 - cls, cls);
+                    if (!wait(barD, phD)) break;
+                    stage1(cls, 1u, barA);
+                    ok = mbar_wait(barA, 0);                      // four completions a class: parities 0, 1, 0, 1
+                    if (!ok) break;
+                    load_digits(cls, 1 - cls);
+                    if (!wait(barC, phC) || !wait(barD, phD)) break;
+                    stage1(1 - cls, 0u, barP);
+                    if (!wait(barP, phP)) break;
+                    load_digits(cls, cls);
+                    if (!wait(barD, phD)) break;
+                    stage1(cls, 1u, barA);
+                    ok = mbar_wait(barA, 1);
+                    if (!ok) break;
+                    if (cls == 1 && leaf + gridDim.x < count) load_pixels(leaf + gridDim.x);
+                    for (int qh = 0; qh < 2 && ok; ++qh) {
+                        if (!wait(barC, phC)) break;              // digits written; the pass before drained
+                        fence_after();
+                        issue_stage2(tmem, sE, sD + qh * 192 * 128, 0, 4);
+                        mma_commit(barA);
+                    }
+                }
+            }
+        }
+    } else {
+        const int quarter = warp & 3, cg = warp >> 2;
+        const int row = quarter * 32 + lane;
+        const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
+        const int k = row & 63;                                   // stage 1: row of a class
+        const int p = 2 * (8 * (row >> 4) + (row & 7)) + ((row >> 3) & 1);     // stage 2: M index -> p
+        uint32_t phA = 0, phY = 0;
+        uint32_t T[8][4];
+        auto wait = [&](uint32_t bar, uint32_t &phase) {
+            ok = __all_sync(0xffffffffu, mbar_wait(bar, phase)) && ok;
+            phase ^= 1u;
+            fence_after();
+            return ok;
+        };
+        // this warp's reads of tensor memory and writes of shared memory are done
+        auto done = [&]() {
+            fence_before();
+            fence_async();
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(barC) : "memory");
+        };
+        auto finish = [&](long long leaf, int cls, int qh) {
+            float2 *out = c0 + leaf * M + (2 * (32 * qh + 8 * cg) + cls) * b + p;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const df v = biased_to_df(T[j][0], T[j][1], T[j][2], T[j][3]);
+                out[2 * j * b] = make_float2(v.hi, v.lo);
+            }
+        };
+        long long pending = -1;
+        for (long long leaf = blockIdx.x; ok && leaf < count; leaf += gridDim.x) {
+            if (!wait(barY, phY)) break;
+            // rows m and 127 - m, two 16-byte chunks a thread
+            for (int o = tid; o < 1024; o += 512) {
+                const int kh = o >> 9, m = (o >> 3) & 63, j = o & 7;
+                unsigned char *t = gbase + kOffY128 + kh * 128 * 128;
+                fold_chunks(reinterpret_cast<uint4 *>(t + m * 128 + ((j ^ (m & 7)) << 4)),
+                            reinterpret_cast<uint4 *>(t + (127 - m) * 128 + ((j ^ (7 - (m & 7))) << 4)));
+            }
+            done();
+            if (pending >= 0) finish(pending, 1, 1);
+            for (int cls = 0; cls < 2 && ok; ++cls) {
+                // ---- stage 1 and the digits, the p of parity 1 - cls, then of cls
+                for (int turn = 0; turn < 2; ++turn) {
+                    const int a = turn ? cls : 1 - cls;
+                    if (!wait(barA, phA)) break;
+                    if ((quarter >> 1) == cls) {
+#pragma unroll 1
+                        for (int h = 0; h < 2; ++h) {
+                            // p' = 16 cg + 8 h + (0 .. 7)
+                            uint32_t z[2][4][2];
+#pragma unroll
+                            for (int g = 0; g < 2; ++g) {
+                                uint32_t v[6][4];
+#pragma unroll
+                                for (int sd = 0; sd < 6; ++sd)
+                                    tmem_ld4(lane_base + 192 * (cg >> 1) + 32 * sd + 16 * (cg & 1) + 8 * h + 4 * g, v[sd]);
+                                wait_ld();
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) {
+                                    const unsigned long long x =
+                                        join_digits(v[0][i], v[1][i], v[2][i], v[3][i], v[4][i], v[5][i],
+                                                    cls ? 0ull : cen[2 * (16 * cg + 8 * h + 4 * g + i) + a]);
+                                    z[g][i][0] = (uint32_t)x;
+                                    z[g][i][1] = (uint32_t)(x >> 32);
+                                }
+                            }
+                            const int chunk = 2 * (2 * cg + h) + a;
+                            unsigned char *dst = gbase + kOffE128 + (chunk >> 3) * kTileE + k * 128 +
+                                                 (((chunk & 7) ^ (k & 7)) << 4);
+#pragma unroll
+                            for (int t = 0; t < 8; ++t) {
+                                const int w = t >> 2, y = t & 3;
+                                *reinterpret_cast<uint4 *>(dst + t * 2 * kTileE) =
+                                    make_uint4(bytes_less_128(z[0][0][w], z[0][1][w], y),
+                                               bytes_less_128(z[0][2][w], z[0][3][w], y),
+                                               bytes_less_128(z[1][0][w], z[1][1][w], y),
+                                               bytes_less_128(z[1][2][w], z[1][3][w], y));
+                            }
+                        }
+                    }
+                    done();
+                }
+                // ---- stage 2
+                for (int qh = 0; qh < 2 && ok; ++qh) {
+                    if (!wait(barA, phA)) break;
+                    drain_diagonals(lane_base, 8 * cg, T);
+                    if (qh == 0 || cls == 0) {
+                        done();
+                        finish(leaf, cls, qh);
+                    }
+                }
+            }
+            pending = leaf;
+        }
+        if (ok && pending >= 0) finish(pending, 1, 1);
+    }
+    fence_before();
+    const bool all_ok = __syncthreads_and(ok) != 0;
+    if (tid == 0 && !all_ok && ctr) raise_error(ctr, kDevErrTimeout, 13u);
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+}
+
+bool corr_sep_tc_available(int b, int) { return b == septc::kB || b == 128; }
 
 cudaError_t launch_corr_sep_tc(const CorrArgs &a, cudaStream_t st) {
     const DictDev &d = *a.d;
-    if (d.b != septc::kB || !d.tmap_sepd || !a.tmap_Ysep) return cudaErrorInvalidValue;
+    if (!corr_sep_tc_available(d.b, d.nf) || !d.tmap_sepd || !a.tmap_Ysep) return cudaErrorInvalidValue;
     const long long rows = a.count ? (long long)a.capacity : a.fixed_count;
     if (rows <= 0) return cudaSuccess;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if (d.b == 128) {
+        if (d.fam0 != 0 || a.fmask != 1) return cudaErrorInvalidValue;            // the DCT-II family alone
+        e = cudaFuncSetAttribute(corr_sep_tc128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 septc::kSmemBytes128);
+        if (e != cudaSuccess) return e;
+        corr_sep_tc128_kernel<<<(unsigned)(rows < sms ? rows : sms), septc::kThreads128, septc::kSmemBytes128, st>>>(
+            *reinterpret_cast<const CUtensorMap *>(a.tmap_Ysep), *reinterpret_cast<const CUtensorMap *>(d.tmap_sepd),
+            d.nf * 128 * 128, d.Rs, a.count, a.fixed_count, a.c0, a.ctr);
+        return cudaGetLastError();
+    }
     const long long pairs = (rows + 1) / 2;
     const unsigned grid = (unsigned)(pairs < sms ? pairs : sms);
     e = cudaFuncSetAttribute(corr_sep_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, septc::kSmemBytes);

@@ -290,6 +290,10 @@ cudaError_t corr_sep_hybrid(const CorrArgs &ca, int b, cudaStream_t st) {
     return e;
 }
 
+// Whether the tuner times the two: at side 128 the tensor cores (0.62 + 0.24 ms
+// with the Haar family, for 3072 leaves) leave the SIMT path (3.65 ms) no size.
+bool corr_tuned(int b, int nf) { return b == 64 && corr_sep_tc_available(b, nf); }
+
 // ------------------------------------------------------------ autotuner
 //
 // Choice points whose candidates give the same result bit for bit: the
@@ -507,7 +511,7 @@ int get_dict(Ctx *c, int b, int dict_id, cudaStream_t st, Dict **out, bool table
             CK(cudaMemcpyAsync(d.Rs, rows.data(), sizeof(long long) * rows.size(), cudaMemcpyHostToDevice, st));
             if (corr_sep_tc_available(b, d.nf)) {
                 // balanced base-2^8 digits d_s of Bf (s = 0..5) as BF16, 6 b rows
-                // a family: row r of digit s at (r mod 2, s, r / 2)
+                // a family: row r of digit s at (r mod 2, r / 64, s, r / 2 mod 32)
                 std::vector<__nv_bfloat16> dg(6 * 2 * bb);
                 for (int F = 0; F < 2; ++F)
                     for (int r = 0; r < b; ++r)
@@ -516,49 +520,63 @@ int get_dict(Ctx *c, int b, int dict_id, cudaStream_t st, Dict **out, bool table
                             for (int sd = 0; sd < 6; ++sd) {
                                 long long dv = sd < 5 ? ((f + 128) & 255) - 128 : f;
                                 f = (f - dv) >> 8;
-                                const size_t at = (size_t)F * 6 * b + (r & 1) * 3 * b + sd * (b / 2) + (r >> 1);
+                                const size_t at = (size_t)F * 6 * b + (r & 1) * 3 * b + (r >> 6) * 192 + sd * 32 + ((r >> 1) & 31);
                                 dg[at * b + col] = __float2bfloat16((float)dv);
                             }
                         }
+                // side 128: the digit sums of stage 2 (corr_sep_tc.cu), products with
+                // eight digits of magnitude 128, have to stay below 2^22
+                if (b == 128)
+                    for (int r = 0; r < b; ++r) {
+                        double sum[6] = {};
+                        for (int sd = 0; sd < 6; ++sd)
+                            for (int col = 0; col < b / 2; ++col)
+                                sum[sd] += std::fabs(__bfloat162float(
+                                    dg[((size_t)(r & 1) * 3 * b + (r >> 6) * 192 + sd * 32 + ((r >> 1) & 31)) * b + col]));
+                        if (128.0 * (sum[0] + sum[1] + sum[2] + sum[3] + sum[4] + sum[5]) >= 4194304.0)
+                            return AQMP_E_UNSUPPORTED;
+                    }
                 if ((rc0 = Dn->sepd.reserve(sizeof(__nv_bfloat16) * dg.size()))) return rc0;
                 d.sepd = (__nv_bfloat16 *)Dn->sepd.p;
                 CK(cudaMemcpyAsync(d.sepd, dg.data(), sizeof(__nv_bfloat16) * dg.size(), cudaMemcpyHostToDevice, st));
                 if ((rc0 = encode_bf16_map(&Dn->tmap_sd, d.sepd, 6ull * 2 * b, b, 128))) return rc0;
                 d.tmap_sepd = &Dn->tmap_sd;
-                // the BF16 form with rescore (corr_sepbf_tc.cu): three
-                // 128-row tiles of 1-D rows, [bf16(B_0); bf16(B_0 - bf16(B_0))],
-                // the same for family 1, then [|B_0| ; |B_1|] rounded up to
-                // BF16; and the row sums R[F][p] = sum_i B[F][p][i] as (hi, lo)
-                std::vector<__nv_bfloat16> sb(3 * 2 * bb);
-                std::vector<float2> rs(2 * (size_t)b);
-                for (int F = 0; F < 2; ++F)
-                    for (int r = 0; r < b; ++r) {
-                        double sum = 0.0;
-                        for (int col = 0; col < b; ++col) {
-                            const double x = basis[F * bb + (size_t)r * b + col];
-                            sum += x;
-                            const __nv_bfloat16 hi = __float2bfloat16_rn((float)x);
-                            const double rem = x - (double)__bfloat162float(hi);
-                            const __nv_bfloat16 lo = __float2bfloat16_rn((float)rem);
-                            float ax = (float)std::fabs(x);
-                            if ((double)ax < std::fabs(x)) ax = std::nextafter(ax, INFINITY);
-                            __nv_bfloat16 au = __float2bfloat16_rn(ax);
-                            if (__bfloat162float(au) < ax) au = __float2bfloat16_ru(ax);
-                            sb[((size_t)F * 2 * b + r) * b + col] = hi;
-                            sb[((size_t)F * 2 * b + b + r) * b + col] = lo;
-                            sb[((size_t)4 * b + F * b + r) * b + col] = au;
+                if (corr_sepbf_available(b)) {
+                    // the BF16 form with rescore (corr_sepbf_tc.cu): three
+                    // 128-row tiles of 1-D rows, [bf16(B_0); bf16(B_0 - bf16(B_0))],
+                    // the same for family 1, then [|B_0| ; |B_1|] rounded up to
+                    // BF16; and the row sums R[F][p] = sum_i B[F][p][i] as (hi, lo)
+                    std::vector<__nv_bfloat16> sb(3 * 2 * bb);
+                    std::vector<float2> rs(2 * (size_t)b);
+                    for (int F = 0; F < 2; ++F)
+                        for (int r = 0; r < b; ++r) {
+                            double sum = 0.0;
+                            for (int col = 0; col < b; ++col) {
+                                const double x = basis[F * bb + (size_t)r * b + col];
+                                sum += x;
+                                const __nv_bfloat16 hi = __float2bfloat16_rn((float)x);
+                                const double rem = x - (double)__bfloat162float(hi);
+                                const __nv_bfloat16 lo = __float2bfloat16_rn((float)rem);
+                                float ax = (float)std::fabs(x);
+                                if ((double)ax < std::fabs(x)) ax = std::nextafter(ax, INFINITY);
+                                __nv_bfloat16 au = __float2bfloat16_rn(ax);
+                                if (__bfloat162float(au) < ax) au = __float2bfloat16_ru(ax);
+                                sb[((size_t)F * 2 * b + r) * b + col] = hi;
+                                sb[((size_t)F * 2 * b + b + r) * b + col] = lo;
+                                sb[((size_t)4 * b + F * b + r) * b + col] = au;
+                            }
+                            const float rh = (float)sum;
+                            rs[(size_t)F * b + r] = make_float2(rh, (float)(sum - (double)rh));
                         }
-                        const float rh = (float)sum;
-                        rs[(size_t)F * b + r] = make_float2(rh, (float)(sum - (double)rh));
-                    }
-                if ((rc0 = Dn->sepbf.reserve(sizeof(__nv_bfloat16) * sb.size() + sizeof(float2) * rs.size())))
-                    return rc0;
-                d.sepbf = (__nv_bfloat16 *)Dn->sepbf.p;
-                d.Rbf = (float2 *)(d.sepbf + sb.size());
-                CK(cudaMemcpyAsync(d.sepbf, sb.data(), sizeof(__nv_bfloat16) * sb.size(), cudaMemcpyHostToDevice, st));
-                CK(cudaMemcpyAsync(d.Rbf, rs.data(), sizeof(float2) * rs.size(), cudaMemcpyHostToDevice, st));
-                if ((rc0 = encode_bf16_map(&Dn->tmap_sbf, d.sepbf, 6ull * b, b, 128))) return rc0;
-                d.tmap_sepbf = &Dn->tmap_sbf;
+                    if ((rc0 = Dn->sepbf.reserve(sizeof(__nv_bfloat16) * sb.size() + sizeof(float2) * rs.size())))
+                        return rc0;
+                    d.sepbf = (__nv_bfloat16 *)Dn->sepbf.p;
+                    d.Rbf = (float2 *)(d.sepbf + sb.size());
+                    CK(cudaMemcpyAsync(d.sepbf, sb.data(), sizeof(__nv_bfloat16) * sb.size(), cudaMemcpyHostToDevice, st));
+                    CK(cudaMemcpyAsync(d.Rbf, rs.data(), sizeof(float2) * rs.size(), cudaMemcpyHostToDevice, st));
+                    if ((rc0 = encode_bf16_map(&Dn->tmap_sbf, d.sepbf, 6ull * b, b, 128))) return rc0;
+                    d.tmap_sepbf = &Dn->tmap_sbf;
+                }
             }
         }
         // W = C H^T with exact structural zeros: entries below 2^-40 are the
@@ -931,7 +949,7 @@ int aqmp_encode_planes(const aqmp_params *params, const aqmp_plane *planes, int 
         if (!tune) return true;
         for (int l = 0; l < nlev; ++l) {
             const int b = P.max_block >> l;
-            if (!simt && !bf16 && !fp8 && !(resc && corr_sepbf_available(b)) && corr_sep_tc_available(b, dicts[l]->d.nf) &&
+            if (!simt && !bf16 && !fp8 && !(resc && corr_sepbf_available(b)) && corr_tuned(b, dicts[l]->d.nf) &&
                 c->tuner.slot(Tuner::CORR, b, P.dict_id, P.precision, cap[l]).chosen < 0)
                 return false;
             if (!alt_threads && !omp && mp_has_variant(b, dicts[l]->d.nf) &&
@@ -1028,7 +1046,7 @@ int aqmp_encode_planes(const aqmp_params *params, const aqmp_plane *planes, int 
                           [&] { return launch_corr_tc_fp8(ca, (const float *)c->inv_sl.p, st); }));
         } else if (simt || !tc_ok) {
             CK(corr_simt());
-        } else if (!tune) {
+        } else if (!tune || !corr_tuned(b, d.nf)) {
             CK(corr_tc());
         } else {
             Tuner::Slot &ts = c->tuner.slot(Tuner::CORR, b, P.dict_id, P.precision, cap[l]);
@@ -1688,7 +1706,7 @@ int aqmp_correlate(int b, int dict_id, const uint8_t *blocks, int64_t L, float *
         return fail(AQMP_E_ARG, "gemm must be 0 (separable, best kernel), 1 (separable SIMT), 2 (BF16 form), "
                                 "3 (dense tensor cores), 4 (dense SIMT), 5 (FP8 form) or 6 (separable "
                                 "tensor cores, every family)");
-    if (gemm == 6 && !corr_sep_tc_available(b, 2))
+    if (gemm == 6 && b != 64)
         return fail(AQMP_E_UNSUPPORTED, "no separable tensor-core kernel for side %d", b);
     if (L == 0) return AQMP_OK;
     if (((uintptr_t)corr & 15) != 0) return fail(AQMP_E_ARG, "corr must be 16-byte aligned");
