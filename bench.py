@@ -310,7 +310,10 @@ def roofline(name, launches, total_ms, stats_sum, peaks, peak_kind, sm_mhz, max_
             r["separable_flops_per_leaf"] = 4.0 * fam * b ** 3
             r["frac_separable_count"] = 4.0 * fam * b ** 3 * attempts / per_launch_s / 1e12 / peak
             if kind.startswith("corr_septc"):
-                issued = fam * (3 * 4 * 2 * 128 * 64 * 16 + 2 * 96 * 2 * 128 * 32 * 16)
+                # stage 1: 384 digit columns a tile of 128 rows (two leaves at side 64; at 128 a
+                # tile per class of rows and parity of p); stage 2: 1536 columns a 16-wide step
+                issued = fam * ((128 * 384 * 64 + 2 * 2 * 16 * 128 * 1536) if b == 64
+                                else 2 * (4 * 128 * 384 * 128 + 4 * 4 * 16 * 128 * 1536))
                 r["tensor_flops_issued_per_leaf"] = issued
                 r["tensor_pipe_frac"] = issued * attempts / per_launch_s / 1e12 / peak
     else:
