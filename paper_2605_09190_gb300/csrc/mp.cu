@@ -153,6 +153,7 @@ mp_kernel(MPArgs a) {
     // (whole encodes; same bits).
     constexpr bool SPLIT = NF == 2 && T > 32;
     constexpr int FT = SPLIT ? T / 2 : T;    // threads of one family
+    constexpr bool PLAIN = !DF && E <= 16;   // how the FP32 form finds its leader (plain_lead)
     constexpr int NG = NF == 2 && !SPLIT ? 2 : 1;   // families per thread, a summary for each
     constexpr int G = E / NG;
     using At = Atoms<B, FT, G>;
@@ -330,6 +331,46 @@ mp_kernel(MPArgs a) {
             __syncthreads();
             return unpack_lead(sWin[buf]);
         };
+        // The FP32 form's leader needs no second magnitude: the lowest index of
+        // the largest one, its sign below it in one word, so that two reductions
+        // and a single exchange find it.  With the form's one FMA an element the
+        // look-up above costs more than the update: sides 16 and 32 of a 256x384
+        // RGB image take 26 and 94 us with it and 35 and 127 without.  From 32
+        // slots a thread on, the search through all of them costs more than it
+        // saves: side 64, 338 us against 313.
+        auto plain_lead = [&](int buf) {
+            const float top = sm.top();
+            auto key_of = [&](uint32_t M) {
+                uint32_t slot = 0u, sign = 0u;
+#pragma unroll
+                for (int s = E - 1; s >= 0; --s) {
+                    const uint32_t h = __float_as_uint(c.hi(s));
+                    const bool is = (h & 0x7fffffffu) == M;
+                    slot = is ? (uint32_t)s : slot;
+                    sign = is ? h : sign;
+                }
+                return __reduce_min_sync(0xffffffffu, __float_as_uint(top) == M
+                                                          ? 2u * At::atom(abase, (int)slot) + (sign >> 31) : kNone);
+            };
+            uint32_t M, key;
+            if (T == 32) {
+                M = __reduce_max_sync(0xffffffffu, __float_as_uint(top));
+                key = key_of(M);
+            } else {
+                if (dirty) {
+                    wtop = __reduce_max_sync(0xffffffffu, __float_as_uint(top));
+                    wsec = key_of(wtop);
+                }
+                dirty = false;
+                if ((lane & 31) == 0) sPart[buf * NW + warp] = make_uint2(wtop, wsec);
+                __syncthreads();
+                stop = sMisc[8 + buf] != 0u;
+                const uint2 v = (lane & 31) < NW ? sPart[buf * NW + (lane & 31)] : make_uint2(0u, kNone);
+                M = __reduce_max_sync(0xffffffffu, v.x);
+                key = __reduce_min_sync(0xffffffffu, v.x == M ? v.y : kNone);
+            }
+            return Lead{__uint_as_float(M | (key << 31)), 0.0f, key >> 1, 0u};
+        };
         // whether another magnitude reaches the leader's decision window (the
         // FP32 form: the leader)
         auto window_of = [&](float amax) { return DF ? amax * 0x1p-20f + pre : 0.0f; };
@@ -387,12 +428,12 @@ mp_kernel(MPArgs a) {
                 if (accuracy(En)) { conv = true; break; }
                 if (t == k) break;
             }
-            Lead best = group_lead(t & 1);
+            Lead best = PLAIN ? plain_lead(t & 1) : group_lead(t & 1);
             if (T > 32) {
                 if (stop) { conv = true; break; }
                 if (t == k) break;
             }
-            bool exact = contested(best);       // the leader comes from the full words
+            bool exact = !PLAIN && contested(best);   // the leader comes from the full words
             if (__builtin_expect(exact, 0)) best = group_exact();
             if (best.hi == 0.0f) break;         // every correlation is exactly zero
             if constexpr (RESC) {
