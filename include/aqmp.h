@@ -279,7 +279,8 @@ int aqmp_ssim(const float *x, const float *y, int h, int w, int64_t pitch, doubl
  * memory, 16-byte aligned, aqmp_refine_workspace bytes; may be NULL without
  * want_grad) holds intermediate values and may be reused once the stream has
  * passed the call.  All images are h x w FP32 device images of their pitch
- * (elements per row); nothing is synchronised. */
+ * (elements per row), h and w those of the plane (else AQMP_E_ARG); nothing
+ * is synchronised. */
 typedef struct {
     int     plane;
     int     height, width;      /* >= 11 each */

@@ -1504,6 +1504,10 @@ static int check_refine(const aqmp_code *code, const aqmp_refine_plane *planes, 
     for (int i = 0; i < n; ++i) {
         const aqmp_refine_plane &p = planes[i];
         if (p.plane < 0 || p.plane >= (int)code->shapes.size()) return fail(AQMP_E_ARG, "plane %d: no such plane", i);
+        // the synthesis writes and the adjoint reads the whole plane, the SSIM
+        // all of height x width
+        if (p.height != code->shapes[p.plane].first || p.width != code->shapes[p.plane].second)
+            return fail(AQMP_E_ARG, "plane %d: %d x %d is not the plane's size", i, p.height, p.width);
         if (p.height < 11 || p.width < 11) return fail(AQMP_E_ARG, "plane %d: smaller than the SSIM window", i);
     }
     return AQMP_OK;
@@ -1531,10 +1535,8 @@ int aqmp_refine_forward(const aqmp_code *code, const float *alpha, const aqmp_re
     std::vector<int64_t> pitch(n);
     for (int i = 0; i < n; ++i) {
         const aqmp_refine_plane &p = planes[i];
-        const int w = code->shapes[p.plane].second;
-        if (p.height < code->shapes[p.plane].first) return fail(AQMP_E_ARG, "plane %d: fewer rows than the plane", i);
         if (!p.ref || !p.recon || (want_grad && !p.grad)) return fail(AQMP_E_ARG, "plane %d: NULL image", i);
-        if (p.ref_pitch < p.width || p.recon_pitch < std::max(w, p.width) || (want_grad && p.grad_pitch < p.width))
+        if (p.ref_pitch < p.width || p.recon_pitch < p.width || (want_grad && p.grad_pitch < p.width))
             return fail(AQMP_E_ARG, "plane %d: pitch below width", i);
         id[i] = p.plane;
         recon[i] = p.recon;
@@ -1572,7 +1574,7 @@ int aqmp_refine_backward(const aqmp_code *code, const aqmp_refine_plane *planes,
     std::vector<float *> grad(n);
     std::vector<int64_t> pitch(n);
     for (int i = 0; i < n; ++i) {
-        if (!planes[i].grad || planes[i].grad_pitch < code->shapes[planes[i].plane].second)
+        if (!planes[i].grad || planes[i].grad_pitch < planes[i].width)
             return fail(AQMP_E_ARG, "plane %d: bad gradient image", i);
         id[i] = planes[i].plane;
         grad[i] = planes[i].grad;
