@@ -28,6 +28,7 @@ class SynthesisSSIM(torch.autograd.Function):
         # go through one launch of each kernel.
         want = ctx.needs_input_grad[0]
         dev = alpha.device
+        refs = list(refs)                        # walked several times
         at = [0]
         for _, ref in refs:
             at.append(at[-1] + ref.shape[0] * ref.shape[1])
