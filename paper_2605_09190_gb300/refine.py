@@ -4,8 +4,7 @@ synthesis + SSIM).
 The support -- leaves and atom indices of an encode -- is held fixed and the
 coefficients are refined by gradient ascent on the mean SSIM (Section 3) of
 the synthesised planes (Algorithm 3).  Forward and backward both run in the
-library's kernels (`aqmp_synth_forward` / `aqmp_synth_backward` /
-`aqmp_ssim`); this module only wraps them as a torch.autograd.Function.  The
+library's kernels (`aqmp_refine_forward` / `aqmp_refine_backward`); this module only wraps them as a torch.autograd.Function.  The
 loss uses the unclipped reconstruction (the clip of the reported metric has
 no useful gradient where it saturates).
 """
@@ -41,16 +40,23 @@ class SynthesisSSIM(torch.autograd.Function):
         ssim = torch.empty(len(refs), dtype=torch.float64, device=dev)
         work = torch.empty(aqmp.aqmp_refine_workspace(planes), dtype=torch.uint8, device=dev) if want else None
         aqmp.aqmp_refine_forward(code, alpha, planes, ssim, work)
-        ctx.code, ctx.planes, ctx.images = code, planes, grad
+        # for the backward: the gradient images and where each plane's is (the
+        # synthesis, the workspace and the references are not kept)
+        ctx.code, ctx.images = code, grad
+        ctx.sizes = [(plane, ref.shape[0], ref.shape[1]) for plane, ref in refs]
         ctx.n_alpha = alpha.shape[0]
         return ssim.mean()
 
     @staticmethod
     def backward(ctx, grad):
         grad_alpha = torch.zeros(ctx.n_alpha, dtype=torch.float32, device=grad.device)
-        aqmp.aqmp_refine_backward(ctx.code, ctx.planes, grad_alpha)
+        rows, at = [], ctx.images.data_ptr()
+        for plane, h, w in ctx.sizes:
+            rows.append((plane, h, w, None, 0, None, 0, at, w))
+            at += 4 * h * w
+        aqmp.aqmp_refine_backward(ctx.code, aqmp.aqmp_refine_planes(rows), grad_alpha)
         # the mean over planes and the upstream gradient, on the device
-        return grad_alpha * (grad / len(ctx.planes)).to(torch.float32), None, None
+        return grad_alpha * (grad / len(ctx.sizes)).to(torch.float32), None, None
 
 
 def synthesis_ssim(alpha, code, refs):

@@ -1,5 +1,6 @@
 """What the refinement's autograd function hands to the library, with stand-ins
-for the library's calls: references that can be walked once only."""
+for the library's calls: references that can be walked once only, and in the
+backward no address but those of the gradient images it keeps."""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -37,3 +38,16 @@ def test_references_may_come_from_a_generator(calls, grad):
     if grad:
         s.backward()
         assert torch.equal(alpha.grad, torch.full((5,), 1.5))
+
+
+def test_backward_keeps_no_address_of_the_forward(calls):
+    from paper_2605_09190_gb300 import refine
+    alpha = torch.zeros(5, requires_grad=True)
+    images = [torch.zeros(16, 24), torch.zeros(32, 16)]
+    s = refine.synthesis_ssim(alpha, None, list(enumerate(images)))
+    kept = s.grad_fn.images                                    # alive until the backward
+    s.backward()
+    # plane, height, width, reference, pitch, synthesis, pitch, gradient, pitch
+    at = kept.data_ptr()
+    assert calls["backward"] == [(0, 16, 24, None, 0, None, 0, at, 24), (1, 32, 16, None, 0, None, 0, at + 4 * 16 * 24, 16)]
+    assert not hasattr(s.grad_fn, "planes")
