@@ -637,12 +637,13 @@ def decompress(blob: bytes, stream=None):
     an (h, w, C) uint8 CUDA tensor."""
     import torch
     data = zlib.decompress(blob)
+    info, shapes = _bitstream_head(data)
+    if len(set(shapes)) != 1:
+        aqmp_bitstream_parse(data)                       # a malformed body comes first
+        raise ValueError("planes of different sizes do not form one image")
+    h, w = shapes[0]
     code = aqmp_code_from_bitstream(data)                # the one parse of the leaves and atoms
     try:
-        info, shapes = _bitstream_head(data)
-        if len(set(shapes)) != 1:
-            raise ValueError("planes of different sizes do not form one image")
-        h, w = shapes[0]
         planes = torch.empty((info["n_planes"], h, w), dtype=torch.float32, device="cuda")
         for c in range(info["n_planes"]):
             aqmp_decode(code, c, planes[c], stream)
