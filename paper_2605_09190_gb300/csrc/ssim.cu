@@ -15,7 +15,7 @@
 // window.
 //
 // Everything is double-float (~2^-46 relative, so that E[s] - mu^2 keeps the
-// variance) on the packed FP32 pipes: GB300's FP64 rate is 1/64 of its FP32
+// variance; pixels beyond any image's take the window formula in FP64) on the packed FP32 pipes: GB300's FP64 rate is 1/64 of its FP32
 // rate, and the window formula in FP64 alone took a third of the former
 // window pass.  An 11-tap pass keeps each sum as (s, c): s the running FP32
 // sum, c the sum of the exact errors of its products and additions and of the
@@ -81,6 +81,31 @@ __device__ __forceinline__ df df_recip(df d) {
 }
 
 __device__ __forceinline__ df twice(df a) { return df_scale(a, 2.0f); }
+
+__host__ __device__ __forceinline__ df df_split(double v) {
+    const float hi = (float)v;
+    return df{hi, (float)(v - (double)hi)};
+}
+
+// A window's value and partials.
+struct Window {
+    df f, my, yy, xy;
+};
+
+// ... from its means in FP64, where 1 / (B1 B2) and its low word would leave
+// the range of FP32: E[x^2 + y^2] above 2^48, pixels of 10^7 and more.  Out of
+// line, since no image has such pixels (a refinement that diverges does).
+__device__ __noinline__ void window_fp64(df mx_, df my_, df es_, df exy_, Window *out) {
+    const double mx = df_to_double(mx_), my = df_to_double(my_), es = df_to_double(es_), exy = df_to_double(exy_);
+    const double C1 = (0.01 * 255.0) * (0.01 * 255.0), C2 = (0.03 * 255.0) * (0.03 * 255.0);
+    const double mxy = mx * my, mm = mx * mx + my * my;
+    const double A1 = 2.0 * mxy + C1, A2 = 2.0 * (exy - mxy) + C2, iB1 = 1.0 / (mm + C1), iB2 = 1.0 / ((es - mm) + C2);
+    const double t1 = A2 * iB1 * iB2, t2 = A1 * iB1 * iB2, f = A1 * t1;          // f / A1, f / A2
+    out->f = df_split(f);
+    out->my = df_split(2.0 * mx * (t1 - t2) - 2.0 * my * f * (iB1 - iB2));
+    out->yy = df_split(-f * iB2);
+    out->xy = df_split(2.0 * t2);
+}
 
 // The plane of this CTA's tile, and the tile's place in it.
 __device__ __forceinline__ const SsimPlane &find_plane(const SsimArgs &a, int &ty, int &tx) {
@@ -182,20 +207,30 @@ __global__ void __launch_bounds__(kThreads, 2) ssim_forward_kernel(const __grid_
         if (row + o >= T::TH || r >= ho || c >= wo) continue;
         const df mx = join(f2_x(m[o].s), f2_x(m[o].c)), my = join(f2_y(m[o].s), f2_y(m[o].c));
         const df es = join(f2_x(p[o].s), f2_x(p[o].c)), exy = join(f2_y(p[o].s), f2_y(p[o].c));
-        const df mxy = df_mul(mx, my), mm = df_add(df_mul(mx, mx), df_mul(my, my));
-        const df A1 = df_add(twice(mxy), a.c1), A2 = df_add(twice(df_sub(exy, mxy)), a.c2);
-        const df B1 = df_add(mm, a.c1), B2 = df_add(df_sub(es, mm), a.c2);
-        const df q = df_recip(df_mul(B1, B2));
-        const df t1 = df_mul(A2, q), t2 = df_mul(A1, q);               // f / A1, f / A2
-        const df f = df_mul(A1, t1);
-        sum = df_add(sum, f);
+        Window v;
+        if (__builtin_expect(!(es.hi <= 0x1p48f), 0)) {
+            Window big;
+            window_fp64(mx, my, es, exy, &big);
+            v = big;
+        } else {
+            const df mxy = df_mul(mx, my), mm = df_add(df_mul(mx, mx), df_mul(my, my));
+            const df A1 = df_add(twice(mxy), a.c1), A2 = df_add(twice(df_sub(exy, mxy)), a.c2);
+            const df B1 = df_add(mm, a.c1), B2 = df_add(df_sub(es, mm), a.c2);
+            const df q = df_recip(df_mul(B1, B2));
+            const df t1 = df_mul(A2, q), t2 = df_mul(A1, q);           // f / A1, f / A2
+            v.f = df_mul(A1, t1);
+            if (P.P4) {
+                const df iB1 = df_mul(B2, q), iB2 = df_mul(B1, q);
+                v.my = df_sub(df_mul(twice(mx), df_sub(t1, t2)), df_mul(df_mul(twice(my), v.f), df_sub(iB1, iB2)));
+                v.yy = df_neg(df_mul(v.f, iB2));
+                v.xy = twice(t2);
+            }
+        }
+        sum = df_add(sum, v.f);
         if (P.P4) {
-            const df iB1 = df_mul(B2, q), iB2 = df_mul(B1, q);
-            const df fmy = df_sub(df_mul(twice(mx), df_sub(t1, t2)), df_mul(df_mul(twice(my), f), df_sub(iB1, iB2)));
-            const df fyy = df_neg(df_mul(f, iB2));
             const long long at = (long long)r * wo + c;
-            P.P4[at] = make_float4(fmy.hi, fyy.hi, fmy.lo, fyy.lo);
-            P.P2[at] = make_float2(2.0f * t2.hi, 2.0f * t2.lo);
+            P.P4[at] = make_float4(v.my.hi, v.yy.hi, v.my.lo, v.yy.lo);
+            P.P2[at] = make_float2(v.xy.hi, v.xy.lo);
         }
     }
     // block sum, one atomic per block
@@ -318,11 +353,6 @@ __global__ void __launch_bounds__(kThreads, 2) ssim_backward_kernel(const __grid
         t = df_mul(t, P.scale);
         P.grad[(long long)r * P.grad_pitch + c] = __fadd_rn(t.hi, t.lo);
     }
-}
-
-df df_split(double v) {
-    const float hi = (float)v;
-    return df{hi, (float)(v - (double)hi)};
 }
 
 f2 f2_both(float v) {
