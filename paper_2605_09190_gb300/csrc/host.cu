@@ -1471,7 +1471,9 @@ static void ssim_plane(SsimPlane &p, const float *x, int64_t x_pitch, const floa
     p.sum = sum;
     if (!grad) return;
     const size_t wins = (size_t)(h - 10) * (w - 10);
-    const double scale = grad_scale / (double)wins;
+    // as a fraction and a power of two: the factor may lie outside FP32 where
+    // the gradient does not
+    const double scale = std::frexp(grad_scale / (double)wins, &p.scale_exp);
     p.grad = grad;
     p.grad_pitch = grad_pitch;
     p.scale.hi = (float)scale;

@@ -214,7 +214,8 @@ struct SsimPlane {
     float *grad;
     long long x_pitch, y_pitch, grad_pitch;
     int h, w;
-    df scale;                    // of the gradient
+    df scale;                    // of the gradient, times 2^scale_exp
+    int scale_exp;
     float4 *P4;                  // [(h-10)(w-10)] per-window partials f_my, f_Eyy (high words, low words)
     float2 *P2;                  // [(h-10)(w-10)] f_Exy
     double *sum;

@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(kThreads, 2) ssim_backward_kernel(const __grid
         t = df_sub_mul(t, df{-2.0f * yv, 0.0f}, join(f2_y(m[o].s), f2_y(m[o].c)));
         t = df_sub_mul(t, df{-xv, 0.0f}, join(q[o].s, q[o].c));
         t = df_mul(t, P.scale);
-        P.grad[(long long)r * P.grad_pitch + c] = __fadd_rn(t.hi, t.lo);
+        P.grad[(long long)r * P.grad_pitch + c] = ldexpf(__fadd_rn(t.hi, t.lo), P.scale_exp);
     }
 }
 
@@ -380,7 +380,7 @@ cudaError_t launch_tiles(SsimArgs &a, bool pixels, K kern, cudaStream_t st) {
 }  // namespace
 
 // a.p[i]: x, y, pitches, h, w, sum (zeroed), and with `grad` also grad, scale,
-// P4 and P2; n <= kRefinePlanes.
+// scale_exp, P4 and P2; n <= kRefinePlanes.
 cudaError_t launch_ssim(SsimArgs &a, bool grad, int num_sms, cudaStream_t st) {
     double g[11], s = 0.0;
     for (int i = 0; i < 11; ++i) {

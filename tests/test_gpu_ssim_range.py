@@ -1,6 +1,7 @@
 """The SSIM and its gradient for pixels far beyond any image's, as a refinement
 that diverges meets them: as accurate as inside, up to where the squares of the
-pixels leave FP32.  Reference: the same formula in FP64."""
+pixels leave FP32; and gradients scaled by factors that FP32 does not hold.
+Reference: the same formula in FP64."""
 import numpy as np
 import pytest
 
@@ -49,3 +50,16 @@ def test_pixels_beyond_images(lib, peak):
     # ... and the sum of three terms, rounded to FP32, each at most 50 times the largest gradient
     err = np.abs(grad.cpu().numpy().astype(np.float64) - want_grad).max()
     assert err <= 2.0 ** -23 * np.abs(want_grad).max()
+
+
+@pytest.mark.parametrize("scale", [1.0, -3.0, 3e42, 1e-30, -1e-41, 0.0])
+def test_scaled_gradients(lib, scale):
+    rng = np.random.default_rng(6)
+    x = torch.from_numpy(rng.uniform(0.0, 255.0, (64, 64)).astype(np.float32)).cuda()
+    y = torch.from_numpy(rng.uniform(0.0, 255.0, (64, 64)).astype(np.float32)).cuda()
+    s, grad = torch.zeros((), dtype=torch.float64, device="cuda"), torch.empty_like(y)
+    lib.aqmp_ssim(x, y, s, grad, scale)
+    want = reference(x, y)[1] * scale
+    assert np.abs(want).max() < np.finfo(np.float32).max
+    err = np.abs(grad.cpu().numpy().astype(np.float64) - want).max()
+    assert err <= 2.0 ** -23 * np.abs(want).max() + 2.0 ** -149      # the last: the spacing of the smallest FP32 numbers
