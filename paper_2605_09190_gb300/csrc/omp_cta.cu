@@ -30,8 +30,10 @@
 // so that K g (a thread per row; g is zero on the new atom's own family) and
 // w^T K (a thread per column) both read contiguously; each CTA takes a share
 // of the rows and of the columns and the results meet through distributed
-// shared memory: three cluster barriers a step.
-// A 256x256 image of 64x64 roots (16 leaves, 1285 atoms): 66.8 -> 7.69 ms;
+// shared memory: three cluster barriers a step.  Every sum is formed in an order
+// that the support alone fixes, so the coefficients have the same bits at every
+// width of the cluster.
+// A 256x256 image of 64x64 roots (16 leaves, 1285 atoms): 66.8 -> 7.05 ms;
 // 1024x640 (160 leaves, one CTA each): 13.8 -> 11.4 ms; a 512x512 plane at
 // four tolerances down to side 4, up to 1024 atoms a leaf: 884 -> 551 ms.
 #include <cuda_runtime.h>
@@ -110,6 +112,53 @@ __device__ __forceinline__ void put_all(double *p, double v) {
     for (uint32_t r = 0; r < (uint32_t)C; ++r) put(p, r, v);
 }
 
+// How many partial sums a row's or a column's product with the factor is formed
+// as, given the 32-row blocks of the support: by its size alone, and joined as
+// a tree over neighbours, so that a leaf's coefficients have the same bits
+// whatever the cluster's width (how many leaves share the call, which GPU runs
+// it).  As many as the warps a block gets at the widest cluster.
+constexpr int kMaxBlocks = kMaxBudget / 32;
+__device__ __forceinline__ int parts_of(int blocks) { return blocks <= 8 ? 8 : blocks <= 16 ? 4 : 2; }
+static_assert(kWarps == 8 && kMaxBlocks <= 32, "partial sums, one block a lane");
+
+// p[0] .. p[(n - 1) stride], n a power of two up to 8, joined as that tree.
+__device__ __forceinline__ double join_tree(const double *p, int stride, int n) {
+    double v = p[0];
+    if (n >= 2) v += p[stride];
+    if (n >= 4) v += p[2 * stride] + p[3 * stride];
+    if (n >= 8) v += (p[4 * stride] + p[5 * stride]) + (p[6 * stride] + p[7 * stride]);
+    return v;
+}
+
+// Partial sums at, at + 1 .. at + m - 1 of `of` (a power of two; m one too) of
+// the terms first .. count - 1, partial s taking first + s, first + s + of ...,
+// joined: term(i, sum) adds term i.
+template <int MP, class Term>
+__device__ __forceinline__ double partial_sums_n(int first, int count, int at, int of, Term term) {
+    double p[MP];
+#pragma unroll
+    for (int e = 0; e < MP; ++e) p[e] = 0.0;
+#pragma unroll(MP >= 4 ? 1 : 4 / MP)
+    for (int i = first + at; i < count; i += of) {
+#pragma unroll
+        for (int e = 0; e < MP; ++e)
+            if (i + e < count) p[e] = term(i + e, p[e]);
+    }
+#pragma unroll
+    for (int w = 1; w < MP; w *= 2)
+#pragma unroll
+        for (int e = 0; e + w < MP; e += 2 * w) p[e] += p[e + w];
+    return p[0];
+}
+
+template <class Term>
+__device__ __forceinline__ double partial_sums(int first, int count, int at, int m, int of, Term term) {
+    if (m == 1) return partial_sums_n<1>(first, count, at, of, term);
+    if (m == 2) return partial_sums_n<2>(first, count, at, of, term);
+    if (m == 4) return partial_sums_n<4>(first, count, at, of, term);
+    return partial_sums_n<8>(first, count, at, of, term);
+}
+
 // What one CTA offers to the step's choice.
 struct Offer {
     double amax;               // its largest |c|
@@ -134,7 +183,7 @@ struct OmpLayout {
     static constexpr int wp = 0, wpt = wp + (NF == 2 ? B * NP : 0), wq = wpt + (NF == 2 ? B * NP : 0),
                          wtq = wq + (NF == 2 ? B * Q : 0), vv = wtq + (NF == 2 ? B * Q : 0),
                          uu = vv + (NF == 2 ? B * Q : 0), red = uu + (NF == 2 ? B * Q : 0),
-                         offers = red + 2 * kWarps, sums = offers + 4 * C, claim = sums + 2 * C, part = claim + 2,
+                         offers = red + 2 * kWarps, sums = offers + 4 * C, claim = sums + 2 * kMaxBlocks, part = claim + 2,
                          arrays = part + kThreads;
     __host__ __device__ static constexpr size_t doubles(int k) { return (size_t)arrays + 4 * (size_t)k; }
     // words: the support's atoms, their predecessors in their row, the positions by family; row heads; misc
@@ -170,7 +219,7 @@ __global__ void __launch_bounds__(kThreads, 1) omp_cta_kernel(MPArgs a) {
     double *V = sm + Ly::vv, *U = sm + Ly::uu;         // [row][q]
     double *red = sm + Ly::red;
     Offer *offers = reinterpret_cast<Offer *>(sm + Ly::offers);
-    double *sums = sm + Ly::sums;                      // [C][2]
+    double *sums = sm + Ly::sums;                      // [block of 32 rows][2]: |w|^2 and w . z
     double *part = sm + Ly::part;
     const int k = a.lv.k;
     double *xs = sm + Ly::arrays, *zs = xs + k, *gs = zs + k, *wv = gs + k;
@@ -437,49 +486,36 @@ __global__ void __launch_bounds__(kThreads, 1) omp_cta_kernel(MPArgs a) {
                 __syncthreads();
                 const int others = haar ? nC : nH;
                 const int blocks = (nS + 31) / 32, own = (blocks - rank + C - 1) / C;     // blocks of this CTA
+                const int parts = parts_of(blocks);
                 for (int b0 = 0; b0 < own; b0 += kWarps) {
-                    const int nb = min(kWarps, own - b0), split = kWarps / nb;            // warps per block
-                    const int ib = warp % nb, is = warp / nb;
-                    const int r = ((b0 + ib) * C + rank) * 32 + lane;
+                    const int nb = min(kWarps, own - b0);
+                    const int split = min(parts, nb == 1 ? 8 : nb == 2 ? 4 : nb <= 4 ? 2 : 1);   // warps per block
+                    const int ib = warp % nb, is = warp / nb, block = (b0 + ib) * C + rank;
+                    const int r = block * 32 + lane;
                     double w = 0.0;
                     if (is < split)
-                        for (int i = is; i < others; i += split) {
+                        w = partial_sums(0, others, is * (parts / split), parts / split, parts, [&](int i, double v) {
                             const int at = (int)fam_pos[haar ? i : k - 1 - i];
-                            if (r >= at && r < nS) w = fma(__ldcg(Kc + (size_t)at * k + r), gs[at], w);
-                        }
+                            return r >= at && r < nS ? fma(__ldcg(Kc + (size_t)at * k + r), gs[at], v) : v;
+                        });
                     part[tid] = w;
                     __syncthreads();
-                    if (is == 0 && r < nS) {
-                        for (int s = 1; s < split; ++s) w += part[(s * nb + ib) * 32 + lane];
-                        put_all<C>(wv + r, w);
-                        ww = fma(w, w, ww);
-                        wz = fma(w, zs[r], wz);
+                    if (is == 0) {
+                        w = join_tree(part + ib * 32 + lane, nb * 32, split);
+                        if (r < nS) put_all<C>(wv + r, w);
+                        ww = warp_sum(w * w);
+                        wz = warp_sum(r < nS ? w * zs[r] : 0.0);
+                        if (lane == 0) {
+                            put_all<C>(sums + 2 * block, ww);
+                            put_all<C>(sums + 2 * block + 1, wz);
+                        }
                     }
                     __syncthreads();
                 }
-                ww = warp_sum(ww);
-                wz = warp_sum(wz);
-                if (lane == 0) {
-                    red[warp] = ww;
-                    red[kWarps + warp] = wz;
-                }
-                __syncthreads();
-                if (tid == 0) {
-                    ww = wz = 0.0;
-                    for (int i = 0; i < kWarps; ++i) {
-                        ww += red[i];
-                        wz += red[kWarps + i];
-                    }
-                    put_all<C>(sums + 2 * rank, ww);
-                    put_all<C>(sums + 2 * rank + 1, wz);
-                }
                 cluster_sync<C>();
-                ww = wz = 0.0;
-#pragma unroll
-                for (int r = 0; r < C; ++r) {
-                    ww += sums[2 * r];
-                    wz += sums[2 * r + 1];
-                }
+                // a block a lane: the same tree on every warp of the cluster
+                ww = warp_sum(lane < blocks ? sums[2 * lane] : 0.0);
+                wz = warp_sum(lane < blocks ? sums[2 * lane + 1] : 0.0);
             }
             const double d = 1.0 - ww;
             if (d > kPivotMin * 0x1p-4 && d < kPivotMin * 0x1p4) tie = true;
@@ -491,21 +527,21 @@ __global__ void __launch_bounds__(kThreads, 1) omp_cta_kernel(MPArgs a) {
             // blocks of 32 lanes as the rows above
             {
                 const int cols = nS + 1, blocks = (cols + 31) / 32, own = (blocks - rank + C - 1) / C;
+                const int parts = parts_of(blocks);
                 for (int b0 = 0; b0 < own; b0 += kWarps) {
-                    const int nb = min(kWarps, own - b0), split = kWarps / nb;
-                    const int ib = warp % nb, is = warp / nb;
-                    const int c = ((b0 + ib) * C + rank) * 32 + lane;
+                    const int nb = min(kWarps, own - b0);
+                    const int split = min(parts, nb == 1 ? 8 : nb == 2 ? 4 : nb <= 4 ? 2 : 1);
+                    const int ib = warp % nb, is = warp / nb, first = ((b0 + ib) * C + rank) * 32;
+                    const int c = first + lane;
                     double v = 0.0;
-                    if (NF == 2 && is < split) {
-                        const int first = ((b0 + ib) * C + rank) * 32;
-#pragma unroll 4
-                        for (int i = first + is; i < nS; i += split)
-                            if (c <= i) v = fma(wv[i], __ldcg(Kr + tri64(i) + c), v);
-                    }
+                    if (NF == 2 && is < split)
+                        v = partial_sums(first, nS, is * (parts / split), parts / split, parts, [&](int i, double u) {
+                            return c <= i ? fma(wv[i], __ldcg(Kr + tri64(i) + c), u) : u;
+                        });
                     part[tid] = v;
                     __syncthreads();
                     if (is == 0 && c <= nS) {
-                        for (int s = 1; s < split; ++s) v += part[(s * nb + ib) * 32 + lane];
+                        v = join_tree(part + ib * 32 + lane, nb * 32, split);
                         v = c == nS ? rd : -v * rd;
                         __stcg(Kr + tri64(nS) + c, v);
                         __stcg(Kc + (size_t)c * k + nS, v);
@@ -655,7 +691,7 @@ static cudaError_t launch_omp_cta_t(const MPArgs &a, cudaStream_t st) {
         return cudaErrorInvalidValue;
     if constexpr (NF == 2) {
         // omp_slots = the device's SMs.  A step's products shrink with C and
-        // its barriers and chains do not: 16 leaves of side 64 take 7.69, 11.2,
+        // its barriers and chains do not: 16 leaves of side 64 take 7.05, 11.2,
         // 18.7 and 33.3 ms with 8, 4, 2 CTAs and one, 64 leaves 8.0 with two
         // against 14.5 with one.  More CTAs than SMs would queue whole leaves
         const long long leaves = a.lv.capacity;
