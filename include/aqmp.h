@@ -107,8 +107,11 @@ extern "C" {
                                       64 keep the inverse Cholesky factor of
                                       each leaf in flight (at most one per SM)
                                       in device memory, by rows and by columns:
-                                      k(k+1)/2 + k^2 doubles (12.6 MB at
-                                      k = 1024). */
+                                      k(k+1) doubles (8.4 MB at k = 1024).
+                                      Where the device has no room for all of
+                                      them, fewer leaves are in flight.  The
+                                      coefficients of a leaf depend on neither
+                                      this nor on the other leaves of the call. */
 /* Autotuning: kernel choices that leave the result unchanged bit for bit
  * are measured on the first calls of each configuration and the fastest
  * is kept for the life of the process: the initial correlation on the

@@ -205,6 +205,22 @@ struct DeviceBuf {
         bytes = want;
         return AQMP_OK;
     }
+    // `want` bytes where the device has them, else half of that and so on, at
+    // least `least`; what is there stays while the device could not double it.
+    int reserve_up_to(size_t want, size_t least) {
+        if (want <= bytes) return AQMP_OK;
+        size_t avail = 0, total = 0;
+        if (bytes >= least && cudaMemGetInfo(&avail, &total) == cudaSuccess && avail < bytes) return AQMP_OK;
+        for (;; want /= 2) {
+            const int rc = reserve(std::max(want, least));
+            if (rc == AQMP_OK) {
+                g_last_error.clear();
+                return AQMP_OK;
+            }
+            (void)cudaGetLastError();                    // the failed allocation's
+            if (want <= least) return rc;
+        }
+    }
 };
 
 // ------------------------------------------------------ kernel timing
@@ -886,16 +902,18 @@ int aqmp_encode_planes(const aqmp_params *params, const aqmp_plane *planes, int 
     CK(cudaMallocFromPoolAsync((void **)&code->alpha_lo, sizeof(float) * std::max<unsigned long long>(1, atom_cap),
                                c->out_pool, st));
     if ((rc = c->counters.reserve(sizeof(Counters)))) return rc;
-    // OMP at sides 32 and 64: the inverse factor of each leaf in flight
-    unsigned long long omp_doubles = 0;
+    // OMP at sides 32 and 64: the inverse factor of each leaf in flight; where
+    // the device has no room for all of them, fewer leaves at a time
+    unsigned long long omp_doubles = 0, omp_least = 0;
     if (omp)
         for (int l = 0; l < nlev; ++l) {
             const int b = P.max_block >> l;
             if (b < 32) continue;
             const int kb = (int)std::max<long long>(1, (long long)b * b * P.cap_num / P.cap_den);
             omp_doubles = std::max(omp_doubles, omp_cta_workspace_doubles(kb, c->num_sms, cap[l]));
+            omp_least = std::max(omp_least, omp_cta_slot_doubles(kb));
         }
-    if (omp_doubles && (rc = c->omp_L.reserve(sizeof(double) * omp_doubles))) return rc;
+    if (omp_doubles && (rc = c->omp_L.reserve_up_to(sizeof(double) * omp_doubles, sizeof(double) * omp_least))) return rc;
 
     // plane descriptors (and host pixels copied in)
     std::vector<PlaneDesc> pd(n_planes);
@@ -1076,8 +1094,8 @@ int aqmp_encode_planes(const aqmp_params *params, const aqmp_plane *planes, int 
         ma.cells = cells;
         ma.ctr = ctr;
         ma.omp_L = (double *)c->omp_L.p;
-        ma.omp_slots = c->num_sms;
-        ma.omp_L_doubles = omp_doubles;
+        ma.omp_sms = c->num_sms;
+        ma.omp_L_doubles = c->omp_L.bytes / sizeof(double);
         ma.fam0 = d.fam0;
         if (resc_l) {
             ma.ebound = (const float *)c->ebound.p;

@@ -25,11 +25,11 @@ struct MPArgs {
     unsigned long long atom_cap;
     CellMap cells;               // emitted leaves are marked here
     Counters *ctr;
-    // OMP at sides 32 and 64: the inverse factor of a leaf in flight, by rows
-    // (packed) and by columns; omp_slots is the device's SMs, the most leaves
-    // in flight (omp_L_doubles in all, see omp_cta_workspace_doubles)
+    // OMP at sides 32 and 64: the inverse factor of each leaf in flight, by rows
+    // and by columns, as many as omp_L_doubles hold (omp_cta_slot_doubles each)
+    // and as the device has SMs
     double *omp_L;
-    int omp_slots;
+    int omp_sms;
     unsigned long long omp_L_doubles;
     // the BF16 form with rescore (side 64; ebound NULL: off): the BF16
     // correlation's per-atom bounds, the leaves' mean-centred pixels and their
@@ -63,6 +63,7 @@ cudaError_t launch_mp_cluster(const MPArgs &a, int nf, bool double_float, int nu
 // served); same arguments and outputs as the MP kernel (the coefficients
 // emitted are the final least-squares values).
 int omp_max_budget(int b);
+unsigned long long omp_cta_slot_doubles(int k);                  // a leaf in flight
 unsigned long long omp_cta_workspace_doubles(int k, int sms, unsigned long long leaves);
 cudaError_t launch_omp(const MPArgs &a, int nf, int num_sms, cudaStream_t st);
 int omp_cta_max_budget();

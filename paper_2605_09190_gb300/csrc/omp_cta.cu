@@ -54,8 +54,10 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kMaxBudget = 1024;
 
 __host__ __device__ __forceinline__ long long tri64(long long i) { return i * (i + 1) / 2; }
-// Doubles of a slot: K by rows (packed) and by columns (k x k).
-__host__ __device__ __forceinline__ long long slot_doubles(long long k) { return tri64(k) + k * k; }
+// Doubles of a slot: K by rows and by columns, both packed.
+__host__ __device__ __forceinline__ long long slot_doubles(long long k) { return 2 * tri64(k); }
+// Where row 0 of column c of K would be in the packed columns (its rows are c .. k - 1).
+__device__ __forceinline__ int column_at(int c, int k) { return c * (2 * k - c - 1) / 2; }
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -496,7 +498,7 @@ __global__ void __launch_bounds__(kThreads, 1) omp_cta_kernel(MPArgs a) {
                     if (is < split)
                         w = partial_sums(0, others, is * (parts / split), parts / split, parts, [&](int i, double v) {
                             const int at = (int)fam_pos[haar ? i : k - 1 - i];
-                            return r >= at && r < nS ? fma(__ldcg(Kc + (size_t)at * k + r), gs[at], v) : v;
+                            return r >= at && r < nS ? fma(__ldcg(Kc + column_at(at, k) + r), gs[at], v) : v;
                         });
                     part[tid] = w;
                     __syncthreads();
@@ -544,7 +546,7 @@ __global__ void __launch_bounds__(kThreads, 1) omp_cta_kernel(MPArgs a) {
                         v = join_tree(part + ib * 32 + lane, nb * 32, split);
                         v = c == nS ? rd : -v * rd;
                         __stcg(Kr + tri64(nS) + c, v);
-                        __stcg(Kc + (size_t)c * k + nS, v);
+                        __stcg(Kc + column_at(c, k) + nS, v);
                         put_all<C>(xs + c, c == nS ? zn * v : fma(zn, v, xs[c]));
                     }
                     __syncthreads();
@@ -641,15 +643,17 @@ __global__ void __launch_bounds__(kThreads, 1) omp_cta_kernel(MPArgs a) {
     }
 }
 
+unsigned long long omp_cta_slot_doubles(int k) { return k < 1 ? 0ull : (unsigned long long)slot_doubles(k); }
+
 // A slot per cluster: as many as there are SMs or leaves.
 unsigned long long omp_cta_workspace_doubles(int k, int sms, unsigned long long leaves) {
     const unsigned long long slots = leaves < (unsigned long long)sms ? leaves : (unsigned long long)sms;
-    return k < 1 ? 0ull : slots * (unsigned long long)slot_doubles(k);
+    return slots * omp_cta_slot_doubles(k);
 }
 
 // C CTAs a leaf: the most that the level's leaves leave SMs for.
 template <int B, int NF, int C>
-static cudaError_t launch_omp_cta_c(const MPArgs &a, cudaStream_t st) {
+static cudaError_t launch_omp_cta_c(const MPArgs &a, long long leaves, cudaStream_t st) {
     const int k = a.lv.k;
     const size_t bytes = OmpLayout<B, NF, C>::bytes(k);
     auto kern = omp_cta_kernel<B, NF, C>;
@@ -667,18 +671,16 @@ static cudaError_t launch_omp_cta_c(const MPArgs &a, cudaStream_t st) {
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = C > 1 ? 1 : 0;
-    long long clusters = a.omp_slots;
+    long long clusters = leaves;
     if (C > 1) {
         int most = 0;
         e = cudaOccupancyMaxActiveClusters(&most, kern, &cfg);
         if (e != cudaSuccess) return e;
         if constexpr (C > 1) {
-            if (most < 1) return launch_omp_cta_c<B, NF, C / 2>(a, st);      // no room for a cluster this wide
+            if (most < 1) return launch_omp_cta_c<B, NF, C / 2>(a, leaves, st);      // no room for a cluster this wide
         }
         if (most < clusters) clusters = most;
     }
-    if ((long long)a.lv.capacity < clusters) clusters = a.lv.capacity;
-    if (clusters < 1) clusters = 1;
     cfg.gridDim = dim3((unsigned)(clusters * C), 1, 1);
     return cudaLaunchKernelEx(&cfg, kern, a);
 }
@@ -686,20 +688,23 @@ static cudaError_t launch_omp_cta_c(const MPArgs &a, cudaStream_t st) {
 template <int B, int NF>
 static cudaError_t launch_omp_cta_t(const MPArgs &a, cudaStream_t st) {
     const int k = a.lv.k;
-    if (k < 1 || k > kMaxBudget || !a.omp_L || a.omp_slots < 1 ||
-        a.omp_L_doubles < omp_cta_workspace_doubles(k, a.omp_slots, a.lv.capacity))
+    if (k < 1 || k > kMaxBudget || !a.omp_L || a.omp_sms < 1 || a.omp_L_doubles < omp_cta_slot_doubles(k))
         return cudaErrorInvalidValue;
+    // the most leaves in flight: those there are, one an SM, one a slot
+    const long long slots = (long long)(a.omp_L_doubles / omp_cta_slot_doubles(k));
+    long long leaves = a.lv.capacity < 1u ? 1 : (long long)a.lv.capacity;
+    if (leaves > a.omp_sms) leaves = a.omp_sms;
+    if (leaves > slots) leaves = slots;
     if constexpr (NF == 2) {
-        // omp_slots = the device's SMs.  A step's products shrink with C and
-        // its barriers and chains do not: 16 leaves of side 64 take 7.05, 11.2,
-        // 18.7 and 33.3 ms with 8, 4, 2 CTAs and one, 64 leaves 8.0 with two
-        // against 14.5 with one.  More CTAs than SMs would queue whole leaves
-        const long long leaves = a.lv.capacity;
-        if (B == 64 && leaves * 8 <= a.omp_slots) return launch_omp_cta_c<B, NF, (B == 64 ? 8 : 1)>(a, st);
-        if (B == 64 && leaves * 4 <= a.omp_slots) return launch_omp_cta_c<B, NF, (B == 64 ? 4 : 1)>(a, st);
-        if (leaves * 2 <= a.omp_slots) return launch_omp_cta_c<B, NF, 2>(a, st);
+        // A step's products shrink with C and its barriers and chains do not:
+        // 16 leaves of side 64 took 7.69, 11.2, 18.7 and 33.3 ms with 8, 4, 2
+        // CTAs and one, 64 leaves 8.0 with two against 14.5 with one.  More
+        // CTAs than SMs would queue whole leaves
+        if (B == 64 && leaves * 8 <= a.omp_sms) return launch_omp_cta_c<B, NF, (B == 64 ? 8 : 1)>(a, leaves, st);
+        if (B == 64 && leaves * 4 <= a.omp_sms) return launch_omp_cta_c<B, NF, (B == 64 ? 4 : 1)>(a, leaves, st);
+        if (leaves * 2 <= a.omp_sms) return launch_omp_cta_c<B, NF, 2>(a, leaves, st);
     }
-    return launch_omp_cta_c<B, NF, 1>(a, st);
+    return launch_omp_cta_c<B, NF, 1>(a, leaves, st);
 }
 
 int omp_cta_max_budget() { return kMaxBudget; }
