@@ -1,21 +1,24 @@
 // corr_sep_tc.cu -- (a2) the separable exact correlation (sep.cuh) on the
-// 5th-generation tensor cores, side 64: the same exact integer T = B Y B^T
+// 5th-generation tensor cores, sides 64 and 128 (the latter: the DCT-II family
+// alone, in the second half of the file): the same exact integer T = B Y B^T
 // per family as the SIMT twin (corr_sep.cu), rounded the same way, so both
 // give identical bits.
 //
-// A CTA takes two leaves at a time: 128 rows of a tile are (leaf, row), and
-// every value ends in the lane and the thread that uses it.
+// At side 64 a CTA takes two leaves at a time: 128 rows of a tile are (leaf,
+// row), and every value ends in the lane and the thread that uses it.
 //
-// Digits.  Bf = sum_{s<6} d_s 2^(8s) with balanced digits |d_s| <= 128 (the
-// top one <= 181), all exact BF16 values, as are the centred pixels.
+// Digits.  Bf = sum_{s<6} d_s 2^(8s) with balanced digits |d_s| <= 128 (the top
+// one <= 45 in a DCT-II row of side 64, 181 in a Haar row), all exact BF16
+// values, as are the centred pixels.  The bounds on their sums below are
+// checked against the digits there are when the table is made (host.cu).
 //   Fold (DCT-II).  Row q of Bf equals (-1)^q times its mirror image, so row m
 //   of the pixels becomes y~[m] + y~[63-m] (m < 32) or y~[m] - y~[63-m]
 //   (m >= 32), in place: at most 256 in magnitude, exact BF16.  The even rows
 //   of Bf need the first 32 only, the odd ones the last 32: half of stage 2.
 //   Stage 1: Z~^T[m][p] = sum_i y~[i][m] Bf[p][i].  A = the pixels (rows
 //     (leaf, m), K = i), B = the digits (rows (parity of p, s, p / 2)): lane
-//     (leaf, m) holds the six digit sums of each p, each below 256 x 181 x 64
-//     < 2^22 in magnitude: exact.  They are joined in int64 with the centring
+//     (leaf, m) holds the six digit sums of each p, each at most 0.42 x 2^22
+//     in magnitude: exact.  They are joined in int64 with the centring
 //     term 128 R[p] of each pixel row (R[p] the row sums of Bf; a difference
 //     has none) and split into eight balanced base-2^8 digits e_t, written to
 //     shared memory as stage 2's A operand: rows (leaf, p), K = m, M-major, so
@@ -24,9 +27,9 @@
 //     one parity at a time.  B = the digits d_0 .. d_5 of those q stacked (192
 //     rows), so that one MMA with A = e_t adds into the columns of the digit
 //     diagonals t .. t + 5 (32 columns each): the sum of at most six digit
-//     products, each below 128 x 181 x 32: below 2^22, exact.  Without the fold
-//     (the Haar family) K = 64, and the bound holds since a Haar row of 64
-//     nonzero entries is a power of two, with one nonzero digit.
+//     products, 128 times a row's digits, at most 0.39 x 2^22: exact.  Without
+//     the fold (the Haar family) K = 64, and 0.34 x 2^22 (a Haar row of 64
+//     nonzero entries is a power of two, with one nonzero digit).
 //   The epilogue joins the 13 diagonals of an output: adjacent ones in one
 //   32-bit multiply-add on their biased bit patterns (no wrap), those as
 //   disjoint words of two 128-bit numbers, and biased_to_df rounds the sum

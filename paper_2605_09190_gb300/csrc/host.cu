@@ -540,17 +540,26 @@ int get_dict(Ctx *c, int b, int dict_id, cudaStream_t st, Dict **out, bool table
                                 dg[at * b + col] = __float2bfloat16((float)dv);
                             }
                         }
-                // side 128: the digit sums of stage 2 (corr_sep_tc.cu), products with
-                // eight digits of magnitude 128, have to stay below 2^22
-                if (b == 128)
+                // the digit sums of the tensor-core kernels are exact below 2^22
+                // (corr_sep_tc.cu): stage 1's products with folded pixels (the
+                // Haar family of side 64: with plain ones), stage 2's with digits of magnitude
+                // 128, six of them on a diagonal, over the half of a row
+                // that the fold leaves (the Haar family: all of it)
+                for (int F = 0; F < (b == 64 ? 2 : 1); ++F)
                     for (int r = 0; r < b; ++r) {
-                        double sum[6] = {};
-                        for (int sd = 0; sd < 6; ++sd)
-                            for (int col = 0; col < b / 2; ++col)
-                                sum[sd] += std::fabs(__bfloat162float(
-                                    dg[((size_t)(r & 1) * 3 * b + (r >> 6) * 192 + sd * 32 + ((r >> 1) & 31)) * b + col]));
-                        if (128.0 * (sum[0] + sum[1] + sum[2] + sum[3] + sum[4] + sum[5]) >= 4194304.0)
-                            return AQMP_E_UNSUPPORTED;
+                        double all = 0.0, most = 0.0;
+                        for (int sd = 0; sd < 6; ++sd) {
+                            double row = 0.0;
+                            for (int col = 0; col < b; ++col) {
+                                const double v = std::fabs(__bfloat162float(
+                                    dg[((size_t)F * 6 * b + (r & 1) * 3 * b + (r >> 6) * 192 + sd * 32 + ((r >> 1) & 31)) * b + col]));
+                                row += v;
+                                if (F == 1 || col < b / 2) all += v;
+                            }
+                            most = std::max(most, row);
+                        }
+                        if (128.0 * all >= 0x1p22 || (F == 0 ? 256.0 : 128.0) * most >= 0x1p22)
+                            return fail(AQMP_E_DICT, "digit sums of row %d, side %d, are not exact in FP32", r, b);
                     }
                 if ((rc0 = Dn->sepd.reserve(sizeof(__nv_bfloat16) * dg.size()))) return rc0;
                 d.sepd = (__nv_bfloat16 *)Dn->sepd.p;
