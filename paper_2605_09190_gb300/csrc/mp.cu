@@ -333,21 +333,22 @@ mp_kernel(MPArgs a) {
         };
         // The FP32 form's leader needs no second magnitude: the lowest index of
         // the largest one, its sign below it in one word, so that two reductions
-        // and a single exchange find it.  With the form's one FMA an element the
-        // look-up above costs more than the update: sides 16 and 32 of a 256x384
-        // RGB image take 26 and 94 us with it and 35 and 127 without.  From 32
-        // slots a thread on, the search through all of them costs more than it
-        // saves: side 64, 338 us against 313.
+        // and a single exchange find it.  With the form's one FMA an element,
+        // group_lead's look-up costs more than the update.  256x384 RGB at
+        // tolerance 4, this against the summaries of the two largest that the
+        // kernel carried before: side 16 26.6 us against 27.0, side 32 98
+        // against 113.  From 32 slots a thread on, the search through all of
+        // them costs more than it saves (side 64: 338 us against 313).
         auto plain_lead = [&](int buf) {
             const float top = sm.top();
             auto key_of = [&](uint32_t M) {
+                const float Mf = __uint_as_float(M);
                 uint32_t slot = 0u, sign = 0u;
 #pragma unroll
                 for (int s = E - 1; s >= 0; --s) {
-                    const uint32_t h = __float_as_uint(c.hi(s));
-                    const bool is = (h & 0x7fffffffu) == M;
+                    const bool is = fabsf(c.hi(s)) == Mf;
                     slot = is ? (uint32_t)s : slot;
-                    sign = is ? h : sign;
+                    sign = is ? __float_as_uint(c.hi(s)) : sign;
                 }
                 return __reduce_min_sync(0xffffffffu, __float_as_uint(top) == M
                                                           ? 2u * At::atom(abase, (int)slot) + (sign >> 31) : kNone);
