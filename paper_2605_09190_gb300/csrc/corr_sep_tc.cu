@@ -45,7 +45,8 @@
 // One CTA per SM (16 warps, all 512 TMEM columns: stage 1 in 0..383, stage 2
 // in 0..415), persistent over the pairs; thread 0 issues the TMA loads and the
 // MMAs, all threads drain.  Every wait is bounded by a timer; on expiry the
-// kernel records AQMP_E_TIMEOUT, frees its TMEM and returns.
+// kernel waits, bounded again, for what it has in flight, records
+// AQMP_E_TIMEOUT, frees its TMEM and returns.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
@@ -265,8 +266,8 @@ corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constan
     for (long long pair = blockIdx.x; ok && pair < pairs; pair += gridDim.x, ++it) {
         const int buf = it & 1;
         ok = __syncthreads_and(mbar_wait(buf ? barY1 : barY0, y_phase[buf])) != 0;
-        y_phase[buf] ^= 1u;
         if (!ok) break;
+        y_phase[buf] ^= 1u;
         // prefetch the next pair into the other buffer (its last reader, the
         // previous pair's stage 1, has been waited for)
         if (tid == 0 && pair + gridDim.x < pairs) load_pair(pair + gridDim.x, buf ^ 1);
@@ -296,8 +297,8 @@ corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constan
         }
         if (pending >= 0) finish(pending, 1);
         ok = __syncthreads_and(mbar_wait(barMma, mma_phase)) != 0;
-        mma_phase ^= 1u;
         if (!ok) break;
+        mma_phase ^= 1u;
         fence_after();
         // ---- drain 1: p = 16 cg + 8 h + (0 .. 7), one chunk of each digit's row
 #pragma unroll
@@ -344,8 +345,8 @@ corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constan
             }
             if (par == 1) finish(pair, 0);
             ok = __syncthreads_and(mbar_wait(barMma, mma_phase)) != 0;
-            mma_phase ^= 1u;
             if (!ok) break;
+            mma_phase ^= 1u;
             fence_after();
             // ---- drain 2: q = 2 (8 cg + j) + par, 13 diagonals each
             drain_diagonals(lane_base, 8 * cg, T);
@@ -355,6 +356,14 @@ corr_sep_tc_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_constan
         pending = pair;
     }
     if (ok && pending >= 0) finish(pending, 1);
+    if (tid == 0 && !ok) {
+        // what may be in flight, before shared memory and TMEM are given up: the
+        // phase that each barrier is at
+        mbar_wait(barD, 0);
+        mbar_wait(barY0, y_phase[0]);
+        mbar_wait(barY1, y_phase[1]);
+        mbar_wait(barMma, mma_phase);
+    }
     fence_before();
     __syncthreads();
     if (tid == 0 && !ok && ctr) raise_error(ctr, kDevErrTimeout, 12u);
@@ -438,11 +447,14 @@ corr_sep_tc128_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_cons
     if (warp == 16) {
         if (lane == 0) {
             uint32_t phD = 0, phP = 0, phC = 0;
+            uint32_t nD = 0, nY = 0, nP = 0, nA = 0;              // issued on each barrier
             auto load_digits = [&](int a, int kh) {
+                ++nD;
                 mbar_expect_tx(barD, kChunk);
                 for (int t = 0; t < 3; ++t) tma_load_2d(sD + t * 128 * 128, &tmD, barD, 64 * kh, 384 * a + 128 * t);
             };
             auto load_pixels = [&](long long leaf) {
+                ++nY;
                 mbar_expect_tx(barY, 2 * 128 * 128);
                 for (int kh = 0; kh < 2; ++kh) tma_load_2d(sY + kh * 128 * 128, &tmY, barY, 64 * kh, (int)(128 * leaf));
             };
@@ -461,6 +473,7 @@ corr_sep_tc128_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_cons
                         mma_ss(tmem + 192 * qh, ad + 2ull * kk, bd + (unsigned long long)(qh * 192 * 128 >> 4) + 2ull * kk,
                                idesc(192, false), kk > 0 ? 1u : acc);
                 mma_commit(bar);
+                ++(bar == barP ? nP : nA);
             };
             load_digits(1, 1);
             load_pixels(blockIdx.x);
@@ -492,9 +505,16 @@ corr_sep_tc128_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_cons
                         fence_after();
                         issue_stage2(tmem, sE, sD + qh * 192 * 128, 0, 4);
                         mma_commit(barA);
+                        ++nA;
                     }
                 }
             }
+            // the last of each, before shared memory and TMEM are given up (after
+            // an expired wait, the drainers' too: they see MMAs come in late)
+            mbar_wait(barD, (nD - 1u) & 1u);
+            mbar_wait(barY, (nY - 1u) & 1u);
+            if (nP) mbar_wait(barP, (nP - 1u) & 1u);
+            if (nA) mbar_wait(barA, (nA - 1u) & 1u);
         }
     } else {
         const int quarter = warp & 3, cg = warp >> 2;
