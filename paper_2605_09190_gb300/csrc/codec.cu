@@ -70,7 +70,6 @@ struct Reader {
         take(b, 4);
         return (uint32_t)b[0] | ((uint32_t)b[1] << 8) | ((uint32_t)b[2] << 16) | ((uint32_t)b[3] << 24);
     }
-    float f32() { uint32_t v = u32(); float f; std::memcpy(&f, &v, 4); return f; }
     uint32_t varint() {
         if (ok && p < end && *p < 0x80u) return *p++;
         uint32_t v = 0;

@@ -132,9 +132,8 @@ __device__ __forceinline__ int haar_join(const int *s, int stride, int r) {
 // kept negated in three signed 32-bit limbs (2^95 fits with that sign), so
 // T + the rounding's bias is a chain of three 32-bit multiply-adds.  The
 // integer work of an output is now the smaller part of it beside the rounding.
-// Side 64, 50 910 leaves, this family alone: 1.88 -> 0.85 ms (a
-// summed-area table, nine reads and an int128 product per output, before; with
-// that rounding's general form 1.50).
+// Side 64, 50 910 leaves, this family alone: 1.88 -> 0.85 ms (a summed-area
+// table, nine reads and an int128 product per output, before).
 template <int B, bool HO>
 __global__ void __launch_bounds__(sep_threads<B>())
 corr_sep_simt_kernel(int nf, int fam0, int fmask, int Kpad, const int2 *__restrict__ Bs, const int2 *__restrict__ BsT,

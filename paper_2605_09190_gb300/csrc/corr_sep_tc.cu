@@ -38,9 +38,10 @@
 // What bounds it: the instructions of the epilogue and of the digit split
 // (about 105 an output and 35 a value of Z~), which therefore overlap the MMAs where they can:
 // a pass's outputs are rounded and stored while the next pass or the next
-// pair's stage 1 runs.  Side 64, DCT-II family, 50 910 leaves: 4.60 -> 1.51
+// pair's stage 1 runs.  Side 64, DCT-II family, 50 910 leaves: 5.26 -> 1.53
 // ms (one leaf at a time with two digits in the 128 rows, halves that met
-// through shared memory and 24 accumulators an output, before).
+// through shared memory, 24 accumulators an output and the general rounding,
+// before).
 //
 // One CTA per SM (16 warps, all 512 TMEM columns: stage 1 in 0..383, stage 2
 // in 0..415), persistent over the pairs; thread 0 issues the TMA loads and the

@@ -289,7 +289,8 @@ std::string kname(const char *k, int b) { return std::string(k) + "_b" + std::to
 
 // The exact separable correlation on the tensor-core path: the DCT-II family
 // on the tensor cores, the Haar family on the SIMT pipes, where it is two
-// passes of sums and differences with no contraction left to speed up.  Bit for bit the SIMT kernel's result for both families.
+// passes of sums and differences with no contraction left to speed up.  Bit for
+// bit the SIMT kernel's result for both families.
 cudaError_t corr_sep_hybrid(const CorrArgs &ca, int b, cudaStream_t st) {
     const DictDev &d = *ca.d;
     const bool dct = d.nf == 2 || d.fam0 == 0, haar = d.nf == 2 || d.fam0 == 1;

@@ -147,10 +147,11 @@ mp_kernel(MPArgs a) {
     // summaries, one of them carries the energy, the stop test and the step
     // record, and the owner's work on its zeroed element is off the critical
     // path.  A sub-partition holds as many warps of each family, so the update
-    // itself keeps all FP32 pipes busy either way.  With the packed update and
-    // the magnitude-only summaries: 12 uneven RGB piecewise images 20.7 -> 17.3
-    // ms, 64 gradient ones 17.3 -> 15.9 ms, the 512x512 sweep 1.85 -> 1.72 ms
-    // (whole encodes; same bits).
+    // itself keeps all FP32 pipes busy either way.  Side 64, this kernel against
+    // the one before it (both families on every warp, no packed update, sign,
+    // slot, low word and runner-up carried through the summaries; same bits):
+    // 50 910 gradient leaves 9.35 -> 7.92 ms, 12 uneven piecewise images 18.0 ->
+    // 14.6 ms, a 512x512 image at four tolerances 1.01 -> 0.89 ms.
     constexpr bool SPLIT = NF == 2 && T > 32;
     constexpr int FT = SPLIT ? T / 2 : T;    // threads of one family
     constexpr bool PLAIN = !DF && E <= 16;   // how the FP32 form finds its leader (plain_lead)

@@ -19,9 +19,9 @@
 // rank r), and each thread loads its row entry from the owning peer through
 // distributed shared memory.
 //
-// Each step every warp reduces its own top-2 summary (the same summaries,
-// window rule and certification as the single-CTA kernel) and stores it into
-// every CTA of the cluster through distributed shared memory -- a 16-byte
+// Each step every warp whose correlations changed finds its leader (the same
+// summaries, window rule and certification as the single-CTA kernel), and every
+// warp stores its leader into every CTA of the cluster through distributed shared memory -- a 16-byte
 // slot per warp and CTA, written by st.async, which completes its bytes on
 // the receiving CTA's mbarrier -- so after one wait every CTA merges the same
 // values into the same choice.  The energy, the stop test and the choice then

@@ -12,20 +12,22 @@
 //     are left out;
 //   - argmax |c| with the MP kernel's tie rule (values within 2^-32 ||y|| of
 //     the largest are tied, lowest index wins) and certification band;
-//   - the Cholesky factor L of G_SS grows by a row (w, sqrt(d)) with
-//     w = L^-1 G[S, j], d = 1 - |w|^2 (a pivot d <= 2^-40 ends the pursuit, the
-//     atom being dependent on the support); z grows by (c0_j - w . z) / sqrt(d)
-//     and the re-fit x_S = L^-T z by z_new times the new column of L^-T.
+//   - the inverse K = L^-1 of the Cholesky factor of G_SS grows by the row
+//     (-w^T K, 1) / sqrt(d) with w = K G[S, j], d = 1 - |w|^2 (a pivot
+//     d <= 2^-40 ends the pursuit, the atom being dependent on the support); z
+//     grows by z_new = (c0_j - w . z) / sqrt(d) and the re-fit x_S = K^T z by
+//     z_new times that row.
 //
 // Everything is FP64, at 1/64 of GB300's FP32 rate, and that bounds the
-// kernel: a warp's FP64 instruction takes the SM 16 cycles.  So the inverse
-// factor K = L^-1 is kept instead of L (packed, in shared memory): its new row
-// is (-w^T K, 1) / sqrt(d), and a step takes the two products K g (over the
-// support atoms of the other family alone, g being zero on its own) and w^T K,
-// about 2.5 t instructions for t atoms, where two forward and one back
-// substitution with L took 9 t, in chains of shuffles.  The argmax compares
-// the doubles' bit patterns on the integer pipes.  A 512x512 plane at
-// four tolerances, sides 16..4: the whole encode 6.53 -> 3.86 ms.  A leaf's budget k must be <= 64 (two rows per lane).
+// kernel: a warp's FP64 instruction takes the SM 16 cycles.  K is kept packed
+// in shared memory; a step takes the two products K g (over the support atoms
+// of the other family alone, g being zero on its own) and w^T K, about 2.5 t
+// instructions for t atoms.  With L itself, two forward substitutions and a
+// back substitution take 9 t, in chains of shuffles.  The argmax compares the
+// doubles' bit patterns on the integer pipes.  A 512x512 plane at four
+// tolerances, sides 16, 8 and 4, against the kernel with L: 6.01, 0.82 and
+// 0.37 ms -> 3.27, 0.48 and 0.31.  A leaf's budget k must be <= 64 (two rows
+// per lane).
 #include <cuda_runtime.h>
 
 #include "common.cuh"

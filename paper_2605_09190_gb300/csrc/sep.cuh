@@ -114,8 +114,8 @@ __device__ __forceinline__ float fast_sum(float a, float b, float &e) {
 // them); or r alone, which rounds to even by itself when nothing is below it.
 // Other values, near a tie, take the general form: none in 10^7 random
 // integers above 2^65 (|c| > 2^-31), up to a fifth at 50 to 56 bits.
-// Side-64 correlation of 50 910 leaves: DCT-II family 5.25 -> 4.60 ms (in the
-// kernel of that time), Haar family 1.50 -> 0.85 ms.
+// Side 64, 50 910 leaves: the Haar family's kernel takes 0.85 ms with it and
+// 1.50 with the general form alone.
 constexpr unsigned long long kDigitBiasLo = (1ull << 22) | (1ull << 45);      // half a unit of each of the four
 constexpr unsigned long long kDigitBiasHi = (1ull << 4) | (1ull << 27);       // lower digits, as 128 bits
 
