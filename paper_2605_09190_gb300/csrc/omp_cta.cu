@@ -33,9 +33,11 @@
 // shared memory: three cluster barriers a step.  Every sum is formed in an order
 // that the support alone fixes, so the coefficients have the same bits at every
 // width of the cluster.
-// A 256x256 image of 64x64 roots (16 leaves, 1285 atoms): 66.8 -> 7.05 ms;
-// 1024x640 (160 leaves, one CTA each): 13.8 -> 11.4 ms; a 512x512 plane at
-// four tolerances down to side 4, up to 1024 atoms a leaf: 884 -> 551 ms.
+// Piecewise scenes, whole encodes against one CTA a leaf with dense cross terms
+// and triangular solves: 256x256 of 64x64 roots 115 -> 10.5 ms, 512x512 67.2 ->
+// 19.8, 1024x640 (160 leaves, one CTA each) 42.0 -> 24.0; 512x512 of 32x32 roots
+// 26.1 -> 13.1; 512x512 at four tolerances down to side 4, up to 1024 atoms a
+// leaf, 883 -> 546.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
