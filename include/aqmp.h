@@ -269,7 +269,8 @@ int aqmp_synth_backward(const aqmp_code *code, int plane, const float *grad_out,
  * window of sigma 1.5, valid region) of `y` against the reference `x`, both
  * h x w FP32 images with `pitch` elements per row, h, w >= 11.  Window
  * sums and the per-window formula are evaluated in double-float (~2^-46
- * relative; the formula in FP64 for windows with E[x^2 + y^2] above 2^48).
+ * relative; the formula in FP64 for windows whose squared means or variances
+ * exceed 2^48).
  * Pixels may reach 10^19, where their squares leave FP32.  *ssim (device, FP64) receives the
  * mean; with grad_y != NULL, grad_y (h x w, pitch) receives
  * grad_scale * d(mean SSIM)/dy. */

@@ -226,7 +226,7 @@ struct SsimArgs {
     SsimPlane p[kRefinePlanes];
     int n;
     df c1, c2;                                       // filled by the launch, as are the window's
-    unsigned long long gh[11], ngh[11], gl[11];      // weights: high word, its negative, low word, twice each
+    unsigned long long gh[11], ngh[11], ngl[11];     // weights: high word, its negative, the low word's, twice each
 };
 cudaError_t launch_ssim(SsimArgs &a, bool grad, int num_sms, cudaStream_t st);
 

@@ -3,10 +3,13 @@
 //
 // SSIM over the valid region with an 11 x 11 Gaussian window w = g g^T
 // (sigma 1.5), K1 = 0.01, K2 = 0.03, L = 255.  Per window, with the window
-// means mx, my, Es = E[x^2 + y^2] and Exy:
-//   A1 = 2 mx my + C1, A2 = 2 (Exy - mx my) + C2,
-//   B1 = mx^2 + my^2 + C1, B2 = (Es - mx^2 - my^2) + C2,
+// means mx, my, Exy = E[x y] and Ed = E[(x - y)^2]:
+//   A1 = 2 mx my + C1, B1 = A1 + (mx - my)^2 = mx^2 + my^2 + C1,
+//   A2 = 2 (Exy - mx my) + C2,
+//   B2 = A2 + (Ed - (mx - my)^2) = var x + var y + C2,
 //   f = A1 A2 / (B1 B2).
+// Ed in the place of E[x^2 + y^2]: an error of Exy, the larger one, then moves
+// A2 and B2 together, and f by 1 - A2 / B2 of it alone.
 // With S = mean f over the N windows, for a pixel k of y:
 //   dS/dy[k] = (1/N) sum_win w(k - win) (f_my + 2 y[k] f_Eyy + x[k] f_Exy),
 //   f_my = f (2 mx / A1 - 2 mx / A2 - 2 my / B1 + 2 my / B2),
@@ -20,10 +23,17 @@
 // window pass.  An 11-tap pass keeps each sum as (s, c): s the running FP32
 // sum, c the sum of the exact errors of its products and additions and of the
 // low words' terms, joined once at the end (Ogita, Rump and Oishi's Dot2
-// scheme) -- 12 operations a tap, against 15 with a renormalised pair.
+// scheme) -- 12 operations a tap, against 15 with a renormalised pair.  A
+// product's small terms meet before they meet c, and taps come smallest weights
+// first where the order is free, so that few roundings are of c's size.
+// Error of a window's value against long double, root mean square, of
+// renormalised pairs with E[x^2], E[y^2], E[x y] and the formula in FP64, and
+// here: 3.1e-12 and 0.8e-12 for a piecewise scene with noise of 4 grey values,
+// 3.0e-12 and 0.1e-12 with 1, 1.0e-12 and 0.6e-12 for a gradient one with 8,
+// 1.6e-14 and 1.5e-14 for two independent images.
 //
 // Forward: a CTA loads the pixels of a tile of windows once, filters the four
-// fields x, y, x^2 + y^2, x y along the rows into shared memory and down the
+// fields x, y, x y, (x - y)^2 along the rows into shared memory and down the
 // columns into registers, and writes the three partials (24 bytes a window);
 // backward: the same with the partials' tile, columns first.  Bound by the
 // FP32 pipes (about 154 taps a pixel); the four passes over global memory
@@ -52,22 +62,25 @@ struct Acc1 {
     float s, c;
 };
 
-// acc + g (v + vl) for two sums at once, g = gh + gl, ngh = -gh.
+// acc + g (v + vl) for two sums at once, g = gh - ngl, ngh = -gh.
 template <bool LO>
-__device__ __forceinline__ void tap(Acc2 &a, f2 gh, f2 ngh, f2 gl, f2 v, f2 vl) {
-    const f2 p = f2_mul(gh, v), ne = f2_fma(ngh, v, p);         // g v = p - ne exactly
+__device__ __forceinline__ void tap(Acc2 &a, f2 gh, f2 ngh, f2 ngl, f2 v, f2 vl) {
+    const f2 p = f2_mul(gh, v);
+    f2 ne = f2_fma(ngh, v, p);                                  // gh v = p - ne exactly
+    if (LO) ne = f2_fma(ngh, vl, ne);
+    ne = f2_fma(ngl, v, ne);
     const f2 s = f2_add(a.s, p);
     const f2 bb = f2_sub(s, a.s);
     const f2 t = f2_add(f2_sub(a.s, f2_sub(s, bb)), f2_sub(p, bb));
-    a.c = f2_fma(gl, v, f2_add(a.c, f2_sub(t, ne)));
-    if (LO) a.c = f2_fma(gh, vl, a.c);
+    a.c = f2_add(a.c, f2_sub(t, ne));
     a.s = s;
 }
 
-__device__ __forceinline__ void tap(Acc1 &a, float gh, float gl, float v, float vl) {
-    const df p = df_two_prod(gh, v), s = df_two_sum(a.s, p.hi);
-    a.c = __fmaf_rn(gl, v, __fadd_rn(a.c, __fadd_rn(s.lo, p.lo)));
-    a.c = __fmaf_rn(gh, vl, a.c);
+__device__ __forceinline__ void tap(Acc1 &a, float gh, float ngh, float ngl, float v, float vl) {
+    const float p = __fmul_rn(gh, v);
+    const float ne = __fmaf_rn(ngl, v, __fmaf_rn(ngh, vl, __fmaf_rn(ngh, v, p)));
+    const df s = df_two_sum(a.s, p);
+    a.c = __fadd_rn(a.c, __fsub_rn(s.lo, ne));
     a.s = s.hi;
 }
 
@@ -93,13 +106,13 @@ struct Window {
 };
 
 // ... from its means in FP64, where 1 / (B1 B2) and its low word would leave
-// the range of FP32: E[x^2 + y^2] above 2^48, pixels of 10^7 and more.  Out of
+// the range of FP32: B1 or B2 above 2^48, pixels of 10^7 and more.  Out of
 // line, since no image has such pixels (a refinement that diverges does).
-__device__ __noinline__ void window_fp64(df mx_, df my_, df es_, df exy_, Window *out) {
-    const double mx = df_to_double(mx_), my = df_to_double(my_), es = df_to_double(es_), exy = df_to_double(exy_);
+__device__ __noinline__ void window_fp64(df mx_, df my_, df exy_, df ed_, Window *out) {
+    const double mx = df_to_double(mx_), my = df_to_double(my_), exy = df_to_double(exy_), ed = df_to_double(ed_);
     const double C1 = (0.01 * 255.0) * (0.01 * 255.0), C2 = (0.03 * 255.0) * (0.03 * 255.0);
-    const double mxy = mx * my, mm = mx * mx + my * my;
-    const double A1 = 2.0 * mxy + C1, A2 = 2.0 * (exy - mxy) + C2, iB1 = 1.0 / (mm + C1), iB2 = 1.0 / ((es - mm) + C2);
+    const double mxy = mx * my, ee = (mx - my) * (mx - my);
+    const double A1 = 2.0 * mxy + C1, A2 = 2.0 * (exy - mxy) + C2, iB1 = 1.0 / (A1 + ee), iB2 = 1.0 / (A2 + (ed - ee));
     const double t1 = A2 * iB1 * iB2, t2 = A1 * iB1 * iB2, f = A1 * t1;          // f / A1, f / A2
     out->f = df_split(f);
     out->my = df_split(2.0 * mx * (t1 - t2) - 2.0 * my * f * (iB1 - iB2));
@@ -124,8 +137,9 @@ struct FwdTile {
     static constexpr int HR = RV == 7 ? 64 : 32;              // pixel rows of the tile
     static constexpr int TH = HR - 10;                        // window rows
     static constexpr int XW = 44;                             // pixel row stride
-    static constexpr size_t bytes = sizeof(float2) * HR * XW + 2 * sizeof(float4) * HR * kTW;
-    static_assert(8 * RV >= TH, "rows");
+    static constexpr int PAD = 8 * RV + 10 - HR;              // rows past the tile that the column pass reads, unused
+    static constexpr size_t bytes = sizeof(float2) * HR * XW + sizeof(float4) * (2 * HR + PAD) * kTW;
+    static_assert(8 * RV >= TH && PAD >= 0 && PAD < HR, "rows");
 };
 
 template <int RV>
@@ -134,7 +148,7 @@ __global__ void __launch_bounds__(kThreads, 2) ssim_forward_kernel(const __grid_
     extern __shared__ __align__(16) unsigned char smem[];
     float2 *xy = reinterpret_cast<float2 *>(smem);                        // [HR][XW] (x, y)
     float4 *Hm = reinterpret_cast<float4 *>(xy + T::HR * T::XW);           // [HR][TW] x, y: high words, low words
-    float4 *Hp = Hm + T::HR * kTW;                                         // [HR][TW] x^2 + y^2, x y
+    float4 *Hp = Hm + T::HR * kTW;                                         // [HR][TW] x y, (x - y)^2
     int ty, tx;
     const SsimPlane &P = find_plane(a, ty, tx);
     const int r0 = ty * T::TH, c0 = tx * kTW, wo = P.w - 10, ho = P.h - 10;
@@ -156,20 +170,21 @@ __global__ void __launch_bounds__(kThreads, 2) ssim_forward_kernel(const __grid_
         for (int o = 0; o < 4; ++o) m[o] = p[o] = Acc2{0ull, 0ull};
         const ulonglong2 *row = reinterpret_cast<const ulonglong2 *>(xy + r * T::XW + c);
 #pragma unroll
-        for (int k = 0; k < 14; ++k) {
-            const ulonglong2 two = row[k / 2];
+        for (int i = 0; i < 14; ++i) {
+            // pairs of pixels from both ends, the middle last
+            const int two_at = i & 2 ? 6 - (i >> 2) : i >> 2, k = 2 * two_at + (i & 1);
+            const ulonglong2 two = row[two_at];
             const f2 v = k & 1 ? two.y : two.x;
             const float x = f2_x(v), y = f2_y(v);
-            const df xx = df_two_prod(x, x), yy = df_two_prod(y, y), c2 = df_two_prod(x, y);
-            const df s2 = df_two_sum(xx.hi, yy.hi);
-            const f2 ph = f2_make(s2.hi, c2.hi);
-            const f2 pl = f2_make(__fadd_rn(s2.lo, __fadd_rn(xx.lo, yy.lo)), c2.lo);
+            const df c2 = df_two_prod(x, y), d = df_two_sum(x, -y), dd = df_two_prod(d.hi, d.hi);
+            const f2 ph = f2_make(c2.hi, dd.hi);
+            const f2 pl = f2_make(c2.lo, __fmaf_rn(2.0f * d.hi, d.lo, dd.lo));
 #pragma unroll
             for (int o = 0; o < 4; ++o) {
                 const int j = k - o;
                 if (j < 0 || j > 10) continue;
-                tap<false>(m[o], a.gh[j], a.ngh[j], a.gl[j], v, 0ull);
-                tap<true>(p[o], a.gh[j], a.ngh[j], a.gl[j], ph, pl);
+                tap<false>(m[o], a.gh[j], a.ngh[j], a.ngl[j], v, 0ull);
+                tap<true>(p[o], a.gh[j], a.ngh[j], a.ngl[j], ph, pl);
             }
         }
 #pragma unroll
@@ -188,15 +203,16 @@ __global__ void __launch_bounds__(kThreads, 2) ssim_forward_kernel(const __grid_
 #pragma unroll
     for (int o = 0; o < RV; ++o) m[o] = p[o] = Acc2{0ull, 0ull};
 #pragma unroll 1
-    for (int j = 0; j < 11; ++j) {
-        const f2 gh = a.gh[j], ngh = a.ngh[j], gl = a.gl[j];
+    for (int i = 0; i < 11; ++i) {
+        const int j = i & 1 ? 10 - (i >> 1) : i >> 1;                 // smallest weights first: 0, 10, 1, 9, ..., 5
+        const f2 gh = a.gh[j], ngh = a.ngh[j], ngl = a.ngl[j];
+        const int at = (row + j) * kTW + col;
 #pragma unroll
         for (int o = 0; o < RV; ++o) {
-            const int at = min(row + o + j, T::HR - 1) * kTW + col;       // rows past the tile are not used
-            const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(Hm + at);
-            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(Hp + at);
-            tap<true>(m[o], gh, ngh, gl, u.x, u.y);
-            tap<true>(p[o], gh, ngh, gl, v.x, v.y);
+            const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(Hm + at + o * kTW);
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(Hp + at + o * kTW);
+            tap<true>(m[o], gh, ngh, ngl, u.x, u.y);
+            tap<true>(p[o], gh, ngh, ngl, v.x, v.y);
         }
     }
 
@@ -206,16 +222,16 @@ __global__ void __launch_bounds__(kThreads, 2) ssim_forward_kernel(const __grid_
         const int r = r0 + row + o, c = c0 + col;
         if (row + o >= T::TH || r >= ho || c >= wo) continue;
         const df mx = join(f2_x(m[o].s), f2_x(m[o].c)), my = join(f2_y(m[o].s), f2_y(m[o].c));
-        const df es = join(f2_x(p[o].s), f2_x(p[o].c)), exy = join(f2_y(p[o].s), f2_y(p[o].c));
+        const df exy = join(f2_x(p[o].s), f2_x(p[o].c)), ed = join(f2_y(p[o].s), f2_y(p[o].c));
+        const df mxy = df_mul(mx, my), e = df_sub(mx, my), ee = df_mul(e, e);
+        const df A1 = df_add(twice(mxy), a.c1), B1 = df_add(A1, ee);
+        const df A2 = df_add(twice(df_sub(exy, mxy)), a.c2), B2 = df_add(A2, df_sub(ed, ee));
         Window v;
-        if (__builtin_expect(!(es.hi <= 0x1p48f), 0)) {
+        if (__builtin_expect(!(fmaxf(B1.hi, B2.hi) <= 0x1p48f), 0)) {
             Window big;
-            window_fp64(mx, my, es, exy, &big);
+            window_fp64(mx, my, exy, ed, &big);
             v = big;
         } else {
-            const df mxy = df_mul(mx, my), mm = df_add(df_mul(mx, mx), df_mul(my, my));
-            const df A1 = df_add(twice(mxy), a.c1), A2 = df_add(twice(df_sub(exy, mxy)), a.c2);
-            const df B1 = df_add(mm, a.c1), B2 = df_add(df_sub(es, mm), a.c2);
             const df q = df_recip(df_mul(B1, B2));
             const df t1 = df_mul(A2, q), t2 = df_mul(A1, q);           // f / A1, f / A2
             v.f = df_mul(A1, t1);
@@ -295,14 +311,14 @@ __global__ void __launch_bounds__(kThreads, 2) ssim_backward_kernel(const __grid
         if (on) {
 #pragma unroll 1
             for (int j = 0; j < 11; ++j) {
-                const f2 gh = a.gh[j], ngh = a.ngh[j], gl = a.gl[j];
+                const f2 gh = a.gh[j], ngh = a.ngh[j], ngl = a.ngl[j];
 #pragma unroll
                 for (int o = 0; o < RC; ++o) {
                     const int at = min(row + o + 10 - j, T::HR - 1) * kCols + col;
                     const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(S4 + at);
                     const float2 v = S2[at];
-                    tap<true>(m[o], gh, ngh, gl, u.x, u.y);
-                    tap(q[o], f2_x(gh), f2_x(gl), v.x, v.y);
+                    tap<true>(m[o], gh, ngh, ngl, u.x, u.y);
+                    tap(q[o], f2_x(gh), f2_x(ngh), f2_x(ngl), v.x, v.y);
                 }
             }
         }
@@ -332,14 +348,14 @@ __global__ void __launch_bounds__(kThreads, 2) ssim_backward_kernel(const __grid
     }
 #pragma unroll 1
     for (int j = 0; j < 11; ++j) {
-        const f2 gh = a.gh[j], ngh = a.ngh[j], gl = a.gl[j];
+        const f2 gh = a.gh[j], ngh = a.ngh[j], ngl = a.ngl[j];
 #pragma unroll
         for (int o = 0; o < T::RH; ++o) {
             const int at = min(warp + 8 * o, T::HR - 1) * kCols + col + 10 - j;
             const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(S4 + at);
             const float2 v = S2[at];
-            tap<true>(m[o], gh, ngh, gl, u.x, u.y);
-            tap(q[o], f2_x(gh), f2_x(gl), v.x, v.y);
+            tap<true>(m[o], gh, ngh, ngl, u.x, u.y);
+            tap(q[o], f2_x(gh), f2_x(ngh), f2_x(ngl), v.x, v.y);
         }
     }
 #pragma unroll
@@ -392,7 +408,7 @@ cudaError_t launch_ssim(SsimArgs &a, bool grad, int num_sms, cudaStream_t st) {
         const df v = df_split(g[i] / s);
         a.gh[i] = f2_both(v.hi);
         a.ngh[i] = f2_both(-v.hi);
-        a.gl[i] = f2_both(v.lo);
+        a.ngl[i] = f2_both(-v.lo);
     }
     a.c1 = df_split((0.01 * 255.0) * (0.01 * 255.0));
     a.c2 = df_split((0.03 * 255.0) * (0.03 * 255.0));
