@@ -7,7 +7,7 @@
 // 2^-32 ||y|| going to the lowest index, the inverse factor K = L^-1 of G_SS
 // grown by a row per selection (a pivot <= 2^-40 ends the pursuit), and the
 // re-fit x_S += z_new times that row.  Everything is FP64, at 1/64 of GB300's
-// FP32 rate: FP64 instructions bound the kernel (16 SM cycles a warp), so the
+// FP32 rate: FP64 instructions bound a leaf in flight (16 SM cycles a warp), so the
 // work is cut by structure and spread over idle SMs.
 //
 // A cluster of C CTAs owns one leaf (as many as the level's leaves leave SMs
